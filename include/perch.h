@@ -148,8 +148,8 @@ int perch_destroy(perch_ctx* ctx);
 const char* perch_last_error(const perch_ctx* ctx);
 
 /* Upload n object meshes (Sec. III: the known 3D models). Replaces any
- * previous meshes. Meshes are split into chunks on the host (at most 512
- * vertices and 1024 triangles each). Errors: PERCH_E_ARG for empty meshes,
+ * previous meshes. Meshes are split into chunks on the host (at most 680
+ * vertices and 1536 triangles each). Errors: PERCH_E_ARG for empty meshes,
  * out-of-range indices or n < 1. */
 int perch_load_meshes(perch_ctx* ctx, const perch_mesh* meshes, int32_t n);
 
@@ -420,8 +420,8 @@ int perch_set_threads(perch_ctx* ctx, int32_t mesh, int32_t threads);
 /* The launch configuration evaluations use now, per mesh (arrays of the
  * number of meshes, any may be NULL): the CTA width of the render (or
  * per-hypothesis evaluation) launch, the render's inline limit (a front-facing
- * triangle with at most that many candidate pixel centres is rasterised by
- * its own thread, a larger one by a warp through the CTA's queue) and the CTA
+ * triangle with at most about that many candidate pixel centres is rasterised
+ * by its own thread, a larger one by several through the CTA's queue) and the CTA
  * width of the cost launch. With shared renders on, perch_autotune times
  * every render width with every inline limit (8, 16, 32), then the cost
  * widths 128 and 256. */
@@ -434,7 +434,7 @@ int perch_set_inline_pixels(perch_ctx* ctx, int32_t mesh, int32_t inline_pixels)
 
 /* The render's bin of larger triangles (the shared-memory queue each CTA
  * fills with front faces whose box holds more than the inline limit's
- * candidate centres, one warp per queued triangle): set its depth (32, 64 or
+ * candidate centres, each shared by eight lanes): set its depth (32, 64 or
  * 128 entries) for one mesh (mesh = -1: all), overriding the default 128 or
  * an autotuned choice; a triangle that finds the bin full is rasterised by
  * its own thread, so records do not depend on it. perch_autotune times the

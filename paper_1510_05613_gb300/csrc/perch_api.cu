@@ -83,7 +83,7 @@ Geometry perch_ctx::geometry() const {
   g.chunk_tris = chunk_tris.as<uint32_t>();
   g.chunk_verts = chunk_verts.as<float4>();
   g.n_cverts = n_cverts;
-  g.vtab = vtab.as<float4>();
+  g.vtab = vtab.as<float>();
   g.pose_off = pose_off.as<float4>();
   g.xs = xs.as<float>();
   g.ys = ys.as<float>();
@@ -92,6 +92,7 @@ Geometry perch_ctx::geometry() const {
   g.ny = ny;
   g.n_yaw = n_yaw;
   g.pose_bbox = pose_bbox.as<int4>();
+  g.pose_general = pose_general.as<uint8_t>();
   g.rx = rx.as<float>();
   g.ry = ry.as<float>();
   g.vol_normals = vol_normals.as<float2>();
@@ -128,17 +129,19 @@ int perch_ctx::ensure_tables() {
   const long long n = (long long)n_mesh * nx * ny * n_yaw;
   CK(yaw_mats.ensure(sizeof(float) * 9 * n_yaw), "alloc yaw matrices");
   CK(pose_off.ensure(sizeof(float4) * nx * ny), "alloc pose offsets");
-  CK(vtab.ensure(sizeof(float4) * (size_t)n_yaw * n_cverts), "alloc vertex tables");
+  CK(vtab.ensure(12 * (size_t)n_yaw * n_cverts), "alloc vertex tables");
   CK(pose_bbox.ensure(sizeof(int4) * n), "alloc pose boxes");
+  CK(pose_general.ensure((size_t)n), "alloc pose paths");
   CK(scratch_small.ensure(64), "alloc");
   DevBuf& wh = g_cursor;  // per-mesh tile sizes (scratch until the first batch)
   CK(wh.ensure(sizeof(int) * (2 * (size_t)n_mesh + 1)), "alloc");
   int* d = wh.as<int>();
   CK(cudaMemsetAsync(d, 0, sizeof(int) * (2 * (size_t)n_mesh + 1), stream), "memset");
   const Geometry g = geometry();
-  CK(launch_pose_tables(cam, g, yaw_mats.as<float>(), pose_off.as<float4>(), vtab.as<float4>(), stream),
+  CK(launch_pose_tables(cam, g, yaw_mats.as<float>(), pose_off.as<float4>(), vtab.as<float>(), stream),
      "pose tables kernel");
-  CK(launch_pose_bbox(cam, g, yaw_mats.as<float>(), pose_bbox.as<int4>(), d, d + 2 * n_mesh, stream),
+  CK(launch_pose_bbox(cam, g, yaw_mats.as<float>(), pose_bbox.as<int4>(), d, d + 2 * n_mesh,
+                      pose_general.as<uint8_t>(), stream),
      "pose_bbox kernel");
   std::vector<int> h(2 * (size_t)n_mesh + 1);
   CK(cudaMemcpyAsync(h.data(), d, sizeof(int) * h.size(), cudaMemcpyDeviceToHost, stream), "copy pose boxes");
@@ -454,7 +457,7 @@ int perch_load_meshes(perch_ctx* ctx, const perch_mesh* meshes, int32_t n) {
         d.lo[k] = std::min(d.lo[k], x);
         d.hi[k] = std::max(d.hi[k], x);
       }
-    // greedy chunks in triangle order: <= 1024 vertices, <= 2048 triangles
+    // greedy chunks in triangle order
     d.chunk_begin = (int)info.size();
     std::vector<int> local(m.n_verts, -1);
     std::vector<int> cur_v;
@@ -467,17 +470,24 @@ int perch_load_meshes(perch_ctx* ctx, const perch_mesh* meshes, int32_t n) {
         local[gv] = -1;
       }
       tris.insert(tris.end(), cur_t.begin(), cur_t.end());
-      while (tris.size() % 4) tris.push_back(0xffffffffu);  // 16-byte aligned chunk lists (bulk copies)
+      while (verts.size() % 4) verts.push_back(make_float4(0.0f, 0.0f, 0.0f, 0.0f));  // 16-byte aligned slices
       info.push_back(in);
       cur_v.clear();
       cur_t.clear();
     };
+    double edge2 = 0.0;
     for (int t = 0; t < m.n_tris; ++t) {
       int idx[3];
       for (int k = 0; k < 3; ++k) {
         idx[k] = m.tris[3 * t + k];
         if (idx[k] < 0 || idx[k] >= m.n_verts)
           return ctx->fail(PERCH_E_ARG, "mesh %d: triangle %d has vertex index %d out of range", i, t, idx[k]);
+      }
+      for (int k = 0; k < 3; ++k) {
+        const float *p = m.verts + 3 * (size_t)idx[k], *q = m.verts + 3 * (size_t)idx[(k + 1) % 3];
+        double e2 = 0.0;
+        for (int c = 0; c < 3; ++c) e2 += ((double)p[c] - q[c]) * ((double)p[c] - q[c]);
+        edge2 = std::max(edge2, e2);
       }
       int need = 0;
       for (int k = 0; k < 3; ++k) {
@@ -497,6 +507,7 @@ int perch_load_meshes(perch_ctx* ctx, const perch_mesh* meshes, int32_t n) {
       cur_t.push_back(pk);
     }
     flush();
+    d.edge = (float)(std::sqrt(edge2) * (1.0 + 1e-5));
     d.chunk_count = (int)info.size() - d.chunk_begin;
     max_ml = std::max(max_ml, d.chunk_count);
     max_tris = std::max(max_tris, m.n_tris);

@@ -85,7 +85,7 @@ struct perch_ctx {
   int max_obs = 0;                // largest cloud over the scenes
 
   // camera-frame pose tables and the screen box of every (mesh, pose)
-  DevBuf yaw_mats, pose_off, vtab, pose_bbox;
+  DevBuf yaw_mats, pose_off, vtab, pose_bbox, pose_general;
   bool tables_valid = false;
   int tile_w = 0, tile_h = 0;             // largest over all meshes
   std::vector<int> mesh_tile_w, mesh_tile_h;  // per mesh
@@ -169,7 +169,7 @@ struct perch_ctx {
   std::vector<DevBuf*> all_buffers() {
     return {&meshes, &chunk_verts, &chunk_info, &chunk_tris, &vol_normals, &yaw_mats, &pose_off, &vtab, &xs, &ys, &cs, &depth, &rx, &ry, &blockcnt, &blockoff,
             &scan_tmp, &cam_pts, &world_pts, &keys, &counts, &cursor, &d_scenes, &d_scene_img,
-            &scratch_small, &pose_bbox, &parent_z, &uset, &uset_count, &b_parents, &b_plen, &b_hp, &b_hyp,
+            &scratch_small, &pose_bbox, &pose_general, &parent_z, &uset, &uset_count, &b_parents, &b_plen, &b_hp, &b_hyp,
             &b_out, &g_hist, &g_off, &g_cursor, &g_order, &g_next, &net_crops, &net_onehot, &net_pred,
             &solo, &solo_rec, &solo_hyp, &solo_hp, &solo_parent, &ptile_counts, &ptile_sat, &skip, &n_short,
             &tile_store, &tile_off, &tile_sizes, &pose_flags, &pg_cnt, &pg_start, &pg_flag, &pg_gix, &pg_gpose,

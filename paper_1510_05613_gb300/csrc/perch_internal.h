@@ -12,14 +12,15 @@ namespace perch {
 constexpr uint32_t kInfBits = 0x7f800000u;  // +inf: empty z-buffer pixel
 constexpr uint32_t kFlagBadIndex = 0x80000000u;
 constexpr uint32_t kFlagTimeout = 0x40000000u;  // a bounded wait in the kernel gave up
-constexpr int kChunkMaxVerts = 512;   // vertices of one mesh chunk (10-bit local indices)
-constexpr int kChunkMaxTris = 1024;   // triangles of one mesh chunk (list padded to 4 entries)
+constexpr int kChunkMaxVerts = 680;   // vertices of one mesh chunk (10-bit local indices)
+constexpr int kChunkMaxTris = 1536;   // triangles of one mesh chunk
 constexpr int kEvalThreads = 256;
 constexpr int kEvalWarps = kEvalThreads / 32;
 constexpr int kInlinePixels = 16;  // a lane tests at most this many pixel centres per triangle (k_eval;
                                    // k_render takes 8, 16 or 32 per mesh from the autotuner)
 constexpr int kBigQueue = 128;     // per-chunk queue of larger triangles, shared by the CTA
 constexpr int kWaitSpins = 1 << 20;  // bound on mbarrier polls before a kernel gives up
+constexpr int kSmallPixels = 60;  // triangles of at most this extent have exact binary32 edge values
 constexpr int kMaxObjectPixels = 1000;  // screen box limit that keeps edge arithmetic in int32
 constexpr float kNearZ = 0.05f;    // cull: vertex depth at or below this
 constexpr float kGuard = 2048.0f;  // cull: |u| or |v| beyond this (pixels)
@@ -35,12 +36,13 @@ struct Camera {
   float delta, delta2;
 };
 
-// One object type, split into chunks of <= 512 vertices / <= 1024 triangles.
+// One object type, split into chunks of <= 680 vertices / <= 1536 triangles.
 struct DevMesh {
   int chunk_begin, chunk_count;
   int n_tris, n_verts;
   float vol_r2, vol_zlo, vol_zhi;  // the inscribed cylinder (also the crops' reference height)
   float lo[3], hi[3];  // object-frame bounding box
+  float edge;          // longest triangle edge, rounded up
   float fp_r;          // max(largest horizontal vertex radius, V(O) radius), rounded up
   // V(O) (in_volume): kind 0 the inscribed cylinder; 1 box, p = (half x,
   // half y); 2 regular prism of vol_n <= 256 sides, p = (apothem, quick
@@ -79,13 +81,14 @@ struct Geometry {
   const uint32_t* chunk_tris; // 3 x 10-bit chunk-local vertex indices
   const float4* chunk_verts;  // object-frame positions, chunk order (all meshes)
   int n_cverts;               // length of chunk_verts
-  const float4* vtab;         // per yaw: M_yaw * v for every chunk vertex (n_yaw x n_cverts)
+  const float* vtab;          // per yaw: M_yaw * v for every chunk vertex (n_yaw x n_cverts x 3)
   const float4* pose_off;     // per (ix, iy): b = R_cw (x, y, 0) + t_cw
   const float* xs;
   const float* ys;
   const float2* cs;
   int nx, ny, n_yaw;
   const int4* pose_bbox;  // per (mesh, ix, iy, iyaw): x0, y0, w, h in pixels
+  const uint8_t* pose_general;  // per (mesh, pose): 1 = tile renders take the general triangle path
   const float* rx;        // ray slope per column
   const float* ry;        // ray slope per row
   const float2* vol_normals;  // face normals of the prism volumes
@@ -207,9 +210,9 @@ cudaError_t launch_scatter(const int* keys, int n, int* cursor, const float4* a_
 cudaError_t launch_rays(const Camera& cam, float* rx, float* ry, cudaStream_t s);
 cudaError_t launch_dilate3(const int* start3, int n3x, int n3y, int n3z, uint32_t* dil3, cudaStream_t s);
 cudaError_t launch_pose_tables(const Camera& cam, const Geometry& g, float* yaw_mats, float4* pose_off,
-                               float4* vtab, cudaStream_t s);
+                               float* vtab, cudaStream_t s);
 cudaError_t launch_pose_bbox(const Camera& cam, const Geometry& g, const float* yaw_mats, int4* bbox,
-                             int* max_wh, int* bad, cudaStream_t s);
+                             int* max_wh, int* bad, uint8_t* general, cudaStream_t s);
 cudaError_t launch_render_parents(const Camera& cam, const Geometry& g, const Batch& b, int max_chunks,
                                   unsigned long long* culled, cudaStream_t s);
 cudaError_t launch_uset(const Camera& cam, const Geometry& g, const ObsIndex& obs, const Batch& b,
