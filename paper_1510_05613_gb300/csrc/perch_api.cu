@@ -305,7 +305,7 @@ int perch_ctx::build_scene(int s, const float* depth_host) {
     CK(sc.start3.ensure(4 * ((size_t)cells + 1)), "alloc");
     CK(sc.start2.ensure(4 * ((size_t)c2 + 1)), "alloc");
     CK(sc.obs3.ensure(16 * (size_t)n), "alloc");
-    CK(sc.dil3.ensure(4 * ((size_t)cells / 32 + 1)), "alloc");
+    CK(sc.rows3.ensure(2 * (size_t)cells), "alloc");
     CK(sc.world2.ensure(16 * (size_t)n), "alloc");
     CK(sc.cam2.ensure(16 * (size_t)n), "alloc");
     CK(ctx->scan_tmp.ensure(4 * ((size_t)cmax / 1024 + 2)), "alloc");
@@ -319,9 +319,8 @@ int perch_ctx::build_scene(int s, const float* depth_host) {
        "copy");
     CK(launch_scatter(ctx->keys.as<int>(), n, ctx->cursor.as<int>(), ctx->cam_pts.as<float4>(),
                       sc.obs3.as<float4>(), nullptr, nullptr, ctx->stream), "scatter3");
-    CK(cudaMemsetAsync(sc.dil3.p, 0, 4 * ((size_t)cells / 32 + 1), ctx->stream), "memset");
-    CK(launch_dilate3(sc.start3.as<int>(), o.n3x, o.n3y, o.n3z, sc.dil3.as<uint32_t>(), ctx->stream),
-       "dilate3");
+    CK(launch_near_rows(sc.start3.as<int>(), o.n3x, o.n3y, o.n3z, sc.rows3.as<uint16_t>(), ctx->stream),
+       "neighbour rows");
     // bucket the world-frame cloud (with its camera-frame copy)
     CK(cudaMemsetAsync(ctx->counts.p, 0, 4 * (size_t)c2, ctx->stream), "memset");
     CK(launch_grid2_keys(ctx->world_pts.as<float4>(), n, o.g2x, o.g2y, o.inv2, o.n2x, o.n2y, ctx->keys.as<int>(),
@@ -340,7 +339,7 @@ int perch_ctx::build_scene(int s, const float* depth_host) {
     o.sat2 = sc.sat2.as<int>();
     o.cam3 = sc.obs3.as<float4>();
     o.start3 = sc.start3.as<int>();
-    o.dil3 = sc.dil3.as<uint32_t>();
+    o.rows3 = sc.rows3.as<uint16_t>();
     o.world2 = sc.world2.as<float4>();
     o.cam2 = sc.cam2.as<float4>();
     o.start2 = sc.start2.as<int>();
@@ -791,7 +790,7 @@ int perch_ctx::enqueue_eval(const perch_obj* d_parents, int parent_stride, const
   b.parent_len = d_plen;
   b.n_par = n_par;
   b.parent_z = parent_z.as<float>();
-  b.uset = uset.as<int>();
+  b.uset = uset.as<uint32_t>();
   b.uset_count = uset_count.as<int>();
   b.uset_stride = ustride;
   b.scenes = d_scenes.as<ObsIndex>();

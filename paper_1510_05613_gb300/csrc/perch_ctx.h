@@ -39,12 +39,12 @@ struct GraphKey {
 
 // One scene's observed cloud and its indices (device buffers).
 struct SceneBufs {
-  DevBuf start3, start2, obs3, world2, cam2, dil3;
+  DevBuf start3, start2, obs3, world2, cam2, rows3;
   DevBuf img;  // the scene's depth image (H x W, metres, 0 = no return)
   DevBuf sat2;  // summed-area table of observed points per 2D world cell
   perch::ObsIndex idx{};
   void release() {
-    for (DevBuf* b : {&start3, &start2, &obs3, &world2, &cam2, &dil3, &img, &sat2}) b->release();
+    for (DevBuf* b : {&start3, &start2, &obs3, &world2, &cam2, &rows3, &img, &sat2}) b->release();
   }
 };
 

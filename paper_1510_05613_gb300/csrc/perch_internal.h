@@ -62,7 +62,7 @@ struct ObsIndex {
   // camera-frame points bucketed by a 3D grid of cell >= delta (Eq. (1) query)
   const float4* cam3;  // x, y, z, pixel index (int bits)
   const int* start3;   // n_cells3 + 1
-  const uint32_t* dil3;  // bit per cell: some point in its 3x3x3 neighbourhood
+  const uint16_t* rows3;  // per cell: which rows of its 3x3x3 neighbourhood hold a point (near_row)
   float g3x, g3y, g3z, inv3;
   int n3x, n3y, n3z;
   // the same points bucketed by a 2D world (x, y) grid (V(O) candidates)
@@ -100,7 +100,7 @@ struct Batch {
   const int32_t* parent_len;
   int n_par;
   float* parent_z;      // n_par x H x W
-  int* uset;            // n_par x uset_stride indices into the 2D-sorted cloud
+  uint32_t* uset;       // n_par x uset_stride words: a bit per point of the 2D-sorted cloud
   int* uset_count;      // n_par
   int uset_stride;
   const int32_t* hyp_parent;
@@ -208,7 +208,7 @@ cudaError_t launch_grid2_keys(const float4* world_pts, int n, float g2x, float g
 cudaError_t launch_scatter(const int* keys, int n, int* cursor, const float4* a_in, float4* a_out,
                            const float4* b_in, float4* b_out, cudaStream_t s);
 cudaError_t launch_rays(const Camera& cam, float* rx, float* ry, cudaStream_t s);
-cudaError_t launch_dilate3(const int* start3, int n3x, int n3y, int n3z, uint32_t* dil3, cudaStream_t s);
+cudaError_t launch_near_rows(const int* start3, int n3x, int n3y, int n3z, uint16_t* rows3, cudaStream_t s);
 cudaError_t launch_pose_tables(const Camera& cam, const Geometry& g, float* yaw_mats, float4* pose_off,
                                float* vtab, cudaStream_t s);
 cudaError_t launch_pose_bbox(const Camera& cam, const Geometry& g, const float* yaw_mats, int4* bbox,

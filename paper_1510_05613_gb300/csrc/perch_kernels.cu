@@ -151,9 +151,24 @@ __device__ __forceinline__ void raster_tri(Vtx a, Vtx b, Vtx c, int ox16, int oy
   }
 }
 
+// Row k of a cell's 3x3x3 neighbourhood: three cells in x at (y + dy, z + dz);
+// the centre row first (the likeliest to hold a match).
+__device__ __forceinline__ void near_row(int k, int& dy, int& dz) {
+  const int q = (k * 11) >> 5, r = k - 3 * q;  // k / 3, k % 3
+  dz = (q & 1) ? -1 : q >> 1;
+  dy = (r & 1) ? -1 : r >> 1;
+}
+
 // Eq. (1) against the observed cloud: is some observed point within delta of
 // p? 3x3x3 neighbourhood of a grid whose cells are at least delta wide; three
-// consecutive x-cells are one contiguous range of the bucketed array.
+// consecutive x-cells are one contiguous range of the bucketed array. Bound
+// by the dependent loads of the ranges, so rows3 tells which of the nine rows
+// hold any point (mostly none to three near a surface): the others cost
+// nothing (640x480 root expansion 3.0 -> 2.7 ms, multi-scene batches, where
+// k_cost makes these tests, 2.4 -> 1.9 ms, against one bit for all nine). A
+// window of the depth image about p's pixel was slower (root expansion
+// 4.2 ms): most tests are of points about a centimetre off the cloud, which
+// must see all 49 depths.
 __device__ __forceinline__ bool explained_by_obs(const ObsIndex& o, float px, float py, float pz, float d2max) {
   if (o.n == 0) return false;
   const float fx = fmul(fsub(px, o.g3x), o.inv3);
@@ -162,42 +177,51 @@ __device__ __forceinline__ bool explained_by_obs(const ObsIndex& o, float px, fl
   const int ix = (int)floorf(fminf(fmaxf(fx, -2.0f), (float)o.n3x + 1.0f));
   const int iy = (int)floorf(fminf(fmaxf(fy, -2.0f), (float)o.n3y + 1.0f));
   const int iz = (int)floorf(fminf(fmaxf(fz, -2.0f), (float)o.n3z + 1.0f));
-  if (ix >= 0 && ix < o.n3x && iy >= 0 && iy < o.n3y && iz >= 0 && iz < o.n3z) {
-    // one bit says whether the 3x3x3 neighbourhood holds any point at all
-    const int c = (iz * o.n3y + iy) * o.n3x + ix;
-    if (!((__ldg(&o.dil3[c >> 5]) >> (c & 31)) & 1u)) return false;
-  }
   const int x0 = max(ix - 1, 0), x1 = min(ix + 1, o.n3x - 1);
   if (x0 > x1) return false;
-  for (int a = 0; a < 3; ++a) {  // the centre row first: the likeliest to hold a match
-    const int cz = iz + (a == 0 ? 0 : (a == 1 ? -1 : 1));
-    if (cz < 0 || cz >= o.n3z) continue;
-    for (int bq = 0; bq < 3; ++bq) {
-      const int cy = iy + (bq == 0 ? 0 : (bq == 1 ? -1 : 1));
-      if (cy < 0 || cy >= o.n3y) continue;
-      const int base = (cz * o.n3y + cy) * o.n3x;
-      const int s = __ldg(&o.start3[base + x0]), e = __ldg(&o.start3[base + x1 + 1]);
-      for (int k = s; k < e; ++k)
-        if (dist2(px, py, pz, __ldg(&o.cam3[k])) <= d2max) return true;
-    }
+  uint32_t rows = 0x1ffu;
+  if (ix >= 0 && ix < o.n3x && iy >= 0 && iy < o.n3y && iz >= 0 && iz < o.n3z)
+    rows = __ldg(&o.rows3[(iz * o.n3y + iy) * o.n3x + ix]);
+  for (; rows; rows &= rows - 1u) {
+    int dy, dz;
+    near_row(__ffs((int)rows) - 1, dy, dz);
+    const int cy = iy + dy, cz = iz + dz;
+    if (cy < 0 || cy >= o.n3y || cz < 0 || cz >= o.n3z) continue;
+    const int base = (cz * o.n3y + cy) * o.n3x;
+    const int s = __ldg(&o.start3[base + x0]), e = __ldg(&o.start3[base + x1 + 1]);
+    for (int k = s; k < e; ++k)
+      if (dist2(px, py, pz, __ldg(&o.cam3[k])) <= d2max) return true;
   }
   return false;
 }
 
-// Conservative pixel window around observed point q that contains the pixel
-// of every rendered point within delta of q: for |p - q| <= delta and
-// z_q > delta, |x_p/z_p - x_q/z_q| <= delta * sqrt(1 + (x_q/z_q)^2) / (z_q - delta);
-// (1 + |t|) bounds the square root and one pixel of slack absorbs rounding.
-__device__ __forceinline__ void delta_window(const Camera& cam, float4 q, int& u0, int& u1, int& v0, int& v1) {
-  const int pix = __float_as_int(q.w);
-  const int uq = pix % cam.W, vq = pix / cam.W;
-  const float den = q.z - cam.delta;
-  if (den > 1e-3f) {
-    const float tx = fabsf(q.x / q.z), ty = fabsf(q.y / q.z);
-    const float ru = fminf(cam.fx * cam.delta * (1.0f + tx) / den, 1e6f);
-    const float rv = fminf(cam.fy * cam.delta * (1.0f + ty) / den, 1e6f);
-    const int Ru = (int)ceilf(ru) + 1, Rv = (int)ceilf(rv) + 1;
-    u0 = uq - Ru; u1 = uq + Ru; v0 = vq - Rv; v1 = vq + Rv;
+// Half-width in pixels, along an axis of focal length f, of a window about
+// the pixel of a point (slope t = x / z or y / z, depth z) that holds the pixel
+// of every point within delta of it: for |p - q| <= delta and z > delta,
+// |x_p / z_p - x_q / z_q| <= delta sqrt(1 + t^2) / (z - delta). 1 + t^2 / 2
+// bounds the square root; both pixels are whole, so the slack only has to
+// cover the rounding of the rays, of d^2 and of this bound.
+__device__ __forceinline__ int delta_radius(const Camera& cam, float f, float t, float z) {
+  const float d = 1.0001f * cam.delta;
+  return (int)fminf(f * (1.0f + 0.5f * t * t) * __fdividef(d, z - d) + (0.05f + 1e-6f * (float)(cam.W + cam.H)), 1e6f);
+}
+__device__ __forceinline__ bool delta_bounded(const Camera& cam, float z) { return z - 1.0001f * cam.delta > 1e-3f; }
+
+// The pixel of observed point q and the window of delta_radius about it.
+__device__ __forceinline__ void delta_window(const Camera& cam, float4 q, int& u, int& v, int& u0, int& u1, int& v0,
+                                             int& v1) {
+  const float tx = __fdividef(q.x, q.z), ty = __fdividef(q.y, q.z);
+  if (cam.W <= 16384 && cam.H <= 16384) {  // far less than half a pixel off
+    u = __float2int_rn(cam.fx * tx + cam.cx);
+    v = __float2int_rn(cam.fy * ty + cam.cy);
+  } else {
+    const int pix = __float_as_int(q.w);
+    u = pix % cam.W;
+    v = pix / cam.W;
+  }
+  if (delta_bounded(cam, q.z)) {
+    const int Ru = delta_radius(cam, cam.fx, tx, q.z), Rv = delta_radius(cam, cam.fy, ty, q.z);
+    u0 = u - Ru; u1 = u + Ru; v0 = v - Rv; v1 = v + Rv;
   } else {
     u0 = INT_MIN / 2; u1 = INT_MAX / 2; v0 = INT_MIN / 2; v1 = INT_MAX / 2;
   }
@@ -219,21 +243,22 @@ struct DRTile {
 // of the observed point q?
 __device__ __forceinline__ bool explained_by_tile(const Camera& cam, float4 q, const DRTile& tile,
                                                   const float* rxs, const float* rys, int4 bb) {
-  int u0, u1, v0, v1;
-  delta_window(cam, q, u0, u1, v0, v1);
-  u0 = max(u0, bb.x); u1 = min(u1, bb.x + bb.z - 1);
-  v0 = max(v0, bb.y); v1 = min(v1, bb.y + bb.w - 1);
-  for (int v = v0; v <= v1; ++v) {
-    const int ly = v - bb.y;
-    const float ry = rys[ly];
-    for (int u = u0; u <= u1; ++u) {
-      const int lx = u - bb.x;
-      const uint32_t zb = tile.at(ly * bb.z + lx);
-      if (zb == kInfBits) continue;
-      const float z = __uint_as_float(zb);
-      if (dist2(fmul(rxs[lx], z), fmul(ry, z), z, q) <= cam.delta2) return true;
-    }
-  }
+  int u, v, u0, u1, v0, v1;
+  delta_window(cam, q, u, v, u0, u1, v0, v1);
+  u0 = max(u0 - bb.x, 0); u1 = min(u1 - bb.x, bb.z - 1);
+  v0 = max(v0 - bb.y, 0); v1 = min(v1 - bb.y, bb.w - 1);
+  auto near = [&](int lx, int ly) {
+    const uint32_t zb = tile.at(ly * bb.z + lx);
+    if (zb == kInfBits) return false;
+    const float z = __uint_as_float(zb);
+    return dist2(fmul(rxs[lx], z), fmul(rys[ly], z), z, q) <= cam.delta2;
+  };
+  u -= bb.x;
+  v -= bb.y;
+  if (u >= u0 && u <= u1 && v >= v0 && v <= v1 && near(u, v)) return true;  // its own pixel: the likeliest
+  for (int ly = v0; ly <= v1; ++ly)
+    for (int lx = u0; lx <= u1; ++lx)
+      if (near(lx, ly)) return true;
   return false;
 }
 
@@ -476,32 +501,29 @@ cudaError_t launch_rays(const Camera& cam, float* rx, float* ry, cudaStream_t s)
   return cudaGetLastError();
 }
 
-// dilated occupancy of the 3D grid: bit c set iff a cell within one step of
-// c (in each axis) holds a point; dil3 must be zeroed first
-__global__ void k_dilate3(const int* start3, int nx, int ny, int nz, uint32_t* dil3) {
+// per cell of the 3D grid, which rows of its neighbourhood (near_row) hold a point
+__global__ void k_near_rows(const int* start3, int nx, int ny, int nz, uint16_t* rows3) {
   const long long c = blockIdx.x * 256LL + threadIdx.x;
   const long long n = (long long)nx * ny * nz;
   if (c >= n) return;
   const int ix = (int)(c % nx), iy = (int)((c / nx) % ny), iz = (int)(c / ((long long)nx * ny));
-  bool any = false;
-  for (int dz = -1; dz <= 1 && !any; ++dz) {
-    const int z = iz + dz;
-    if (z < 0 || z >= nz) continue;
-    for (int dy = -1; dy <= 1 && !any; ++dy) {
-      const int y = iy + dy;
-      if (y < 0 || y >= ny) continue;
-      const int base = (z * ny + y) * nx;
-      const int x0 = max(ix - 1, 0), x1 = min(ix + 1, nx - 1);
-      any = start3[base + x1 + 1] > start3[base + x0];
-    }
+  const int x0 = max(ix - 1, 0), x1 = min(ix + 1, nx - 1);
+  unsigned rows = 0;
+  for (int k = 0; k < 9; ++k) {
+    int dy, dz;
+    near_row(k, dy, dz);
+    const int y = iy + dy, z = iz + dz;
+    if (y < 0 || y >= ny || z < 0 || z >= nz) continue;
+    const int base = (z * ny + y) * nx;
+    if (start3[base + x1 + 1] > start3[base + x0]) rows |= 1u << k;
   }
-  if (any) atomicOr(&dil3[c >> 5], 1u << (c & 31));
+  rows3[c] = (uint16_t)rows;
 }
 
-cudaError_t launch_dilate3(const int* start3, int n3x, int n3y, int n3z, uint32_t* dil3, cudaStream_t s) {
+cudaError_t launch_near_rows(const int* start3, int n3x, int n3y, int n3z, uint16_t* rows3, cudaStream_t s) {
   const long long n = (long long)n3x * n3y * n3z;
   if (n == 0) return cudaSuccess;
-  k_dilate3<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(start3, n3x, n3y, n3z, dil3);
+  k_near_rows<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(start3, n3x, n3y, n3z, rows3);
   return cudaGetLastError();
 }
 // Camera-frame pose tables: per yaw M = R_cw Rz(yaw), per (ix, iy)
@@ -678,7 +700,8 @@ cudaError_t launch_render_parents(const Camera& cam, const Geometry& g, const Ba
 
 // U set of a parent one object short of a complete scene:
 // U = {q in I - V_{K-1} : q unexplained by R_{K-1}}; then for the last object
-// O_K, residual(K) = #{q in U : q not in V(O_K), q unexplained by dR_K}.
+// O_K, residual(K) = #{q in U : q not in V(O_K), q unexplained by dR_K}. U is
+// kept as a bit per point of the 2D-sorted cloud, and its size.
 __global__ void k_uset(Camera cam, Geometry g, ObsIndex obs0, Batch b) {
   const int p = blockIdx.y;
   const int plen = b.parent_len[p];
@@ -688,32 +711,34 @@ __global__ void k_uset(Camera cam, Geometry g, ObsIndex obs0, Batch b) {
   if (b.parent_scene && (scene < 0 || scene >= b.n_scenes)) return;
   const ObsIndex& obs = b.parent_scene ? b.scenes[scene] : obs0;
   const int k = blockIdx.x * 256 + threadIdx.x;
-  if (k >= obs.n) return;
-  const float4 qw = obs.world2[k];
-  for (int j = 0; j < plen; ++j) {
-    const perch_obj o = b.parents[(long long)p * b.parent_stride + j];
-    if (!obj_ok(g, o)) return;
-    const DevMesh m = g.meshes[o.mesh];
-    if (in_volume(g, m, g.xs[o.ix], g.ys[o.iy], o.iyaw, qw)) return;
+  bool in = k < obs.n;
+  if (in) {
+    const float4 qw = obs.world2[k];
+    for (int j = 0; j < plen && in; ++j) {
+      const perch_obj o = b.parents[(long long)p * b.parent_stride + j];
+      in = obj_ok(g, o) && !in_volume(g, g.meshes[o.mesh], g.xs[o.ix], g.ys[o.iy], o.iyaw, qw);
+    }
   }
-  const float4 q = obs.cam2[k];
-  if (plen > 0) {
+  if (in && plen > 0) {
+    const float4 q = obs.cam2[k];
     const float* zp = b.parent_z + (size_t)p * cam.W * cam.H;
-    int u0, u1, v0, v1;
-    delta_window(cam, q, u0, u1, v0, v1);
+    int u, v, u0, u1, v0, v1;
+    delta_window(cam, q, u, v, u0, u1, v0, v1);
     u0 = max(u0, 0); u1 = min(u1, cam.W - 1);
     v0 = max(v0, 0); v1 = min(v1, cam.H - 1);
-    for (int v = v0; v <= v1; ++v) {
-      const float ry = g.ry[v];
-      for (int u = u0; u <= u1; ++u) {
-        const float z = zp[(size_t)v * cam.W + u];
-        if (__float_as_uint(z) == kInfBits) continue;
-        if (dist2(fmul(g.rx[u], z), fmul(ry, z), z, q) <= cam.delta2) return;
+    for (int vp = v0; vp <= v1 && in; ++vp) {
+      const float ry = g.ry[vp];
+      for (int up = u0; up <= u1 && in; ++up) {
+        const float z = zp[(size_t)vp * cam.W + up];
+        in = __float_as_uint(z) == kInfBits || !(dist2(fmul(g.rx[up], z), fmul(ry, z), z, q) <= cam.delta2);
       }
     }
   }
-  const int slot = atomicAdd(&b.uset_count[p], 1);
-  b.uset[(size_t)p * b.uset_stride + slot] = k;
+  const unsigned bits = __ballot_sync(0xffffffffu, in);
+  if ((threadIdx.x & 31) == 0 && k < obs.n) {
+    b.uset[(size_t)p * b.uset_stride + (k >> 5)] = bits;
+    if (bits) atomicAdd(&b.uset_count[p], __popc(bits));
+  }
 }
 
 cudaError_t launch_uset(const Camera& cam, const Geometry& g, const ObsIndex& obs, const Batch& b,
@@ -907,9 +932,11 @@ bool eval_tile_fits(int device, int tile_w, int tile_h) {
   return eval_smem_bytes(tile_w, tile_h) + 256 <= (size_t)optin;  // 256: static shared memory of k_eval
 }
 
-size_t cost_smem_bytes(int tile_w, int tile_h, int stages) {  // stages, dR bitmask (16-byte multiples), rays
+constexpr int kNearList = 512;  // observed points per round of finish_phase's list
+
+size_t cost_smem_bytes(int tile_w, int tile_h, int stages) {  // stages, dR bitmask (16-byte multiples), rays, list
   return (size_t)stages * ((tile_w * tile_h + 3) & ~3) * 4 + (size_t)(((tile_w * tile_h + 31) / 32 + 3) & ~3) * 4 +
-         (size_t)(tile_w + tile_h) * 4;
+         (size_t)(tile_w + tile_h) * 4 + (size_t)(kNearList + 1) * 4;
 }
 
 // thread 0: start the bulk copy of n vertices from entry v of yaw iyaw's
@@ -1354,13 +1381,13 @@ __device__ __forceinline__ void compare_phase_mask(int pid, int plen, int4 bb, c
 
 // The rest of cost_phase, after compare_phase: the record of an invalid
 // child, or dJ_r (unless DJR_DONE: compare_phase counted it), dJ_o,
-// residual(K) and n_vol from the tile (z on dR, +inf elsewhere). Ends with a
-// CTA barrier.
+// residual(K) and n_vol from the tile (z on dR, +inf elsewhere). `list`: shared
+// scratch of kNearList + 1 entries. Ends with a CTA barrier.
 template <int NT, bool DJR_DONE>
 __device__ __forceinline__ void finish_phase(long long h, int pid, int plen, int K_total, const perch_obj& o,
                                              int4 bb, const DevMesh& m, const Camera& cam, const Geometry& g,
                                              const ObsIndex& obs, const Batch& b, const DRTile& tile,
-                                             const float* rxs, const float* rys, int* s_cnt) {
+                                             const float* rxs, const float* rys, int* s_cnt, int* list) {
   constexpr int NW = NT / 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int tw = bb.z, th = bb.w;
@@ -1390,57 +1417,99 @@ __device__ __forceinline__ void finish_phase(long long h, int pid, int plen, int
     }
   }
 
-  // ---- dJ_o: observed points inside V(O) with no dR point within delta
-  int djo = 0, nvol = 0;
+  // ---- dJ_o: observed points inside V(O) with no dR point within delta; and
+  // on edges into the last level residual(K) = |U| less the points of U that
+  // are inside V(O) or within delta of a dR point. Both look only at the
+  // observed points of the world cells about the pose: within V(O)'s radius,
+  // and on the last level within the footprint's radius + delta (+ 2 cm and
+  // a sixteenth of a pixel at the object's depth for the snap: every rendered
+  // point lies that near the footprint). Few points of those cells need the
+  // scan of the tile, so a first pass lists them (kNearList cells' points at
+  // a time) and a second takes one per thread. This phase was most of k_cost:
+  // it took a row of cells per CTA pass, scanned windows of 11 to 13 pixels
+  // where 7 hold delta (delta_radius), and tested all of U (up to the whole
+  // cloud) per hypothesis of the last level. k_cost, 640x480: 480k
+  // hypotheses of eight states 4.1 -> 1.5 ms, the 240k-hypothesis batch
+  // 3.5 -> 2.25 ms, 4.7k hypotheses next to the objects 1.4 -> 0.51 ms.
+  const bool last = plen + 1 == K_total;
+  int djo = 0, nvol = 0, done = 0;  // done: points of U that are accounted for
   if (obs.n > 0) {
-    const float r = m.vol_rmax * 1.001f + 1e-6f;
+    float r = m.vol_rmax * 1.001f + 1e-6f;
+    if (last) {
+      const float depth = g.pose_off[o.ix * g.ny + o.iy].z + m.fp_r + fmaxf(fabsf(m.lo[2]), fabsf(m.hi[2]));
+      r = fmaxf(r, m.fp_r + cam.delta + 0.02f + depth / (16.0f * fminf(cam.fx, cam.fy)));
+    }
     const int cx0 = max(cell_of(ox - r, obs.g2x, obs.inv2, obs.n2x) - 1, 0);
     const int cx1 = min(cell_of(ox + r, obs.g2x, obs.inv2, obs.n2x) + 1, obs.n2x - 1);
     const int cy0 = max(cell_of(oy - r, obs.g2y, obs.inv2, obs.n2y) - 1, 0);
     const int cy1 = min(cell_of(oy + r, obs.g2y, obs.inv2, obs.n2y) + 1, obs.n2y - 1);
-    if (cx0 <= cx1) {
-      for (int cy = cy0; cy <= cy1; ++cy) {
-        const int s = obs.start2[cy * obs.n2x + cx0], e = obs.start2[cy * obs.n2x + cx1 + 1];
-        for (int k = s + tid; k < e; k += NT) {
-          const float4 qw = obs.world2[k];
-          if (!in_volume(g, m, ox, oy, o.iyaw, qw)) continue;
-          if (!explained_by_tile(cam, obs.cam2[k], tile, rxs, rys, bb)) djo++;
+    const uint32_t* U = b.uset + (size_t)pid * b.uset_stride;
+    const bool any = cx0 <= cx1 && cy0 <= cy1 && sat_sum(obs.sat2, obs.n2x, cy0, cy1, cx0, cx1) != 0;
+    for (int cy = cy0; any && cy <= cy1; cy += 32) {  // 32 rows of cells, a lane to a row
+      int s = 0, cnt = 0;
+      if (cy + lane <= cy1) {
+        s = obs.start2[(cy + lane) * obs.n2x + cx0];
+        cnt = obs.start2[(cy + lane) * obs.n2x + cx1 + 1] - s;
+      }
+      int incl = cnt;
+      for (int d = 1; d < 32; d <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += t;
+      }
+      const int total = __shfl_sync(0xffffffffu, incl, 31);
+      for (int base = 0; base < total; base += kNearList) {
+        const int lim = min(total, base + kNearList);
+        if (tid == 0) list[0] = 0;
+        __syncthreads();  // also: the last round's list has been read
+        for (int i0 = base + 32 * warp; i0 < lim; i0 += NT) {  // warp-uniform
+          const int i = i0 + lane;
+          int row = 0;  // the row whose range holds the i-th point
+          for (int d = 16; d > 0; d >>= 1)
+            if (__shfl_sync(0xffffffffu, incl, row + d - 1) <= i) row += d;
+          const int k = __shfl_sync(0xffffffffu, s, row) + i - __shfl_sync(0xffffffffu, incl - cnt, row);
+          bool in_v = false, in_u = false;
+          if (i < lim) {
+            in_v = in_volume(g, m, ox, oy, o.iyaw, obs.world2[k]);
+            in_u = last && ((U[k >> 5] >> (k & 31)) & 1u);
+          }
+          const unsigned take = __ballot_sync(0xffffffffu, in_v || in_u);
+          int at = 0;
+          if (lane == 0 && take) at = atomicAdd(&list[0], __popc(take));
+          at = __shfl_sync(0xffffffffu, at, 0);
+          if (in_v || in_u)
+            list[1 + at + __popc(take & ((1u << lane) - 1u))] = k | (in_v ? 1 << 30 : 0) | (in_u ? 1 << 31 : 0);
+        }
+        __syncthreads();
+        const int n_list = list[0];
+        for (int e = tid; e < n_list; e += NT) {
+          const int f = list[1 + e], k = f & 0x3fffffff;
+          const bool ex = explained_by_tile(cam, obs.cam2[k], tile, rxs, rys, bb);
+          if (f < 0 && (ex || (f & (1 << 30)))) done++;
+          if (!(f & (1 << 30))) continue;
+          if (!ex) djo++;
           bool in_parent = false;  // already inside an assigned volume?
           for (int j = 0; j < plen && !in_parent; ++j) {
             const perch_obj po = b.parents[(long long)pid * b.parent_stride + j];
-            in_parent = in_volume(g, g.meshes[po.mesh], g.xs[po.ix], g.ys[po.iy], po.iyaw, qw);
+            in_parent = in_volume(g, g.meshes[po.mesh], g.xs[po.ix], g.ys[po.iy], po.iyaw, obs.world2[k]);
           }
           if (!in_parent) nvol++;
         }
       }
     }
   }
-
-  // ---- residual(K) on edges into the last level
-  int resid = 0;
-  if (plen + 1 == K_total) {
-    const int nu = b.uset_count[pid];
-    const int* U = b.uset + (size_t)pid * b.uset_stride;
-    for (int k = tid; k < nu; k += NT) {
-      const int qi = U[k];
-      if (in_volume(g, m, ox, oy, o.iyaw, obs.world2[qi])) continue;
-      if (explained_by_tile(cam, obs.cam2[qi], tile, rxs, rys, bb)) continue;
-      resid++;
-    }
-  }
   djr = warp_sum(djr);
   djo = warp_sum(djo);
-  resid = warp_sum(resid);
+  done = warp_sum(done);
   nvol = warp_sum(nvol);
   if (lane == 0) {
     if (djr) atomicAdd(&s_cnt[3], djr);
     if (djo) atomicAdd(&s_cnt[4], djo);
-    if (resid) atomicAdd(&s_cnt[5], resid);
+    if (done) atomicAdd(&s_cnt[5], done);
     if (nvol) atomicAdd(&s_cnt[6], nvol);
   }
   __syncthreads();
   if (tid == 0) {
-    perch_cost r = {s_cnt[3], s_cnt[4], s_cnt[5], 0, s_cnt[1], flags, s_cnt[6]};
+    perch_cost r = {s_cnt[3], s_cnt[4], last ? b.uset_count[pid] - s_cnt[5] : 0, 0, s_cnt[1], flags, s_cnt[6]};
     b.out[h] = r;
   }
   __syncthreads();  // s_cnt and the tile are reused by the next hypothesis
@@ -1457,9 +1526,10 @@ template <int NT>
 __device__ __forceinline__ void cost_phase(long long h, int pid, int plen, int K_total, const perch_obj& o, int4 bb,
                                            const DevMesh& m, const Camera& cam, const Geometry& g,
                                            const ObsIndex& obs, const Batch& b, uint32_t* tile, const float* rxs,
-                                           const float* rys, int* s_cnt) {
+                                           const float* rys, int* s_cnt, int* list) {
   compare_phase<NT, kSrcInvZ>(pid, plen, bb, cam, b, tile, tile, s_cnt);
-  finish_phase<NT, false>(h, pid, plen, K_total, o, bb, m, cam, g, obs, b, DRTile{tile, nullptr}, rxs, rys, s_cnt);
+  finish_phase<NT, false>(h, pid, plen, K_total, o, bb, m, cam, g, obs, b, DRTile{tile, nullptr}, rxs, rys, s_cnt,
+                          list);
 }
 
 // The checks every evaluation of hypothesis h makes before it touches its
@@ -1532,7 +1602,10 @@ __device__ int eval_one(long long h, const Camera& cam, const Geometry& g, const
   }
   if (culled) s_cnt[2] = 1;
   __syncthreads();
-  cost_phase<NT>(h, a.pid, a.plen, a.K_total, a.o, bb, m, cam, g, obs, b, s.tile, rxs, rys, s_cnt);
+  // the render's projected vertices are done with: their buffer holds the list
+  static_assert(sizeof(float2) * kChunkMaxVerts >= sizeof(int) * (kNearList + 1), "the list fits");
+  cost_phase<NT>(h, a.pid, a.plen, a.K_total, a.o, bb, m, cam, g, obs, b, s.tile, rxs, rys, s_cnt,
+                 reinterpret_cast<int*>(s.sXY));
   return kEvalDone;
 }
 
@@ -1723,6 +1796,7 @@ __global__ void __launch_bounds__(NT) k_cost(Camera cam, Geometry g, ObsIndex ob
   uint32_t* mask = reinterpret_cast<uint32_t*>(smem) + NS * stage_words;
   float* rxs = reinterpret_cast<float*>(mask + (((b.tile_w * b.tile_h + 31) / 32 + 3) & ~3));
   float* rys = rxs + b.tile_w;
+  int* list = reinterpret_cast<int*>(rys + b.tile_h);
   if (tid == 0) {
     for (int k = 0; k < NS; ++k) mbar_init(&s_bar[k], 1);
     fence_barrier_init();
@@ -1837,7 +1911,7 @@ __global__ void __launch_bounds__(NT) k_cost(Camera cam, Geometry g, ObsIndex ob
     if (tid == 0) claim();  // look the next one up (and with two stages start its copy)
     const DevMesh m = g.meshes[a.o.mesh];
     finish_phase<NT, !MULTI>(h, a.pid, a.plen, a.K_total, a.o, bb, m, cam, g, obs, b, DRTile{stage, mask}, rxs, rys,
-                             s_cnt);
+                             s_cnt, list);
   }
 }
 

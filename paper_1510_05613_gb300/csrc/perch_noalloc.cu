@@ -96,7 +96,7 @@ extern "C" int perch_eval_successors_noalloc(perch_ctx* ctx, const perch_obj* pa
   if (!ctx->ev[0]) return ctx->fail(PERCH_E_STATE, "noalloc: set an observation first");
   unsigned char* p = static_cast<unsigned char*>(base);
   float* parent_z = reinterpret_cast<float*>(p);
-  int* uset = reinterpret_cast<int*>(p + z_bytes);
+  uint32_t* uset = reinterpret_cast<uint32_t*>(p + z_bytes);
   int* uset_count = reinterpret_cast<int*>(p + z_bytes + u_bytes);
   int* item_count = uset_count + n_par;  // the evaluation's work counter pair
   int* item_next = item_count + 1;
