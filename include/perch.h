@@ -310,8 +310,8 @@ enum { PERCH_ICP_CONVERGED = 0, PERCH_ICP_CAP = 1, PERCH_ICP_FEW = 2, PERCH_ICP_
  * call returns when out is written. Errors: PERCH_E_ARG (bad index, length,
  * radius or max_iter), PERCH_E_STATE (no observation), PERCH_E_DEVICE (a
  * record with bit 30 or 31). The first call after an observation builds
- * the cloud's world-frame grid of cells >= 1.05 radius (one more set of
- * device buffers, held by the context). */
+ * the cloud's world points by pixel (one more set of device buffers, held by
+ * the context; a world-frame grid where T_world_cam is no rotation). */
 int perch_icp_refine(perch_ctx* ctx, const perch_obj* parents, int32_t parent_stride, const int32_t* parent_len,
                      int32_t n_par, const int32_t* hyp_parent, const perch_obj* hyp, int64_t n_hyp, float radius,
                      int32_t max_iter, perch_icp* out);

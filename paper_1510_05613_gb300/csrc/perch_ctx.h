@@ -147,13 +147,15 @@ struct perch_ctx {
   // records, and in selecting states and building batches (learned scoring included)
   double search_eval_seconds = 0.0, search_absorb_seconds = 0.0, search_host_seconds = 0.0;
 
-  // ICP refinement (perch_icp_refine): scene 0's observed world points
-  // bucketed by a grid of cells >= 1.05 x the radius it was built for,
-  // rebuilt when the observation (obs_serial) or the radius changes
+  // ICP refinement (perch_icp_refine): scene 0's observed world points by
+  // pixel, rebuilt when the observation (obs_serial) changes; or, when the
+  // camera's matrix is no rotation, bucketed by a grid of cells of half the
+  // radius, rebuilt when the radius changes too
   long long obs_serial = 0, icp_serial = -1;
   float icp_radius = -1.0f;
   perch::IcpGrid icp_grid{};
-  DevBuf icp_src, icp_pts, icp_start, icp_next, icp_out, icp_prev;
+  perch::IcpImage icp_img{};
+  DevBuf icp_src, icp_pts, icp_start, icp_next, icp_out, icp_model, icp_img_pts, icp_img_lo, icp_img_hi;
 
   // poll bound of the evaluation kernel's first wait for each bulk copy
   // (perch_set_wait_limit); the solo table always uses the default
@@ -174,7 +176,7 @@ struct perch_ctx {
             &solo, &solo_rec, &solo_hyp, &solo_hp, &solo_parent, &ptile_counts, &ptile_sat, &skip, &n_short,
             &tile_store, &tile_off, &tile_sizes, &pose_flags, &pg_cnt, &pg_start, &pg_flag, &pg_gix, &pg_gpose,
             &pg_tmp, &pg_ranges, &pose_valid, &tile_box, &icp_src, &icp_pts, &icp_start, &icp_next,
-            &icp_out, &icp_prev};
+            &icp_out, &icp_model, &icp_img_pts, &icp_img_lo, &icp_img_hi};
   }
 
   int fail(int code, const char* fmt, ...);
@@ -188,6 +190,7 @@ struct perch_ctx {
   int create_events();
   int build_scene(int s, const float* depth_host);
   int ensure_solo();
+  int ensure_icp_cloud(float radius);
   int ensure_icp_grid(float radius);
   int enqueue_icp(const perch_obj* d_parents, int parent_stride, const int32_t* d_plen, int n_par,
                   const int32_t* d_hp, const perch_obj* d_hyp, long long n_hyp, float radius, int max_iter,

@@ -23,6 +23,40 @@ static float icp_ordered_to_float(int i) {
   return f;
 }
 
+// What the matchings search: the world points by pixel, or the grid when
+// the camera's matrix is too far from a rotation for the pixel windows'
+// bound (its transpose stands for its inverse there).
+int perch_ctx::ensure_icp_cloud(float radius) {
+  perch_ctx* ctx = this;
+  if (icp_serial == obs_serial && (icp_img.pts || icp_radius == radius)) return PERCH_OK;
+  double off = 0.0;
+  for (int i = 0; i < 3; ++i)
+    for (int j = 0; j < 3; ++j) {
+      double d = i == j ? -1.0 : 0.0;
+      for (int k = 0; k < 3; ++k) d += (double)cam.Rwc[k * 3 + i] * cam.Rwc[k * 3 + j];
+      off = std::max(off, std::fabs(d));
+    }
+  icp_img = IcpImage{};
+  if (!(off <= 1e-4)) return ensure_icp_grid(radius);
+  IcpImage q{};
+  q.stride = (cam.W + 3) / 4 * 4;
+  q.blocks_y = (cam.H + 3) / 4;
+  q.ortho = (float)(4.0 * off + 1e-6);
+  const size_t blocks = (size_t)(q.stride / 4) * q.blocks_y;
+  CK(icp_img_pts.ensure(16 * 16 * blocks), "alloc");
+  CK(icp_img_lo.ensure(16 * blocks), "alloc");
+  CK(icp_img_hi.ensure(16 * blocks), "alloc");
+  CK(launch_icp_image(scenes[0].img.as<float>(), cam, rx.as<float>(), ry.as<float>(), q, icp_img_pts.as<float4>(),
+                      icp_img_lo.as<float4>(), icp_img_hi.as<float4>(), stream),
+     "icp image");
+  q.pts = icp_img_pts.as<float4>();
+  q.lo = icp_img_lo.as<float4>();
+  q.hi = icp_img_hi.as<float4>();
+  icp_img = q;
+  icp_serial = obs_serial;
+  return PERCH_OK;
+}
+
 // Bucket scene 0's observed world points by a 3D grid of cells of half the
 // radius (at least 2.5 mm), grown by 1.25 until it has at most 16M cells.
 // The kernel scans the cells that meet its search cube, found with the same
@@ -110,9 +144,9 @@ int perch_ctx::enqueue_icp(const perch_obj* d_parents, int parent_stride, const 
   const size_t npx = (size_t)cam.W * cam.H;
   CK(parent_z.ensure(4 * npx * std::max(n_par, 1)), "alloc parent z-buffers");
   CK(icp_next.ensure(4), "alloc");
-  // each CTA's model list and pair memory: 4 CTAs per SM at most (k_icp's registers)
-  const long long prev_elems = 8LL * sm_count * tile_w * tile_h;
-  CK(icp_prev.ensure(4 * (size_t)std::max(prev_elems, 1LL)), "alloc");
+  // each CTA's model list: 4 CTAs per SM at most (k_icp's registers)
+  const long long model_elems = 4LL * sm_count * tile_w * tile_h;
+  CK(icp_model.ensure(16 * (size_t)std::max(model_elems, 1LL)), "alloc");
   Batch b;
   std::memset(&b, 0, sizeof b);
   b.parents = d_parents;
@@ -136,8 +170,10 @@ int perch_ctx::enqueue_icp(const perch_obj* d_parents, int parent_stride, const 
   w.rwin = (float)(1.01 * (double)radius + 1e-6);
   w.max_iter = max_iter;
   w.out = d_out;
-  w.prev = icp_prev.as<int>();
-  CK(launch_icp(cam, g, b, icp_grid, w, prev_elems, icp_next.as<int>(), sm_count, stream), "icp kernel");
+  w.model = icp_model.as<float4>();
+  w.obs = scenes[0].idx;
+  w.img = icp_img;
+  CK(launch_icp(cam, g, b, icp_grid, w, model_elems, icp_next.as<int>(), sm_count, stream), "icp kernel");
   return PERCH_OK;
 }
 
@@ -194,7 +230,7 @@ int perch_icp_refine(perch_ctx* ctx, const perch_obj* parents, int32_t parent_st
   CK(cudaSetDevice(ctx->device), "cudaSetDevice");
   rc = ctx->ensure_tables();
   if (rc) return rc;
-  rc = ctx->ensure_icp_grid(radius);
+  rc = ctx->ensure_icp_cloud(radius);
   if (rc) return rc;
   const size_t pbytes = sizeof(perch_obj) * std::max<size_t>((size_t)n_par * parent_stride, 1);
   CK(ctx->b_parents.ensure(pbytes), "alloc");
@@ -237,7 +273,7 @@ int perch_icp_refine_dev(perch_ctx* ctx, const perch_obj* parents, int32_t paren
   CK(cudaSetDevice(ctx->device), "cudaSetDevice");
   rc = ctx->ensure_tables();
   if (rc) return rc;
-  rc = ctx->ensure_icp_grid(radius);
+  rc = ctx->ensure_icp_cloud(radius);
   if (rc) return rc;
   return ctx->enqueue_icp(parents, parent_stride, parent_len, n_par, hyp_parent, hyp, n_hyp, radius, max_iter, out);
 }

@@ -186,12 +186,23 @@ struct IcpGrid {
   int nx, ny, nz;
 };
 
+// scene 0's world points by pixel (k_icp_image)
+struct IcpImage {
+  const float4* pts;      // rows of `stride` pixels (a multiple of 4), 4 blocks_y rows; NaN: none
+  const float4 *lo, *hi;  // the box of each 4 x 4 block's points
+  int stride, blocks_y;
+  float ortho;  // how far a point's camera coordinates can be off by the transposed matrix, relative to their sum
+};
+constexpr int kIcpDirect = 25;  // windows of at most this many pixels are scanned without their blocks' boxes
+
 struct IcpWork {
   float r2;      // (float)(radius^2)
-  float rwin;    // 1.01 radius + 1e-6 m: the search window before a pair is known
+  float rwin;    // 1.01 radius + 1e-6 m
   int max_iter;
   perch_icp* out;
-  int* prev;     // per CTA, 2 tile_w x tile_h entries: the model pixels, then each one's last paired point
+  float4* model;  // per CTA, tile_w x tile_h entries: a model point, and its last pair (int bits)
+  ObsIndex obs;   // scene 0 (its world grid says whether a successor meets the cloud)
+  IcpImage img;   // scene 0 by pixel; pts == nullptr: the camera's matrix is no rotation, use the grid
 };
 
 // kernels.cu launchers (all asynchronous on `s`)
@@ -259,8 +270,11 @@ cudaError_t launch_icp_points(const float4* world2, const float4* cam2, int n, f
 // ICP of each hypothesis of the batch (one CTA per hypothesis at a time,
 // claimed from the device counter `next`, zero before the launch; the
 // parents' renders must be in b.parent_z). The grid is capped so that every
-// CTA has its 2 tile_w x tile_h slice of w.prev (prev_elems entries in all).
+// CTA has its tile_w x tile_h slice of w.model (model_elems entries in all).
 cudaError_t launch_icp(const Camera& cam, const Geometry& g, const Batch& b, const IcpGrid& q, const IcpWork& w,
-                       long long prev_elems, int* next, int sm_count, cudaStream_t s);
+                       long long model_elems, int* next, int sm_count, cudaStream_t s);
+// scene 0's world points by pixel, and the boxes of their blocks
+cudaError_t launch_icp_image(const float* depth, const Camera& cam, const float* rx, const float* ry,
+                             const IcpImage& q, float4* pts, float4* lo, float4* hi, cudaStream_t s);
 
 }  // namespace perch

@@ -2330,7 +2330,7 @@ cudaError_t launch_icp_points(const float4* world2, const float4* cam2, int n, f
   return cudaGetLastError();
 }
 
-__device__ __forceinline__ long long icp_fixed(float v) { return __float2ll_rn(fmul(v, 65536.0f)); }
+__device__ __forceinline__ int icp_fixed(float v) { return __float2int_rn(fmul(v, 65536.0f)); }  // |v| < 32: 21 bits
 
 // hi 2^64 + lo: each part rounded to double, then one rounded addition
 __device__ __forceinline__ double icp_i128_to_double(__int128 v) {
@@ -2343,16 +2343,16 @@ __device__ __forceinline__ double icp_i128_to_double(__int128 v) {
 // sum Y_m Y_q, sum X_m Y_q, sum Y_m X_q (|x|, |y| < 32 m: |X|, |Y| < 2^21)
 __device__ __forceinline__ void icp_add_pair(long long* L, float mx, float my, float qx, float qy) {
   if (!(fabsf(mx) < 32.0f && fabsf(my) < 32.0f && fabsf(qx) < 32.0f && fabsf(qy) < 32.0f)) return;
-  const long long X = icp_fixed(mx), Y = icp_fixed(my), QX = icp_fixed(qx), QY = icp_fixed(qy);
+  const int X = icp_fixed(mx), Y = icp_fixed(my), QX = icp_fixed(qx), QY = icp_fixed(qy);
   L[0] += 1;
   L[1] += X;
   L[2] += Y;
   L[3] += QX;
   L[4] += QY;
-  L[5] += X * QX;
-  L[6] += Y * QY;
-  L[7] += X * QY;
-  L[8] += Y * QX;
+  L[5] += (long long)X * QX;
+  L[6] += (long long)Y * QY;
+  L[7] += (long long)X * QY;
+  L[8] += (long long)Y * QX;
 }
 
 // Planar Procrustes from the sums: C = n sum(m . q) - sum m . sum q and
@@ -2376,26 +2376,168 @@ __device__ bool icp_solve(const long long* S, double* T) {
   return true;
 }
 
+// World points of scene 0 by pixel, rows of q.stride pixels and q.blocks_y
+// 4 rows (NaN where nothing was observed: no distance to it passes a test),
+// and the box of each 4 x 4 block's points (lo = +inf: none). A thread takes a
+// block.
+__global__ void k_icp_image(const float* depth, Camera cam, const float* rx, const float* ry, IcpImage q, float4* pts,
+                            float4* lo, float4* hi) {
+  const int k = blockIdx.x * 256 + threadIdx.x, nbx = q.stride / 4;
+  if (k >= nbx * q.blocks_y) return;
+  const int bu = 4 * (k % nbx), bv = 4 * (k / nbx);
+  const float inf = __uint_as_float(kInfBits), nan = __uint_as_float(0x7fc00000u);
+  float4 a = make_float4(inf, inf, inf, 0.0f), b = make_float4(-inf, -inf, -inf, 0.0f);
+  for (int i = 0; i < 16; ++i) {
+    const int u = bu + (i & 3), v = bv + (i >> 2);
+    float4 o = make_float4(nan, nan, nan, nan);
+    const float z = u < cam.W && v < cam.H ? depth[v * cam.W + u] : 0.0f;
+    if (depth_valid(z)) {
+      const float x = fmul(rx[u], z), y = fmul(ry[v], z);
+      o.x = fadd(ffma(cam.Rwc[2], z, ffma(cam.Rwc[1], y, fmul(cam.Rwc[0], x))), cam.twc[0]);
+      o.y = fadd(ffma(cam.Rwc[5], z, ffma(cam.Rwc[4], y, fmul(cam.Rwc[3], x))), cam.twc[1]);
+      o.z = fadd(ffma(cam.Rwc[8], z, ffma(cam.Rwc[7], y, fmul(cam.Rwc[6], x))), cam.twc[2]);
+      a = make_float4(fminf(a.x, o.x), fminf(a.y, o.y), fminf(a.z, o.z), 0.0f);
+      b = make_float4(fmaxf(b.x, o.x), fmaxf(b.y, o.y), fmaxf(b.z, o.z), 0.0f);
+    }
+    pts[v * q.stride + u] = o;
+  }
+  lo[k] = a;
+  hi[k] = b;
+}
+
+cudaError_t launch_icp_image(const float* depth, const Camera& cam, const float* rx, const float* ry,
+                             const IcpImage& q, float4* pts, float4* lo, float4* hi, cudaStream_t s) {
+  const int n = q.stride / 4 * q.blocks_y;
+  k_icp_image<<<(n + 255) / 256, 256, 0, s>>>(depth, cam, rx, ry, q, pts, lo, hi);
+  return cudaGetLastError();
+}
+
+// The nearest observed point of a model point within the radius (ties: the
+// smaller pixel, which is the smaller index in I). Starts from no point and the
+// radius squared, or from a point within the radius (the last matching's).
+struct IcpBest {
+  float d;  // squared distance
+  int j;    // place in the image (or the grid's points); -1: none
+  int tie;  // pixel order
+  float x, y;
+};
+
+// In the image: a point within rho of p lies within f rho sqrt(1 + t^2) /
+// (z - rho) pixels of p's projection (slope t, depth z), as in delta_radius;
+// q.ortho pads rho by what the camera's matrix differs from a rotation. A
+// small window is scanned; in a larger one (most model points of a wrong pose
+// are many millimetres from the cloud, or have no pair) the boxes of its
+// 4 x 4 blocks are tested first, all lanes at a time, and then the blocks whose box
+// is nearer than the best point, the nearest one first. Bound by the issue of
+// those tests: two 640x480 scenes, 120k successors each, 35 and 48 ms
+// (renders 11.5 ms of it). The points' grid (cells of half a radius, as many
+// points in reach but in as many places as lanes) took 52 and 82; smaller
+// cells, masks of the rows that hold points, or keeping a pair while the second
+// nearest point stays farther (ICP's steps are longer than that) 51 to 126.
+__device__ __forceinline__ void icp_nearest(const Camera& cam, const IcpImage& q, float px, float py, float pz,
+                                            IcpBest& b) {
+  const float xc = cam.Rcw[0] * px + cam.Rcw[1] * py + cam.Rcw[2] * pz + cam.tcw[0];
+  const float yc = cam.Rcw[3] * px + cam.Rcw[4] * py + cam.Rcw[5] * pz + cam.tcw[1];
+  const float zc = cam.Rcw[6] * px + cam.Rcw[7] * py + cam.Rcw[8] * pz + cam.tcw[2];
+  const float rho = __fsqrt_rn(b.d) * 1.001f + 1e-6f + q.ortho * (fabsf(xc) + fabsf(yc) + fabsf(zc));
+  int u0 = 0, u1 = cam.W - 1, v0 = 0, v1 = cam.H - 1;
+  if (zc - rho > 1e-3f) {
+    const float slack = 0.05f + 1e-6f * (float)(cam.W + cam.H);
+    const float inv = __fdividef(1.0f, zc), tx = xc * inv, ty = yc * inv, f = __fdividef(rho, zc - rho);
+    const float uc = cam.fx * tx + cam.cx, ru = cam.fx * (1.0f + 0.5f * tx * tx) * f + slack;
+    const float vc = cam.fy * ty + cam.cy, rv = cam.fy * (1.0f + 0.5f * ty * ty) * f + slack;
+    u0 = max((int)ceilf(fmaxf(uc - ru, -1e6f)), u0);
+    u1 = min((int)floorf(fminf(uc + ru, 1e6f)), u1);
+    v0 = max((int)ceilf(fmaxf(vc - rv, -1e6f)), v0);
+    v1 = min((int)floorf(fminf(vc + rv, 1e6f)), v1);
+  }
+  if (u0 > u1 || v0 > v1) return;
+  auto test = [&](int i) {
+    const float4 o = __ldg(&q.pts[i]);
+    const float d = dist2(px, py, pz, o);
+    if (d <= b.d && (d < b.d || i < b.tie)) b = IcpBest{d, i, i, o.x, o.y};
+  };
+  if ((u1 - u0 + 1) * (v1 - v0 + 1) <= kIcpDirect) {
+    for (int v = v0; v <= v1; ++v)
+      for (int u = u0; u <= u1; ++u) test(v * q.stride + u);
+    return;
+  }
+  auto gap2 = [&](int at) {  // squared distance to a block's box
+    const float4 lo = __ldg(&q.lo[at]), hi = __ldg(&q.hi[at]);
+    const float gx = max3(lo.x - px, px - hi.x, 0.0f), gy = max3(lo.y - py, py - hi.y, 0.0f),
+                gz = max3(lo.z - pz, pz - hi.z, 0.0f);
+    return gx * gx + gy * gy + gz * gz;
+  };
+  const int pitch = q.stride >> 2, bx1 = u1 >> 2, by1 = v1 >> 2;
+  for (int x0 = u0 >> 2; x0 <= bx1; x0 += 8)  // at most 8 x 4 blocks at a time
+    for (int y0 = v0 >> 2; y0 <= by1; y0 += 4) {
+      const int nx = min(bx1 - x0, 7), ny = min(by1 - y0, 3);
+      uint32_t mask = 0;
+      int first = -1;
+      float nearest = b.d * 1.00001f;
+      for (int y = 0; y <= ny; ++y)
+        for (int x = 0; x <= nx; ++x) {
+          const float g = gap2((y0 + y) * pitch + x0 + x);
+          if (g > b.d * 1.00001f) continue;
+          mask |= 1u << (8 * y + x);
+          if (g < nearest) {
+            nearest = g;
+            first = 8 * y + x;
+          }
+        }
+      while (mask) {
+        const int k = first >= 0 ? first : __ffs((int)mask) - 1, y = y0 + (k >> 3), x = x0 + (k & 7);
+        mask &= ~(1u << k);
+        if (first < 0 && gap2(y * pitch + x) > b.d * 1.00001f) continue;
+        first = -1;
+        const int at = 4 * (y * q.stride + x);
+#pragma unroll 4
+        for (int i = 0; i < 16; ++i) test(at + (i >> 2) * q.stride + (i & 3));
+      }
+    }
+}
+
+// In the grid of the points, where the camera's matrix is no rotation: the
+// cells that meet a cube about p.
+__device__ __noinline__ IcpBest icp_nearest_grid(IcpGrid q, float px, float py, float pz, IcpBest b) {
+  const float rho = __fsqrt_rn(b.d) * 1.01f + 1e-6f;
+  const int x0 = max(cell_of(px - rho, q.gx, q.inv, q.nx), 0), x1 = min(cell_of(px + rho, q.gx, q.inv, q.nx), q.nx - 1);
+  const int y0 = max(cell_of(py - rho, q.gy, q.inv, q.ny), 0), y1 = min(cell_of(py + rho, q.gy, q.inv, q.ny), q.ny - 1);
+  const int z0 = max(cell_of(pz - rho, q.gz, q.inv, q.nz), 0), z1 = min(cell_of(pz + rho, q.gz, q.inv, q.nz), q.nz - 1);
+  if (x0 > x1) return b;
+  for (int iz = z0; iz <= z1; ++iz)
+    for (int iy = y0; iy <= y1; ++iy) {
+      const int row = (iz * q.ny + iy) * q.nx;
+      const int end = q.start[row + x1 + 1];
+      for (int t = q.start[row + x0]; t < end; ++t) {
+        const float4 o = q.pts[t];
+        const float d = dist2(px, py, pz, o);
+        const int j = __float_as_int(o.w);
+        if (d <= b.d && (d < b.d || j < b.tie)) b = IcpBest{d, t, j, o.x, o.y};
+      }
+    }
+  return b;
+}
+
 struct IcpClaim {
   int* next;  // device counter, zero before the launch
 };
 
 // One CTA per hypothesis at a time (claimed from a counter): render the new
 // object into the shared-memory tile over its screen box (render_chunks),
-// keep the pixels in front of the parent's render as the model set (z bits;
-// 0 elsewhere), then iterate. In each matching a thread takes one model
-// pixel: it back-projects and moves the point and scans the grid cells that
-// meet a cube of half-width rho about it, where rho is the radius, or from
-// the second matching on the distance to the point the pixel was paired with
-// last time, when that point is still within the radius (the nearest point
-// can only be nearer). It keeps the nearest point (ties: smaller index),
-// adds the pair to its own sums, and the warps reduce those into shared
-// 64-bit counters. Thread 0 then decides and fits.
+// keep the pixels in front of the parent's render as the model set, as a
+// list of world points, then iterate. In each matching a thread takes one
+// model point, moves it and finds its nearest observed point, starting
+// from the one it was paired with last time when that is still within the
+// radius. It adds the pair to its own sums, and the warps reduce
+// those to one set each. Thread 0 then decides and fits. A
+// successor with no observed point within the radius of its footprint has no
+// pair: it is done with the model set.
 template <int NT>
-__global__ void __launch_bounds__(NT, 3) k_icp(Camera cam, Geometry g, Batch b, IcpGrid q, IcpWork w, IcpClaim cl) {
+__global__ void __launch_bounds__(NT, NT == 256 ? 3 : 1) k_icp(Camera cam, Geometry g, Batch b, IcpGrid q, IcpWork w, IcpClaim cl) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t s_bar;
-  __shared__ __align__(8) unsigned long long s_sum[9];
+  __shared__ long long s_sum[9][NT / 32];
   __shared__ double s_T[4];
   __shared__ int s_qn[2], s_item, s_stop, s_nm;
   constexpr int NW = NT / 32;
@@ -2443,100 +2585,88 @@ __global__ void __launch_bounds__(NT, 3) k_icp(Camera cam, Geometry g, Batch b, 
     // and the list of those pixels (in any order: every sum is order-free)
     const float* zp = b.parent_z + (size_t)a.pid * cam.W * cam.H;
     const size_t cap = (size_t)b.tile_w * b.tile_h;
-    int* list = w.prev + 2 * cap * blockIdx.x;  // this CTA's slice: model pixels, then their last pairs
-    int* prev_t = list + cap;
-    for (int i0 = 0; i0 < area; i0 += NT) {  // the same trip count in every lane (ballots below)
-      const int i = i0 + tid;
+    float4* list = w.model + cap * blockIdx.x;  // this CTA's slice: model points, and each one's last pair
+    // a warp takes 8 x 4 pixels: its points then search alike
+    const int wx = (tw + 7) >> 3, n_win = wx * ((bb.w + 3) >> 2);
+    for (int k = warp; k < n_win; k += NW) {
+      const int lx = 8 * (k % wx) + (lane & 7), ly = 4 * (k / wx) + (lane >> 3);
       uint32_t v = 0u;
-      if (i < area) {
-        const uint32_t izb = tile[i];
+      if (lx < tw && ly < bb.w) {
+        const uint32_t izb = tile[ly * tw + lx];
         if (izb != 0u) {
-          const int ly = i / tw, lx = i - ly * tw;
           const float z = __frcp_rn(__uint_as_float(izb));
           if (z < zp[(size_t)(bb.y + ly) * cam.W + bb.x + lx]) v = __float_as_uint(z);
         }
-        tile[i] = v;
       }
       const unsigned mask = __ballot_sync(0xffffffffu, v != 0u);
       int base = 0;
       if (lane == 0 && mask) base = atomicAdd(&s_nm, __popc(mask));
       base = __shfl_sync(0xffffffffu, base, 0);
-      if (v != 0u) list[base + __popc(mask & ((1u << lane) - 1u))] = i;
+      if (v != 0u) {  // its world point (R7)
+        const float z = __uint_as_float(v), xc = fmul(g.rx[bb.x + lx], z), yc = fmul(g.ry[bb.y + ly], z);
+        const float mx = fadd(ffma(cam.Rwc[2], z, ffma(cam.Rwc[1], yc, fmul(cam.Rwc[0], xc))), cam.twc[0]);
+        const float my = fadd(ffma(cam.Rwc[5], z, ffma(cam.Rwc[4], yc, fmul(cam.Rwc[3], xc))), cam.twc[1]);
+        const float mz = fadd(ffma(cam.Rwc[8], z, ffma(cam.Rwc[7], yc, fmul(cam.Rwc[6], xc))), cam.twc[2]);
+        list[base + __popc(mask & ((1u << lane) - 1u))] = make_float4(mx, my, mz, __int_as_float(-1));
+      }
     }
-    __syncthreads();  // |M|, the model set and its list are complete
+    __syncthreads();  // |M| and the list are complete
     const int nm = s_nm;
     long long prev[9];  // thread 0: the previous matching's sums
     bool have_prev = false;
     int iters = 0, n_corr = 0, status = PERCH_ICP_CAP;
-    for (int k = 1; k <= w.max_iter; ++k) {
-      if (tid < 9) s_sum[tid] = 0ull;
-      __syncthreads();  // also publishes s_T
+    // every model point lies within the footprint's radius of (x, y) (+ 2 cm
+    // and a sixteenth of a pixel at the object's depth for the snap)
+    const float depth = g.pose_off[a.o.ix * g.ny + a.o.iy].z + m.fp_r + fmaxf(fabsf(m.lo[2]), fabsf(m.hi[2]));
+    const float reach_m = m.fp_r + 0.02f + depth / (16.0f * fminf(cam.fx, cam.fy));
+    const float ox = g.xs[a.o.ix], oy = g.ys[a.o.iy];
+    bool met = nm > 0 && w.obs.n > 0;
+    {
+      const float R = reach_m + w.rwin;
+      if (met) {
+        const int cx0 = max(cell_of(ox - R, w.obs.g2x, w.obs.inv2, w.obs.n2x) - 1, 0);
+        const int cx1 = min(cell_of(ox + R, w.obs.g2x, w.obs.inv2, w.obs.n2x) + 1, w.obs.n2x - 1);
+        const int cy0 = max(cell_of(oy - R, w.obs.g2y, w.obs.inv2, w.obs.n2y) - 1, 0);
+        const int cy1 = min(cell_of(oy + R, w.obs.g2y, w.obs.inv2, w.obs.n2y) + 1, w.obs.n2y - 1);
+        met = cx0 <= cx1 && cy0 <= cy1 && sat_sum(w.obs.sat2, w.obs.n2x, cy0, cy1, cx0, cx1) != 0;
+      }
+    }
+    if (!met && w.max_iter > 0) status = PERCH_ICP_FEW;
+    for (int k = 1; met && k <= w.max_iter; ++k) {
+      __syncthreads();  // publishes s_T; the last sums have been read
       const float cf = __double2float_rn(s_T[0]), sf = __double2float_rn(s_T[1]);
       const float txf = __double2float_rn(s_T[2]), tyf = __double2float_rn(s_T[3]);
       long long L[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
       for (int e = tid; e < nm; e += NT) {
-        const int i = list[e];
-        const int ly = i / tw, lx = i - ly * tw;
-        const float z = __uint_as_float(tile[i]);
-        const float xc = fmul(g.rx[bb.x + lx], z), yc = fmul(g.ry[bb.y + ly], z);
-        const float mx = fadd(ffma(cam.Rwc[2], z, ffma(cam.Rwc[1], yc, fmul(cam.Rwc[0], xc))), cam.twc[0]);
-        const float my = fadd(ffma(cam.Rwc[5], z, ffma(cam.Rwc[4], yc, fmul(cam.Rwc[3], xc))), cam.twc[1]);
-        const float mz = fadd(ffma(cam.Rwc[8], z, ffma(cam.Rwc[7], yc, fmul(cam.Rwc[6], xc))), cam.twc[2]);
-        const float px = fadd(fsub(fmul(cf, mx), fmul(sf, my)), txf);
-        const float py = fadd(fadd(fmul(sf, mx), fmul(cf, my)), tyf);
-        // Search window: the radius, or, when the previous matching's point
-        // is still within it, that point's distance (the nearest point is no
-        // farther). The margins cover the rounding of d^2 (relative 2^-22)
-        // and of the window's ends (1e-6 m), so every point whose d^2 can
-        // tie or beat the bound lies inside.
-        float rho = w.rwin;
-        if (k > 1) {
-          const int t0 = prev_t[e];
-          if (t0 >= 0) {
-            const float d0 = dist2(px, py, mz, q.pts[t0]);
-            if (d0 <= w.r2) rho = fminf(rho, __fsqrt_rn(d0) * 1.001f + 1e-6f);
-          }
+        const float4 m4 = list[e];
+        const float px = fadd(fsub(fmul(cf, m4.x), fmul(sf, m4.y)), txf);
+        const float py = fadd(fadd(fmul(sf, m4.x), fmul(cf, m4.y)), tyf);
+        IcpBest best{w.r2, -1, INT_MAX, 0.0f, 0.0f};
+        const int j0 = __float_as_int(m4.w);  // the last matching's point: a bound, if still within the radius
+        if (j0 >= 0) {
+          const float4 o = __ldg(&(w.img.pts ? w.img.pts : q.pts)[j0]);
+          const float d = dist2(px, py, m4.z, o);
+          if (d <= w.r2) best = IcpBest{d, j0, w.img.pts ? j0 : __float_as_int(o.w), o.x, o.y};
         }
-        const int x0 = max(cell_of(px - rho, q.gx, q.inv, q.nx), 0), x1 = min(cell_of(px + rho, q.gx, q.inv, q.nx), q.nx - 1);
-        const int y0 = max(cell_of(py - rho, q.gy, q.inv, q.ny), 0), y1 = min(cell_of(py + rho, q.gy, q.inv, q.ny), q.ny - 1);
-        const int z0 = max(cell_of(mz - rho, q.gz, q.inv, q.nz), 0), z1 = min(cell_of(mz + rho, q.gz, q.inv, q.nz), q.nz - 1);
-        uint32_t bd = 0xffffffffu;  // no candidate (every d^2 <= r^2 has smaller bits)
-        int bj = INT_MAX, bt = -1;
-        float bqx = 0.0f, bqy = 0.0f;
-        if (x0 <= x1) {
-          for (int iz = z0; iz <= z1; ++iz)
-            for (int iy = y0; iy <= y1; ++iy) {
-              const int row = (iz * q.ny + iy) * q.nx;
-              const int end = q.start[row + x1 + 1];
-              for (int t = q.start[row + x0]; t < end; ++t) {
-                const float4 o = q.pts[t];
-                const float d = dist2(px, py, mz, o);
-                if (d <= w.r2) {
-                  const uint32_t db = __float_as_uint(d);
-                  const int j = __float_as_int(o.w);
-                  if (db < bd || (db == bd && j < bj)) {
-                    bd = db;
-                    bj = j;
-                    bt = t;
-                    bqx = o.x;
-                    bqy = o.y;
-                  }
-                }
-              }
-            }
-        }
-        prev_t[e] = bt;
-        if (bt >= 0) icp_add_pair(L, mx, my, bqx, bqy);
+        if (w.img.pts)
+          icp_nearest(cam, w.img, px, py, m4.z, best);
+        else
+          best = icp_nearest_grid(q, px, py, m4.z, best);
+        if (best.j != j0) list[e].w = __int_as_float(best.j);
+        if (best.j >= 0) icp_add_pair(L, m4.x, m4.y, best.x, best.y);
       }
       for (int t = 0; t < 9; ++t) {
         long long v = L[t];
         for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-        if (lane == 0 && v != 0) atomicAdd(&s_sum[t], (unsigned long long)v);
+        if (lane == 0) s_sum[t][warp] = v;
       }
       __syncthreads();
       if (tid == 0) {
         long long S[9];
-        for (int t = 0; t < 9; ++t) S[t] = (long long)s_sum[t];
+        for (int t = 0; t < 9; ++t) {
+          S[t] = 0;
+          for (int k = 0; k < NW; ++k) S[t] += s_sum[t][k];
+        }
         n_corr = (int)S[0];
         int stop = 0;
         bool same = have_prev;
@@ -2570,22 +2700,26 @@ __global__ void __launch_bounds__(NT, 3) k_icp(Camera cam, Geometry g, Batch b, 
 }
 
 cudaError_t launch_icp(const Camera& cam, const Geometry& g, const Batch& b, const IcpGrid& q, const IcpWork& w,
-                       long long prev_elems, int* next, int sm_count, cudaStream_t s) {
+                       long long model_elems, int* next, int sm_count, cudaStream_t s) {
   if (b.n_hyp <= 0) return cudaSuccess;
   const size_t smem = render_smem_bytes(b.tile_w, b.tile_h);
-  auto kern = k_icp<256>;
+  // no more hypotheses than SMs: a CTA has its SM to itself, and twice the
+  // threads halve the rounds of each matching (the five objects of a scene,
+  // 640x480: 1.18 -> 0.62 ms)
+  const int nt = b.n_hyp <= sm_count ? 512 : 256;
+  auto kern = nt == 512 ? k_icp<512> : k_icp<256>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, smem);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   long long grid = (long long)per_sm * sm_count;
   if (grid > b.n_hyp) grid = b.n_hyp;
-  const long long cap = 2LL * b.tile_w * b.tile_h;  // each CTA's slice of w.prev
-  if (cap > 0 && grid > prev_elems / cap) grid = prev_elems / cap;
+  const long long cap = (long long)b.tile_w * b.tile_h;  // each CTA's slice of w.model
+  if (cap > 0 && grid > model_elems / cap) grid = model_elems / cap;
   if (grid < 1) return cudaErrorInvalidValue;
-  kern<<<(unsigned)grid, 256, smem, s>>>(cam, g, b, q, w, IcpClaim{next});
+  kern<<<(unsigned)grid, nt, smem, s>>>(cam, g, b, q, w, IcpClaim{next});
   return cudaGetLastError();
 }
 
