@@ -10,16 +10,19 @@
 //   -> flatten (h, w, c) ++ one-hot -> FC 96 (ReLU) -> FC 1; loss 0.5 (pred - y)^2
 //
 // Data layout: activations NHWC bfloat16. Every convolution is one GEMM over
-// rows = output pixels (N x Ho x Wo) and columns = (tap, channel) (K = 9 Cin,
-// padded to 32): the 2-channel input layer through an explicit im2col, the
-// others by gathering 16-byte chunks of the NHWC input straight into shared
-// memory (implicit im2col, zero padding through the copy's source size). The
-// GEMM is mma.sync m16n8k16 (BF16 in, FP32 accumulate) fed by a 3-stage
-// cp.async pipeline and ldmatrix (.trans for MN-contiguous operands). Weight
-// gradients reduce over pixels with both operands read in place, split along
-// the reduction and summed in a fixed order (deterministic). Gradients between
-// layers are rounded to bfloat16, like the activations; weights keep an FP32
-// master copy updated by Adam and re-rounded to bfloat16 after each step.
+// rows = output pixels (N x Ho x Wo) and columns = (tap, channel): the 2-channel
+// input layer directly from a strip of the crop (k_conv1, mma.sync), the others
+// and their data gradients on tcgen05 with operands loaded by TMA
+// (k_conv_tma). Weight gradients and the FC layers use k_gemm: mma.sync
+// m16n8k16 (BF16 in, FP32 accumulate) fed by a 3-stage cp.async pipeline and
+// ldmatrix (.trans for MN-contiguous operands); the weight gradients gather
+// 16-byte chunks of the NHWC input straight into shared memory (implicit
+// im2col, zero padding through the copy's source size; the input layer's from
+// an explicit im2col), split along the pixel reduction and summed in a fixed
+// order (deterministic). Gradients between layers are rounded to bfloat16,
+// like the activations; weights keep an FP32 master copy updated by Adam and
+// re-rounded to bfloat16 after each step.
+#include <cuda.h>
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -53,7 +56,6 @@ int kp_of(int l) { return round32(9 * kCin[l]); }
 
 // ---------------------------------------------------------------- GEMM
 constexpr int BM = 128, BK = 32, LDS = BK + 8, STAGES = 3;
-enum { EPI_BIAS_RELU = 0, EPI_F32 = 1, EPI_BF16 = 2, EPI_DGRAD = 3 };
 
 struct GemmArgs {
   const bf16* A;  // [M][lda], K-contiguous
@@ -61,25 +63,12 @@ struct GemmArgs {
   const bf16* B;  // [N][ldb], K-contiguous
   long long ldb;
   int M, N, K, Ksplit;  // split z covers columns [z Ksplit, min(K, (z + 1) Ksplit))
-  float* Cf;            // EPI_F32 output (partial z at Cf + z split_stride)
-  bf16* Cb;             // EPI_BIAS_RELU output
-  long long ldc;
-  int grp;              // output row m lives at (m / grp) ldg + (m % grp) ldc
-  long long ldg;
-  long long split_stride;
-  const float* bias;
-  // implicit im2col (CONV = 1: A, CONV = 2: B): the operand is the NHWC
-  // input of a 3x3 pad-1 convolution with power-of-two channels and output
-  // side; pixel index (n, i, j) and column index (tap, c), tap = 3 kh + kw
+  float* Cf;  // output (partial z at Cf + z split_stride)
+  long long ldc, split_stride;
+  // implicit im2col (CONV): B is the NHWC input of a 3x3 pad-1 convolution with
+  // power-of-two channels and output side; pixel index (n, i, j) and column
+  // index (tap, c), tap = 3 kh + kw
   int cH, cs, lg_c, lg_wo;
-  // fused data gradient of a stride-2 convolution (CONV = 3, EPI_DGRAD), one
-  // parity class (par_h, par_w) of the input pixels: rows = the class's
-  // pixels (n, a, b) at (2a + par_h, 2b + par_w); columns = input channels;
-  // K = (tap of the class, output channel). A gathers dz, B reads W in place,
-  // the epilogue applies the ReLU mask of the layer input and scatters rows
-  // back to NHWC.
-  int par_h, par_w, ntw, dg_lg_ho, dg_lg_co, dg_H, dg_cin, dg_kp;
-  const bf16* mask;
 };
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -138,30 +127,7 @@ __device__ __forceinline__ void dg_tap(int par, int t, int& kofs, int& d) {
   d = (par == 1 && t == 0) ? 1 : 0;
 }
 
-// A chunk of the fused data gradient: class pixel m, columns k .. k + 7 (one
-// tap, 8 output channels) of dz; nullptr where that output pixel is outside.
-__device__ __forceinline__ const bf16* dgrad_a_src(const GemmArgs& p, int m, int k) {
-  const int t = k >> p.dg_lg_co, o = k & ((1 << p.dg_lg_co) - 1);
-  int kh, dh, kw, dw;
-  dg_tap(p.par_h, t / p.ntw, kh, dh);
-  dg_tap(p.par_w, t % p.ntw, kw, dw);
-  const int ho = 1 << p.dg_lg_ho;
-  const int b = m & (ho - 1), a = (m >> p.dg_lg_ho) & (ho - 1), n = m >> (2 * p.dg_lg_ho);
-  const int i = a + dh, j = b + dw;
-  if (i >= ho || j >= ho) return nullptr;
-  return p.A + ((((long long)n * ho + i) * ho + j) << p.dg_lg_co) + o;
-}
-
-// B chunk: K row (tap, o), input channels n .. n + 7 of W[o][kh][kw][.]
-__device__ __forceinline__ const bf16* dgrad_b_src(const GemmArgs& p, int k, int n) {
-  const int t = k >> p.dg_lg_co, o = k & ((1 << p.dg_lg_co) - 1);
-  int kh, dh, kw, dw;
-  dg_tap(p.par_h, t / p.ntw, kh, dh);
-  dg_tap(p.par_w, t % p.ntw, kw, dw);
-  return p.B + (long long)o * p.dg_kp + (kh * 3 + kw) * p.dg_cin + n;
-}
-
-template <int BN, int EPI, bool AK, bool BKC, int CONV>
+template <int BN, bool AK, bool BKC, bool CONV>
 __global__ void __launch_bounds__(256) k_gemm(GemmArgs p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int A_LD = AK ? LDS : BM + 8, A_STAGE = AK ? BM * LDS : BK * (BM + 8);
@@ -190,16 +156,8 @@ __global__ void __launch_bounds__(256) k_gemm(GemmArgs p) {
     if (AK) {
       for (int c = tid; c < BM * 4; c += 256) {
         const int r = c >> 2, q = c & 3, gm = m0 + r;
-        bool ok = gm < p.M;
-        const bf16* src = p.A;
-        if (CONV == 1 || CONV == 3) {
-          const bf16* g = ok ? (CONV == 1 ? conv_src(p, p.A, gm, k0 + q * 8) : dgrad_a_src(p, gm, k0 + q * 8))
-                             : nullptr;
-          ok = g != nullptr;
-          if (ok) src = g;
-        } else if (ok) {
-          src = p.A + (long long)gm * p.lda + k0 + q * 8;
-        }
+        const bool ok = gm < p.M;
+        const bf16* src = ok ? p.A + (long long)gm * p.lda + k0 + q * 8 : p.A;
         cp_async16(smem_addr(as + r * A_LD + q * 8), src, ok);
       }
     } else {
@@ -222,12 +180,10 @@ __global__ void __launch_bounds__(256) k_gemm(GemmArgs p) {
         const int r = c / (BN / 8), q = c % (BN / 8), gn = n0 + q * 8;
         bool ok = gn < p.N;
         const bf16* src = p.B;
-        if (CONV == 2) {
+        if (CONV) {
           const bf16* g = ok ? conv_src(p, p.B, k0 + r, gn) : nullptr;
           ok = g != nullptr;
           if (ok) src = g;
-        } else if (CONV == 3) {
-          if (ok) src = dgrad_b_src(p, k0 + r, gn);
         } else if (ok) {
           src = p.B + (long long)(k0 + r) * p.ldb + gn;
         }
@@ -297,86 +253,133 @@ __global__ void __launch_bounds__(256) k_gemm(GemmArgs p) {
         const int row = m0 + wm * TM + i * 16 + g + h * 8;
         const int col = n0 + wn * 32 + j * 8 + 2 * t;
         if (row >= p.M || col >= p.N) continue;
-        float v0 = acc[i][j][2 * h], v1 = acc[i][j][2 * h + 1];
-        if (EPI == EPI_DGRAD) {  // class pixel -> NHWC input pixel, times the ReLU mask
-          const int ho = 1 << p.dg_lg_ho;
-          const int b = row & (ho - 1), a = (row >> p.dg_lg_ho) & (ho - 1), n = row >> (2 * p.dg_lg_ho);
-          const long long o =
-              (((long long)n * p.dg_H + 2 * a + p.par_h) * p.dg_H + 2 * b + p.par_w) * p.dg_cin + col;
-          const __nv_bfloat162 x = *reinterpret_cast<const __nv_bfloat162*>(p.mask + o);
-          if (!(__low2float(x) > 0.0f)) v0 = 0.0f;
-          if (!(__high2float(x) > 0.0f)) v1 = 0.0f;
-          *reinterpret_cast<__nv_bfloat162*>(p.Cb + o) = __floats2bfloat162_rn(v0, v1);
-          continue;
-        }
-        const long long off = (long long)(row / p.grp) * p.ldg + (long long)(row % p.grp) * p.ldc + col;
-        if (EPI == EPI_BIAS_RELU) {
-          v0 = fmaxf(v0 + p.bias[col], 0.0f);
-          v1 = fmaxf(v1 + p.bias[col + 1], 0.0f);
-          *reinterpret_cast<__nv_bfloat162*>(p.Cb + off) = __floats2bfloat162_rn(v0, v1);
-        } else if (EPI == EPI_BF16) {
-          *reinterpret_cast<__nv_bfloat162*>(p.Cb + off) = __floats2bfloat162_rn(v0, v1);
-        } else {
-          *reinterpret_cast<float2*>(p.Cf + (long long)blockIdx.z * p.split_stride + off) = make_float2(v0, v1);
-        }
+        *reinterpret_cast<float2*>(p.Cf + (long long)blockIdx.z * p.split_stride + (long long)row * p.ldc + col) =
+            make_float2(acc[i][j][2 * h], acc[i][j][2 * h + 1]);
       }
 }
 
-template <int BN, int EPI, bool AK, bool BKC, int CONV>
+template <int BN, bool AK, bool BKC, bool CONV>
 cudaError_t gemm_bn(const GemmArgs& p, int splits, cudaStream_t s) {
   constexpr int A_STAGE = AK ? BM * LDS : BK * (BM + 8), B_STAGE = BKC ? BN * LDS : BK * (BN + 8);
   const int smem = STAGES * (A_STAGE + B_STAGE) * (int)sizeof(bf16);
   cudaError_t e =
-      cudaFuncSetAttribute(k_gemm<BN, EPI, AK, BKC, CONV>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      cudaFuncSetAttribute(k_gemm<BN, AK, BKC, CONV>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   dim3 grid((p.N + BN - 1) / BN, (p.M + BM - 1) / BM, splits);
-  k_gemm<BN, EPI, AK, BKC, CONV><<<grid, 256, smem, s>>>(p);
+  k_gemm<BN, AK, BKC, CONV><<<grid, 256, smem, s>>>(p);
   return cudaGetLastError();
 }
 
 // C = A B^T (layouts as k_gemm); `splits` CTAs along K, each writing its
-// partial at Cf + z split_stride (EPI_F32) or, with one split, the epilogue.
-template <int EPI, bool AK = true, bool BKC = true, int CONV = 0>
-cudaError_t gemm(GemmArgs p, int splits, cudaStream_t s) {
-  if (p.grp <= 0) {
-    p.grp = 1 << 30;
-    p.ldg = 0;
-  }
+// partial at Cf + z split_stride.
+template <bool AK = true, bool BKC = true, bool CONV = false>
+cudaError_t gemm(const GemmArgs& p, int splits, cudaStream_t s) {
   if ((!AK && p.M % 8) || (!BKC && p.N % 8) || p.K % 32 || p.Ksplit % 32) return cudaErrorInvalidValue;
   if (CONV && p.lg_c < 3) return cudaErrorInvalidValue;  // chunks of 8 channels within one tap
-  if (p.N <= 32) return gemm_bn<32, EPI, AK, BKC, CONV>(p, splits, s);
-  if (p.N <= 64) return gemm_bn<64, EPI, AK, BKC, CONV>(p, splits, s);
-  return gemm_bn<128, EPI, AK, BKC, CONV>(p, splits, s);
+  if (p.N <= 32) return gemm_bn<32, AK, BKC, CONV>(p, splits, s);
+  if (p.N <= 64) return gemm_bn<64, AK, BKC, CONV>(p, splits, s);
+  return gemm_bn<128, AK, BKC, CONV>(p, splits, s);
 }
 
-// ------------------------------------------------- tcgen05 convolution
-// Forward 3x3 convolution with implicit im2col (layers 2-4) on the
-// fifth-generation tensor cores: C[M x N] = A B^T, A the im2col rows of the
-// NHWC input (conv_src), B the weights [N][K]. One CTA of 256 threads owns a
-// 128-row tile and all N (64 or 128) columns; its FP32 accumulator lives in
-// tensor memory (N columns, lanes = rows). K advances BK columns per step
-// through a ring of S shared-memory stages filled by cp.async in the
-// canonical no-swizzle K-major layout: core matrices of 8 rows x 16 bytes,
-// the K-adjacent ones 128 bytes apart, the row-adjacent ones BK / 8 x 128
-// bytes apart. One thread issues the step's BK / 16 m128 nN k16 MMAs and
-// commits them to the stage's mbarrier, which frees the stage for the copy
-// of step + S. The epilogue reads the accumulator back with tcgen05.ld (warp
-// w: rows 32 (w mod 4) .. + 31, columns of half w / 4), adds the bias,
-// applies ReLU and stores bfloat16 rows (GemmArgs addressing). Every wait is
-// bounded; a wait that gives up sets *err and skips the stores, and the
-// tensor memory is freed all the same.
+// --------------------------------------- tcgen05 convolutions fed by TMA
+// The 3x3, stride-2, pad-1 convolutions of layers 2-4 and their data gradients,
+// as one persistent warp-specialised kernel on the fifth-generation tensor
+// cores. Both are sums over taps of 128-row GEMMs whose rows are consecutive
+// pixels of a regular grid, so a k-block's A operand (KC channels of one tap) is
+// one box of a 4D tensor map (channel, x, y, image), zero-filled outside the
+// image, and there is no gather:
+// - forward: the input pixels of one tap have one parity in y and in x, so
+//   each layer has four maps of its input, one per parity, with strides of
+//   two pixels (row 2i - 1 + kh is row i - [kh = 0] of parity [kh != 1]);
+// - data gradient: the input pixels of one parity class (py, px) take 1, 2, 2
+//   or 4 taps of dz at (y + dy, x + dx), dy, dx in {0, 1}; the four classes are
+//   tiles of the same launch, the longest first. Its B operand is the
+//   weights with input channels as rows (k_dgrad_weights).
+// K runs over (tap, channel) in order in steps of 16, as the mma.sync kernels
+// run it, and the results are the same bit for bit.
+//
+// One CTA per SM: thread 0 of warp 0 fills a ring of S stages (A 128 x KC and
+// B N x KC, swizzled K-major rows of 2 KC bytes), thread 0 of warp 1 issues the
+// MMAs into one of two tensor-memory accumulators, warps 4-7 read the other
+// one back (bias + ReLU, or the ReLU mask of the layer input) and store
+// bfloat16 rows. Every wait is bounded; a wait that gives up raises s_abort,
+// which ends the other roles' waits, the copies and MMAs in flight are waited
+// for, the tensor memory is freed and *err is set.
+//
+// Bound by the operand boxes through L2 and the store of the output, not by the
+// tensor pipe: N is 32 to 128, so a 16 KB A box feeds 16 to 64 cycles of MMA.
+// 256 crops, before (cp.async gathers of the same GEMMs, mma.sync) and now:
+// conv2 64 -> 48 us, conv3 and conv4 52 -> 18 each (mean), the twelve class
+// launches of the data gradients 341 -> 78 + 39 + 22.
 constexpr int kTcRows = 128, kTcThreads = 256;
 
-template <int BK>
-__device__ __forceinline__ uint32_t tc_canon(int r, int kc) {  // (row r, 16-byte chunk kc) in a stage
-  return (uint32_t)((r >> 3) * (BK / 8) * 128 + kc * 128 + (r & 7) * 16);
+struct ConvMaps {
+  CUtensorMap a[4];  // forward: the input's parities 2 py + px; data gradient: a[0] = dz
+  CUtensorMap b;     // weights
+};
+
+struct ConvArgs {
+  int M, tiles;          // rows of one tile row space, 128-row tiles of it (per class in the data gradient)
+  int lg_wo, lg_ho;      // the row space: images of Ho x Wo pixels
+  int lg_c;              // log2 channels per tap of A
+  int k_blocks;          // forward: k-blocks of a tile
+  const float* bias;     // forward
+  bf16* out;
+  long long ldc, ldg;    // forward: row m at (m / grp) ldg + (m % grp) ldc
+  int grp;
+  const bf16* mask;      // data gradient: the layer input (ReLU mask), NHWC with N channels, side H
+  int H;
+};
+
+__device__ __forceinline__ void tc_mbar_init(uint64_t* bar, int count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
 }
-// shared-memory matrix descriptor: start address, leading (K) byte offset
-// 128, stride (row-group) byte offset, descriptor version 1, no swizzle
-template <int BK>
+__device__ __forceinline__ uint64_t tc_now() {
+  uint64_t t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+__device__ __forceinline__ bool tc_try(uint64_t* bar, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(done)
+      : "r"(smem_addr(bar)), "r"(parity)
+      : "memory");
+  return done != 0;
+}
+// wait for the phase of the given parity: bounded by polls and by 2 s, and
+// ended by `stop` (nullptr: not)
+__device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity, volatile int* stop) {
+  if (tc_try(bar, parity)) return true;
+  const uint64_t t0 = tc_now();
+  for (int i = 0; i < (1 << 22); ++i) {
+    if (tc_try(bar, parity)) return true;
+    if ((i & 63) == 63 && ((stop && *stop) || tc_now() - t0 > 2000000000ull)) break;
+  }
+  if (stop) *stop = 1;
+  return false;
+}
+__device__ __forceinline__ void tc_load4(void* dst, const CUtensorMap* map, int c, int x, int y, int n, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
+      ::"r"(smem_addr(dst)), "l"(map), "r"(c), "r"(x), "r"(y), "r"(n), "r"(smem_addr(bar))
+      : "memory");
+}
+__device__ __forceinline__ void tc_load2(void* dst, const CUtensorMap* map, int k, int row, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
+          smem_addr(dst)),
+      "l"(map), "r"(k), "r"(row), "r"(smem_addr(bar))
+      : "memory");
+}
+// shared-memory matrix descriptor of a K-major operand with rows of 2 KC bytes
+// in the 128-byte (KC = 64) or 64-byte (KC = 32) swizzle: start address, stride
+// between groups of eight rows, descriptor version 1, swizzle mode
+template <int KC>
 __device__ __forceinline__ uint64_t tc_desc(uint32_t saddr) {
-  return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)(128 >> 4) << 16) |
-         ((uint64_t)((BK / 8) * 128 >> 4) << 32) | (1ull << 46);
+  return (uint64_t)((saddr >> 4) & 0x3FFFu) | (1ull << 16) | ((uint64_t)(8 * 2 * KC >> 4) << 32) | (1ull << 46) |
+         ((uint64_t)(KC == 64 ? 2 : 4) << 61);
 }
 // instruction descriptor of kind::f16: FP32 accumulator, BF16 A and B, both
 // K-major, M = 128, N
@@ -384,48 +387,35 @@ template <int N>
 __device__ __forceinline__ uint32_t tc_idesc() {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kTcRows >> 4) << 24);
 }
-__device__ __forceinline__ void tc_mbar_init(uint64_t* bar) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bar)) : "memory");
-}
-__device__ __forceinline__ uint64_t tc_now() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-// wait for the phase of the given parity: bounded by polls and by 2 s
-__device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity) {
-  const uint64_t t0 = tc_now();
-  for (int i = 0; i < (1 << 22); ++i) {
-    uint32_t done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(smem_addr(bar)), "r"(parity)
-        : "memory");
-    if (done) return true;
-    if ((i & 255) == 255 && tc_now() - t0 > 2000000000ull) break;
-  }
-  return false;
-}
 
-template <int N, int BK, int S>
-__global__ void __launch_bounds__(kTcThreads) k_conv_tc(GemmArgs p, int* err) {
-  static_assert(N == 64 || N == 128, "N must be 64 or 128");
-  static_assert(BK % 16 == 0, "BK must be a multiple of 16");
-  constexpr int CH = BK / 8, A_BYTES = kTcRows * BK * 2, STAGE = A_BYTES + N * BK * 2;
+template <int KC, int N, bool DGRAD>
+__global__ void __launch_bounds__(kTcThreads, 1) k_conv_tma(const __grid_constant__ ConvMaps maps, ConvArgs p,
+                                                            int stages, int* err) {
+  static_assert((KC == 32 || KC == 64) && (N == 32 || N == 64 || N == 128), "operand shapes");
+  constexpr int A_BYTES = kTcRows * KC * 2, B_BYTES = N * KC * 2, STAGE = A_BYTES + B_BYTES, kMaxStages = 16;
   extern __shared__ __align__(1024) unsigned char smem[];
-  __shared__ __align__(8) uint64_t bar[S];
+  __shared__ __align__(8) uint64_t full[kMaxStages], empty[kMaxStages], acc_full[2], acc_empty[2], drain;
   __shared__ uint32_t s_tmem;
+  __shared__ int s_abort;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int m0 = blockIdx.x * kTcRows, nk = p.K / BK;
-  const uint32_t sbase = smem_addr(smem);
+  const uint32_t sbase = (smem_addr(smem) + 1023u) & ~1023u;  // the swizzle's period
+  unsigned char* const sgen = smem + (sbase - smem_addr(smem));
   if (tid == 0) {
-    for (int s = 0; s < S; ++s) tc_mbar_init(&bar[s]);
+    for (int s = 0; s < stages; ++s) {
+      tc_mbar_init(&full[s], 1);
+      tc_mbar_init(&empty[s], 1);
+    }
+    for (int k = 0; k < 2; ++k) {
+      tc_mbar_init(&acc_full[k], 1);
+      tc_mbar_init(&acc_empty[k], 4);
+    }
+    tc_mbar_init(&drain, 1);
+    s_abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 0) {  // N columns of tensor memory for the accumulator
+  if (warp == 1) {  // two accumulators of N columns
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&s_tmem)),
-                 "r"(N)
+                 "r"(2 * N)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -433,117 +423,222 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_tc(GemmArgs p, int* err) {
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = s_tmem;
-
-  auto load = [&](int ks) {  // this thread's share of step ks's A and B chunks
-    const uint32_t a = sbase + (uint32_t)((ks % S) * STAGE), b = a + A_BYTES;
-    const int k0 = ks * BK;
-    for (int i = tid; i < kTcRows * CH; i += kTcThreads) {
-      const int r = i / CH, kc = i % CH, m = m0 + r;
-      const bf16* src = m < p.M ? conv_src(p, p.A, m, k0 + 8 * kc) : nullptr;
-      cp_async16(a + tc_canon<BK>(r, kc), src ? src : p.A, src != nullptr);
-    }
-    for (int i = tid; i < N * CH; i += kTcThreads) {
-      const int n = i / CH, kc = i % CH;
-      cp_async16(b + tc_canon<BK>(n, kc), p.B + (long long)n * p.ldb + k0 + 8 * kc, true);
-    }
+  volatile int* stop = &s_abort;
+  const int all = DGRAD ? 4 * p.tiles : p.tiles;
+  // a tile's class (data gradient: 3, 2, 1, 0 in order of the taps they take) and its k-blocks
+  auto cls = [&](int t) { return DGRAD ? 3 - t / p.tiles : 0; };
+  auto blocks = [&](int c) {
+    return DGRAD ? (((c >> 1) + 1) * ((c & 1) + 1) << p.lg_c) / KC : p.k_blocks;
   };
 
-  for (int ks = 0; ks < S - 1; ++ks) {
-    if (ks < nk) load(ks);
-    cp_commit();
-  }
-  bool ok = true;
-  int last = -1;  // last step whose MMAs were issued (the same in every thread)
-  for (int ks = 0; ks < nk; ++ks) {
-    const int kl = ks + S - 1;  // the step loaded now, into the stage step ks - 1 used
-    if (kl < nk) {
-      if (kl >= S) ok = ok && tc_wait(&bar[kl % S], (uint32_t)(((kl - S) / S) & 1));
-      if (ok) load(kl);
-    }
-    cp_commit();
-    cp_wait<S - 1>();  // this thread's copies of step ks have landed
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // visible to the tensor cores
-    ok = __syncthreads_and(ok);
-    if (ok) last = ks;
-    if (ok && tid == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t a = sbase + (uint32_t)((ks % S) * STAGE), b = a + A_BYTES;
-      for (int j = 0; j < BK / 16; ++j) {
-        const uint64_t ad = tc_desc<BK>(a + 256 * j), bd = tc_desc<BK>(b + 256 * j);
-        const uint32_t acc = (ks | j) != 0;
-        asm volatile(
-            "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-            " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-            "l"(ad), "l"(bd), "r"(tc_idesc<N>()), "r"(acc)
-            : "memory");
-      }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                       smem_addr(&bar[ks % S]))
-                   : "memory");
-    }
-  }
-  cp_wait<0>();
-  // the last commit covers every MMA before it; wait for it (bounded) even
-  // after a failure, so that no MMA still writes the tensor memory freed below
-  if (last >= 0 && !tc_wait(&bar[last % S], (uint32_t)((last / S) & 1))) ok = false;
-  ok = __syncthreads_and(ok && last == nk - 1);
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const int q = warp & 3, half = warp >> 2;  // TMEM lanes 32q .. 32q + 31, columns of this half
-  const int row = m0 + 32 * q + lane;
-  const long long off = (long long)(row / p.grp) * p.ldg + (long long)(row % p.grp) * p.ldc;
-  if (ok) {
-    for (int c0 = half * (N / 2); c0 < (half + 1) * (N / 2); c0 += 16) {
-      uint32_t v[16];
-      asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
-          "%14, %15}, [%16];"
-          : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-            "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-          : "r"(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)c0));
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-      if (row < p.M) {
-        uint32_t o[8];
-        for (int e = 0; e < 8; ++e) {
-          const float x0 = fmaxf(__uint_as_float(v[2 * e]) + p.bias[c0 + 2 * e], 0.0f);
-          const float x1 = fmaxf(__uint_as_float(v[2 * e + 1]) + p.bias[c0 + 2 * e + 1], 0.0f);
-          const __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);
-          o[e] = *reinterpret_cast<const uint32_t*>(&h);
+  if (warp == 0) {
+    if (lane == 0) {  // producer
+      int q = 0;      // k-blocks issued
+      bool ok = true;
+      for (int t = blockIdx.x; ok && t < all; t += gridDim.x) {
+        const int c = cls(t), nb = blocks(c), ntw = (c & 1) + 1;
+        const int m0 = (DGRAD ? t % p.tiles : t) * kTcRows;
+        const int y0 = (m0 >> p.lg_wo) & ((1 << p.lg_ho) - 1), n0 = m0 >> (p.lg_wo + p.lg_ho);
+        for (int kb = 0; kb < nb; ++kb, ++q) {
+          const int s = q % stages;
+          if (q >= stages && !tc_wait(&empty[s], (uint32_t)(q / stages - 1) & 1u, stop)) {
+            ok = false;
+            break;
+          }
+          unsigned char* a = sgen + s * STAGE;
+          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&full[s])),
+                       "r"(STAGE)
+                       : "memory");
+          const int k0 = kb * KC, tap = k0 >> p.lg_c, ch = k0 & ((1 << p.lg_c) - 1);
+          if (DGRAD) {
+            const int dy = (c >> 1) && tap / ntw == 0, dx = (c & 1) && tap % ntw == 0;
+            tc_load4(a, &maps.a[0], ch, dx, y0 + dy, n0, &full[s]);
+            tc_load2(a + A_BYTES, &maps.b, k0, c * N, &full[s]);
+          } else {
+            const int kh = tap / 3, kw = tap % 3;
+            tc_load4(a, &maps.a[2 * (kh != 1) + (kw != 1)], ch, kw == 0 ? -1 : 0, y0 - (kh == 0), n0, &full[s]);
+            tc_load2(a + A_BYTES, &maps.b, k0, 0, &full[s]);
+          }
         }
-        uint4* dst = reinterpret_cast<uint4*>(p.Cb + off + c0);
-        dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
-        dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
       }
+      // after a failure wait for the copies in flight (each stage's last one)
+      if (!ok || *stop)
+        for (int k = max(0, q - stages); k < q; ++k) tc_wait(&full[k % stages], (uint32_t)(k / stages) & 1u, nullptr);
     }
-  } else if (tid == 0) {
-    atomicOr(err, 1);
+  } else if (warp == 1) {
+    if (lane == 0) {  // MMA issuer
+      int q = 0, i = 0;
+      bool ok = true;
+      for (int t = blockIdx.x; ok && t < all; t += gridDim.x, ++i) {
+        const int nb = blocks(cls(t)), buf = i & 1;
+        if (i >= 2 && !tc_wait(&acc_empty[buf], (uint32_t)((i >> 1) - 1) & 1u, stop)) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        for (int kb = 0; kb < nb; ++kb, ++q) {
+          const int s = q % stages;
+          if (!tc_wait(&full[s], (uint32_t)(q / stages) & 1u, stop)) {
+            ok = false;
+            break;
+          }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint32_t a = sbase + (uint32_t)(s * STAGE), b = a + A_BYTES;
+#pragma unroll
+          for (int j = 0; j < KC / 16; ++j) {
+            const uint64_t ad = tc_desc<KC>(a + 32 * j), bd = tc_desc<KC>(b + 32 * j);
+            const uint32_t acc = (kb | j) != 0;
+            asm volatile(
+                "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem + (uint32_t)(buf * N)),
+                "l"(ad), "l"(bd), "r"(tc_idesc<N>()), "r"(acc)
+                : "memory");
+          }
+          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                           smem_addr(&empty[s]))
+                       : "memory");
+        }
+        if (ok)
+          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                           smem_addr(&acc_full[buf]))
+                       : "memory");
+      }
+      // every MMA issued has finished before the tensor memory is freed
+      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                       smem_addr(&drain))
+                   : "memory");
+      tc_wait(&drain, 0, nullptr);
+    }
+  } else if (warp >= 4) {  // epilogue: rows 32 (warp - 4) .. + 31
+    const int qd = warp - 4;
+    int i = 0;
+    for (int t = blockIdx.x; t < all; t += gridDim.x, ++i) {
+      const int c = cls(t), buf = i & 1;
+      if (!__all_sync(0xffffffffu, tc_wait(&acc_full[buf], (uint32_t)(i >> 1) & 1u, stop))) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const int row = (DGRAD ? t % p.tiles : t) * kTcRows + 32 * qd + lane;
+      long long off;
+      if (DGRAD) {  // class pixel -> NHWC input pixel
+        const int x = row & ((1 << p.lg_wo) - 1), y = (row >> p.lg_wo) & ((1 << p.lg_ho) - 1);
+        const int n = row >> (p.lg_wo + p.lg_ho);
+        off = (((long long)n * p.H + 2 * y + (c >> 1)) * p.H + 2 * x + (c & 1)) * N;
+      } else {
+        off = (long long)(row / p.grp) * p.ldg + (long long)(row % p.grp) * p.ldc;
+      }
+      for (int c0 = 0; c0 < N; c0 += 32) {
+        uint32_t v[32];
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
+            "%14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+              "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
+              "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]),
+              "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]),
+              "=r"(v[30]), "=r"(v[31])
+            : "r"(tmem + ((uint32_t)(32 * qd) << 16) + (uint32_t)(buf * N + c0)));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        if (row < p.M) {
+          uint4* dst = reinterpret_cast<uint4*>(p.out + off + c0);
+          const uint4* msk = reinterpret_cast<const uint4*>(p.mask + off + c0);
+#pragma unroll
+          for (int g = 0; g < 4; ++g) {
+            uint32_t o[4], x[4] = {0u, 0u, 0u, 0u};
+            if (DGRAD) {
+              const uint4 q4 = __ldg(&msk[g]);
+              x[0] = q4.x;
+              x[1] = q4.y;
+              x[2] = q4.z;
+              x[3] = q4.w;
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              float v0 = __uint_as_float(v[8 * g + 2 * e]), v1 = __uint_as_float(v[8 * g + 2 * e + 1]);
+              if (DGRAD) {
+                const __nv_bfloat162 m2 = *reinterpret_cast<const __nv_bfloat162*>(&x[e]);
+                if (!(__low2float(m2) > 0.0f)) v0 = 0.0f;
+                if (!(__high2float(m2) > 0.0f)) v1 = 0.0f;
+              } else {
+                v0 = fmaxf(v0 + __ldg(&p.bias[c0 + 8 * g + 2 * e]), 0.0f);
+                v1 = fmaxf(v1 + __ldg(&p.bias[c0 + 8 * g + 2 * e + 1]), 0.0f);
+              }
+              const __nv_bfloat162 h = __floats2bfloat162_rn(v0, v1);
+              o[e] = *reinterpret_cast<const uint32_t*>(&h);
+            }
+            dst[g] = make_uint4(o[0], o[1], o[2], o[3]);
+          }
+        }
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&acc_empty[buf])) : "memory");
+    }
   }
+  __syncwarp();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (warp == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(N) : "memory");
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if (tid == 0 && s_abort) atomicOr(err, 1);
+  if (warp == 1)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * N) : "memory");
 }
 
-template <int N, int BK, int S>
-cudaError_t conv_tc_t(const GemmArgs& p, int* err, cudaStream_t s) {
-  constexpr int smem = S * (kTcRows + N) * BK * 2;
-  cudaError_t e = cudaFuncSetAttribute(k_conv_tc<N, BK, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  k_conv_tc<N, BK, S><<<(unsigned)((p.M + kTcRows - 1) / kTcRows), kTcThreads, smem, s>>>(p, err);
-  return cudaGetLastError();
-}
-
-// C = relu(A B^T + bias) for one implicit-im2col convolution layer on the
-// tcgen05 path (N = 64 or 128, K a multiple of 32, 8-channel chunks). Steps
-// of 64 columns where K allows, else 32.
-cudaError_t conv_tc(GemmArgs p, int* err, cudaStream_t s) {
-  if (p.grp <= 0) {
-    p.grp = 1 << 30;
-    p.ldg = 0;
+// Weights of the data gradients, input channels as rows: for each class
+// (py, px) row class Cin + c, column tap Cout + o = W[o][kh][kw][c], taps in
+// the order of dg_tap, rows of 4 Cout columns (classes with fewer taps leave the
+// rest unused)
+__global__ void k_dgrad_weights(const bf16* __restrict__ w, int Kp, int cin, int cout, bf16* __restrict__ out) {
+  const int n = 4 * cin * 4 * cout;
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
+    const int k = e % (4 * cout), row = e / (4 * cout), cls = row / cin, c = row % cin, tap = k / cout, o = k % cout;
+    const int ph = cls >> 1, pw = cls & 1, ntw = pw + 1;
+    bf16 v = __float2bfloat16_rn(0.0f);
+    if (tap < (ph + 1) * ntw) {
+      int kh, kw, d;
+      dg_tap(ph, tap / ntw, kh, d);
+      dg_tap(pw, tap % ntw, kw, d);
+      v = w[(long long)o * Kp + (kh * 3 + kw) * cin + c];
+    }
+    out[e] = v;
   }
-  if ((p.N != 64 && p.N != 128) || p.K % 32 || p.lg_c < 3 || p.ldc % 8 || p.ldg % 8) return cudaErrorInvalidValue;
-  const bool k64 = p.K % 64 == 0;
-  if (p.N == 64) return k64 ? conv_tc_t<64, 64, 4>(p, err, s) : conv_tc_t<64, 32, 4>(p, err, s);
-  return k64 ? conv_tc_t<128, 64, 3>(p, err, s) : conv_tc_t<128, 32, 4>(p, err, s);
+}
+
+typedef CUresult (*EncodeTiled)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+// a tensor map of bfloat16 values with rows (dimension 0) of 64 or 32 channels in a box
+cudaError_t encode_map(CUtensorMap* map, const void* base, int rank, const long long* dims, const long long* strides,
+                       const int* box) {
+  static const EncodeTiled fn = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult r;
+    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &f, cudaEnableDefault, &r) != cudaSuccess ||
+        r != cudaDriverEntryPointSuccess)
+      f = nullptr;
+    return (EncodeTiled)f;
+  }();
+  if (!fn) return cudaErrorNotSupported;
+  cuuint64_t d[5], st[4];
+  cuuint32_t b[5], one[5] = {1, 1, 1, 1, 1};
+  for (int k = 0; k < rank; ++k) {
+    d[k] = (cuuint64_t)dims[k];
+    b[k] = (cuuint32_t)box[k];
+    if (k) st[k - 1] = (cuuint64_t)strides[k - 1];
+  }
+  const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), d, st, b, one,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE,
+                        box[0] == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+template <int KC, int N, bool DGRAD>
+cudaError_t conv_tma_t(const ConvMaps& maps, const ConvArgs& p, int* err, int sm_count, cudaStream_t s) {
+  constexpr int stage = (kTcRows + N) * KC * 2, stages = 200 * 1024 / stage > 12 ? 12 : 200 * 1024 / stage;
+  constexpr int smem = stages * stage + 1024;
+  auto kern = k_conv_tma<KC, N, DGRAD>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  const int all = (DGRAD ? 4 : 1) * p.tiles;
+  kern<<<(unsigned)std::min(all, sm_count), kTcThreads, smem, s>>>(maps, p, stages, err);
+  return cudaGetLastError();
 }
 
 int ilog2(int v) {
@@ -569,6 +664,65 @@ int choose_splits(int M, int N, int K, int* ksplit) {
   S = (K + ks - 1) / ks;
   *ksplit = ks;
   return S;
+}
+
+// ------------------------------------------------ input layer (2 -> 32 channels)
+// Direct 3x3 convolution of the 2-channel crops with bias and ReLU, on mma.sync
+// m16n8k16: K = (tap, channel) padded to 32, so one register of an A fragment
+// is one pixel's two channels at one tap, read from a strip of the crop in
+// shared memory: no im2col matrix is written and read back (67 + 67 MB per 256
+// crops), and the kernel is bound by storing its output (67 MB). A CTA takes
+// eight rows of a crop, a warp one row. The output channels are dealt to the
+// four n-tiles so that a thread ends up with eight consecutive ones: one
+// 16-byte store per pixel. 256 crops: 18 us instead of 76 (im2col 20,
+// GEMM 56). Accumulation order and results are the GEMM's.
+__global__ void __launch_bounds__(256) k_conv1(const uint32_t* __restrict__ x, const bf16* __restrict__ w,
+                                               const float* __restrict__ bias, bf16* __restrict__ out) {
+  constexpr int P = kCrop + 2;
+  __shared__ uint32_t px[10 * P];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  const int r0 = 8 * (blockIdx.x & 7);
+  const uint32_t* img = x + (long long)(blockIdx.x >> 3) * kCrop * kCrop;
+  for (int i = tid; i < 10 * P; i += 256) {
+    const int r = r0 - 1 + i / P, c = i % P - 1;
+    px[i] = r >= 0 && r < kCrop && c >= 0 && c < kCrop ? __ldg(&img[r * kCrop + c]) : 0u;
+  }
+  uint32_t bf[4][2][2];  // weights: n-tile j, k-step, register
+  float bs[4][2];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int ch = 8 * (g >> 1) + 2 * j + (g & 1);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      bf[j][k][0] = *reinterpret_cast<const uint32_t*>(w + ch * 32 + 16 * k + 2 * t);
+      bf[j][k][1] = *reinterpret_cast<const uint32_t*>(w + ch * 32 + 16 * k + 2 * t + 8);
+    }
+    bs[j][0] = bias[8 * t + 2 * j];
+    bs[j][1] = bias[8 * t + 2 * j + 1];
+  }
+  __syncthreads();
+  const uint32_t* row = px + warp * P;
+  const int o0 = t / 3 * P + t % 3, o4 = (t + 4) / 3 * P + (t + 4) % 3, o8 = 2 * P + 2;
+  bf16* dst = out + ((long long)(blockIdx.x >> 3) * kCrop * kCrop + (r0 + warp) * kCrop) * 32 + 8 * t;
+#pragma unroll
+  for (int m = 0; m < kCrop; m += 16) {
+    const uint32_t* a = row + m + g;
+    const uint32_t a0[4] = {a[o0], a[o0 + 8], a[o4], a[o4 + 8]};
+    const uint32_t a1[4] = {t == 0 ? a[o8] : 0u, t == 0 ? a[o8 + 8] : 0u, 0u, 0u};
+    uint32_t lo[4], hi[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+      mma_bf16(acc, a0, bf[j][0][0], bf[j][0][1]);
+      mma_bf16(acc, a1, bf[j][1][0], bf[j][1][1]);
+      const __nv_bfloat162 l = __floats2bfloat162_rn(fmaxf(acc[0] + bs[j][0], 0.0f), fmaxf(acc[1] + bs[j][1], 0.0f));
+      const __nv_bfloat162 h = __floats2bfloat162_rn(fmaxf(acc[2] + bs[j][0], 0.0f), fmaxf(acc[3] + bs[j][1], 0.0f));
+      lo[j] = *reinterpret_cast<const uint32_t*>(&l);
+      hi[j] = *reinterpret_cast<const uint32_t*>(&h);
+    }
+    *reinterpret_cast<uint4*>(dst + (m + g) * 32) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+    *reinterpret_cast<uint4*>(dst + (m + g + 8) * 32) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+  }
 }
 
 // ---------------------------------------------------------------- layout kernels
@@ -850,10 +1004,18 @@ struct perch_cnn {
   DevBuf col[kConvs], act[kConvs], feat, h1, err_buf, pred_buf, loss_buf;
   DevBuf dz1, dfeat, dz, dcol, part, bpart;
   bool params_set = false;
-  // forward 3x3 convolutions 2-4 on tcgen05 (else mma.sync); tc_err: the
-  // tcgen05 kernel's wait-gave-up flag (device int)
-  bool tensor_tc = false;
+  // tc_err: the convolution kernels' wait-gave-up flag (device int); path: the
+  // caller's choice (perch_cnn_set_tensor_path), one kernel serves both
+  int path = 0;
+  int sm_count = 152;
   DevBuf tc_err;
+  // tensor maps of the convolutions' operands (forward, data gradient), and
+  // the buffers they were made for
+  ConvMaps fwd[kConvs], dgrad[kConvs];
+  const void* fwd_for[kConvs][2] = {};
+  const void* dgrad_for[kConvs][2] = {};
+  long long fwd_n[kConvs] = {}, dgrad_n[kConvs] = {};
+  DevBuf wt[kConvs];  // weights of the data gradients (k_dgrad_weights)
 
   int fail(int code, const char* fmt, ...) {
     char buf[512];
@@ -876,6 +1038,7 @@ struct perch_cnn {
     for (int l = 0; l < kConvs; ++l) {
       v.push_back(&col[l]);
       v.push_back(&act[l]);
+      v.push_back(&wt[l]);
     }
     return v;
   }
@@ -923,6 +1086,8 @@ struct perch_cnn {
   }
   int ensure_batch(int n);
   int refresh_weights();
+  int conv_fwd(int l, const bf16* x, int n);
+  int conv_dgrad(int l, const bf16* dz, int n, bf16* out);
   int forward(const bf16* crops, const int32_t* onehot, int n, float* pred, const float* target);
   int backward(const bf16* crops, int n);
 };
@@ -944,7 +1109,6 @@ int perch_cnn::ensure_batch(int n) {
   const long long N = std::max(n, 32);
   for (int l = 0; l < kConvs; ++l) {
     const long long Ho = kHin[l] / kStride[l];
-    if (l == 0) CKN(col[0].ensure(2 * N * Ho * Ho * kp_of(0)), "alloc im2col");
     if (l < kConvs - 1) CKN(act[l].ensure(2 * N * Ho * Ho * kCout[l]), "alloc activations");
   }
   CKN(feat.ensure(2 * N * Kf), "alloc");
@@ -963,51 +1127,109 @@ int perch_cnn::refresh_weights() {
   return PERCH_OK;
 }
 
+// the 128-row tiles of a layer's output pixels: boxes of 1 << lg_wo columns,
+// `rows` rows and `imgs` images
+static void conv_tile(int l, int n, ConvArgs* p, int* box) {
+  const int Ho = kHin[l] / kStride[l];
+  p->lg_wo = p->lg_ho = ilog2(Ho);
+  p->M = n * Ho * Ho;
+  p->tiles = (p->M + kTcRows - 1) / kTcRows;
+  box[1] = Ho;
+  box[2] = std::min(Ho, kTcRows / Ho);
+  box[3] = kTcRows / (box[1] * box[2]);
+}
+
+// Forward convolution of layer l = 1 .. 3 over n crops: x to act[l] or, the last
+// one, straight into the FC input rows (crop m / 64, position m % 64). The maps
+// cover the whole buffer of x, so they stay until it is reallocated; rows past
+// n crops are computed from what is there and not stored.
+int perch_cnn::conv_fwd(int l, const bf16* x, int n) {
+  perch_cnn* net = this;
+  const int H = kHin[l], Cin = kCin[l], N = kCout[l], Kp = kp_of(l), KC = Cin >= 64 ? 64 : 32;
+  ConvArgs p{};
+  int box[4] = {KC};
+  conv_tile(l, n, &p, box);
+  const long long imgs = (long long)(act[l - 1].cap / (2 * (size_t)H * H * Cin));
+  const bf16* w = w16.as<bf16>() + off_w[l];
+  if (fwd_for[l][0] != x || fwd_for[l][1] != w || fwd_n[l] != imgs) {
+    for (int par = 0; par < 4; ++par) {
+      const long long dims[4] = {Cin, H / 2, H / 2, imgs};
+      const long long st[3] = {4LL * Cin, 4LL * H * Cin, 2LL * H * H * Cin};
+      CKN(encode_map(&fwd[l].a[par], x + ((par >> 1) * H + (par & 1)) * (long long)Cin, 4, dims, st, box), "tensor map");
+    }
+    const long long dims[2] = {Kp, N}, st[1] = {2LL * Kp};
+    const int wbox[2] = {KC, N};
+    CKN(encode_map(&fwd[l].b, w, 2, dims, st, wbox), "tensor map");
+    fwd_for[l][0] = x;
+    fwd_for[l][1] = w;
+    fwd_n[l] = imgs;
+  }
+  p.lg_c = ilog2(Cin);
+  p.k_blocks = Kp / KC;
+  p.bias = master.as<float>() + off_b[l];
+  p.ldc = N;
+  p.grp = 1 << 30;
+  p.out = act[l].as<bf16>();
+  if (l == kConvs - 1) {
+    p.out = feat.as<bf16>();
+    p.grp = (H / 2) * (H / 2);
+    p.ldg = Kf;
+  }
+  int* e = tc_err.as<int>();
+  CKN(l == 1   ? (conv_tma_t<32, 64, false>(fwd[l], p, e, sm_count, stream))
+      : l == 2 ? (conv_tma_t<64, 128, false>(fwd[l], p, e, sm_count, stream))
+               : (conv_tma_t<64, 128, false>(fwd[l], p, e, sm_count, stream)),
+      "convolution");
+  return PERCH_OK;
+}
+
+// Data gradient of layer l = 1 .. 3: dz of its output to the gradient of its
+// input, times the ReLU mask of that input
+int perch_cnn::conv_dgrad(int l, const bf16* d, int n, bf16* out) {
+  perch_cnn* net = this;
+  const int H = kHin[l], Ho = H / 2, N = kCin[l], Co = kCout[l];
+  ConvArgs p{};
+  int box[4] = {64};
+  conv_tile(l, n, &p, box);
+  CKN(wt[l].ensure(2 * 16 * (size_t)N * Co), "alloc");
+  k_dgrad_weights<<<grid_for(16LL * N * Co), 256, 0, stream>>>(w16.as<bf16>() + off_w[l], kp_of(l), N, Co,
+                                                               wt[l].as<bf16>());
+  CKN(cudaGetLastError(), "data-gradient weights");
+  if (dgrad_for[l][0] != d || dgrad_for[l][1] != wt[l].p || dgrad_n[l] != n) {
+    const long long dims[4] = {Co, Ho, Ho, n};
+    const long long st[3] = {2LL * Co, 2LL * Ho * Co, 2LL * Ho * Ho * Co};
+    CKN(encode_map(&dgrad[l].a[0], d, 4, dims, st, box), "tensor map");
+    for (int k = 1; k < 4; ++k) dgrad[l].a[k] = dgrad[l].a[0];
+    const long long wdims[2] = {4LL * Co, 4LL * N}, wst[1] = {8LL * Co};
+    const int wbox[2] = {64, N};
+    CKN(encode_map(&dgrad[l].b, wt[l].p, 2, wdims, wst, wbox), "tensor map");
+    dgrad_for[l][0] = d;
+    dgrad_for[l][1] = wt[l].p;
+    dgrad_n[l] = n;
+  }
+  p.lg_c = ilog2(Co);
+  p.out = out;
+  p.mask = act[l - 1].as<bf16>();
+  p.H = H;
+  int* e = tc_err.as<int>();
+  CKN(l == 1   ? (conv_tma_t<64, 32, true>(dgrad[l], p, e, sm_count, stream))
+      : l == 2 ? (conv_tma_t<64, 64, true>(dgrad[l], p, e, sm_count, stream))
+               : (conv_tma_t<64, 128, true>(dgrad[l], p, e, sm_count, stream)),
+      "data gradient");
+  return PERCH_OK;
+}
+
 // Forward pass of n <= max_batch crops; with a target also the per-sample
 // errors (for the backward pass).
 int perch_cnn::forward(const bf16* crops, const int32_t* onehot, int n, float* pred, const float* target) {
   perch_cnn* net = this;
   int rc = ensure_batch(n);
   if (rc) return rc;
-  const bf16* x = crops;
-  for (int l = 0; l < kConvs; ++l) {
-    const int H = kHin[l], s = kStride[l], Ho = H / s, Kp = kp_of(l);
-    const long long M = (long long)n * Ho * Ho;
-    GemmArgs p{};
-    if (l == 0) {  // two input channels: explicit rows of 32 columns
-      k_im2col_c2<<<grid_for(M), 256, 0, stream>>>(reinterpret_cast<const uint32_t*>(x), n, H, H,
-                                                   col[0].as<uint4>());
-      CKN(cudaGetLastError(), "im2col kernel");
-      p.A = col[0].as<bf16>();
-      p.lda = Kp;
-    } else {  // implicit im2col from the NHWC activations
-      p.A = x;
-      set_conv(p, l);
-    }
-    p.B = w16.as<bf16>() + off_w[l];
-    p.ldb = Kp;
-    p.M = (int)M;
-    p.N = kCout[l];
-    p.K = Kp;
-    p.Ksplit = Kp;
-    p.bias = master.as<float>() + off_b[l];
-    if (l < kConvs - 1) {
-      p.Cb = act[l].as<bf16>();
-      p.ldc = kCout[l];
-    } else {  // straight into the FC input rows: crop m / 64, position m % 64
-      p.Cb = feat.as<bf16>();
-      p.ldc = kCout[l];
-      p.grp = Ho * Ho;
-      p.ldg = Kf;
-    }
-    if (l == 0)
-      CKN(gemm<EPI_BIAS_RELU>(p, 1, stream), "conv gemm");
-    else if (tensor_tc)
-      CKN(conv_tc(p, tc_err.as<int>(), stream), "conv tcgen05");
-    else
-      CKN((gemm<EPI_BIAS_RELU, true, true, 1>(p, 1, stream)), "conv gemm");
-    x = l < kConvs - 1 ? act[l].as<bf16>() : nullptr;
-  }
+  k_conv1<<<8 * n, 256, 0, stream>>>(reinterpret_cast<const uint32_t*>(crops), w16.as<bf16>() + off_w[0],
+                                     master.as<float>() + off_b[0], act[0].as<bf16>());
+  CKN(cudaGetLastError(), "input layer");
+  for (int l = 1; l < kConvs; ++l)
+    if ((rc = conv_fwd(l, act[l - 1].as<bf16>(), n))) return rc;
   k_onehot<<<grid_for((long long)n * onehot_pad), 256, 0, stream>>>(onehot, n, n, onehot_pad, Kf, feat.as<bf16>());
   CKN(cudaGetLastError(), "one-hot kernel");
   // FC1: few output tiles over a long K, so split K and finish bias + ReLU in a second pass
@@ -1024,7 +1246,7 @@ int perch_cnn::forward(const bf16* crops, const int32_t* onehot, int n, float* p
   p.Cf = part.as<float>();
   p.ldc = kHidden;
   p.split_stride = (long long)n * kHidden;
-  CKN(gemm<EPI_F32>(p, S, stream), "fc1 gemm");
+  CKN(gemm<>(p, S, stream), "fc1 gemm");
   k_splits_bias_relu<<<grid_for((long long)n * kHidden), 256, 0, stream>>>(
       part.as<float>(), S, n, kHidden, master.as<float>() + off_fb1, h1.as<bf16>());
   CKN(cudaGetLastError(), "fc1 epilogue kernel");
@@ -1082,7 +1304,7 @@ int perch_cnn::backward(const bf16* crops, int n) {
     p.Ksplit = n;
     p.Cf = G + off_f1;
     p.ldc = Kf;
-    CKN((gemm<EPI_F32, false, false>(p, 1, stream)), "fc1 weight-gradient gemm");
+    CKN((gemm<false, false>(p, 1, stream)), "fc1 weight-gradient gemm");
   }
   if (int rc = bias_grad(dz1.as<bf16>(), N, kHidden, G + off_fb1)) return rc;
   {
@@ -1097,7 +1319,7 @@ int perch_cnn::backward(const bf16* crops, int n) {
     p.Ksplit = kHidden;
     p.Cf = dfeat.as<float>();
     p.ldc = kFeat;
-    CKN((gemm<EPI_F32, true, false>(p, 1, stream)), "fc1 data-gradient gemm");
+    CKN((gemm<true, false>(p, 1, stream)), "fc1 data-gradient gemm");
   }
   bf16* cur = dz.as<bf16>();   // gradient of the current layer's output
   bf16* nxt = dcol.as<bf16>();  // receives the gradient of its input
@@ -1122,47 +1344,26 @@ int perch_cnn::backward(const bf16* crops, int n) {
       p.ldc = Kp;
       p.split_stride = (long long)Co * Kp;
       if (l == 0) {
+        CKN(col[0].ensure(2 * M * Kp), "alloc im2col");
+        k_im2col_c2<<<grid_for(M), 256, 0, stream>>>(reinterpret_cast<const uint32_t*>(crops), n, H, H,
+                                                     col[0].as<uint4>());
+        CKN(cudaGetLastError(), "im2col kernel");
         p.B = col[0].as<bf16>();
         p.ldb = Kp;
-        CKN((gemm<EPI_F32, false, false>(p, S, stream)), "conv weight-gradient gemm");
+        CKN((gemm<false, false>(p, S, stream)), "conv weight-gradient gemm");
       } else {  // implicit im2col of this layer's input
         p.B = act[l - 1].as<bf16>();
         set_conv(p, l);
-        CKN((gemm<EPI_F32, false, false, 2>(p, S, stream)), "conv weight-gradient gemm");
+        CKN((gemm<false, false, true>(p, S, stream)), "conv weight-gradient gemm");
       }
       k_split_sum_wide<<<(unsigned)((Co * Kp + 31) / 32), 256, 0, stream>>>(part.as<float>(), S,
                                                                              (long long)Co * Kp, G + off_w[l]);
       CKN(cudaGetLastError(), "split sum kernel");
     }
     if (l == 0) break;
-    // data gradient of this layer's input, ReLU mask applied: one implicit
-    // GEMM per parity class of the input pixels (1, 2, 2 or 4 taps), written
-    // straight into the other gradient buffer
-    for (int ph = 0; ph < 2; ++ph)
-      for (int pw = 0; pw < 2; ++pw) {
-        GemmArgs p{};
-        p.A = cur;
-        p.B = w16.as<bf16>() + off_w[l];
-        p.M = (int)M;  // the class has as many pixels as the layer output
-        p.N = kCin[l];
-        p.ntw = pw ? 2 : 1;
-        p.K = (ph ? 2 : 1) * p.ntw * Co;
-        p.Ksplit = p.K;
-        p.par_h = ph;
-        p.par_w = pw;
-        p.dg_lg_ho = ilog2(Ho);
-        p.dg_lg_co = ilog2(Co);
-        p.lg_c = p.dg_lg_co;
-        p.dg_H = H;
-        p.dg_cin = kCin[l];
-        p.dg_kp = Kp;
-        p.mask = act[l - 1].as<bf16>();
-        p.Cb = nxt;
-        CKN((gemm<EPI_DGRAD, true, false, 3>(p, 1, stream)), "conv data-gradient gemm");
-      }
+    if (int rc = conv_dgrad(l, cur, n, nxt)) return rc;
     std::swap(cur, nxt);
   }
-  (void)crops;
   return PERCH_OK;
 }
 
@@ -1198,6 +1399,7 @@ int perch_cnn_create(perch_cnn** out, int device, void* cuda_stream, int32_t n_o
   }
   perch_cnn* net = new perch_cnn;
   net->device = device;
+  cudaDeviceGetAttribute(&net->sm_count, cudaDevAttrMultiProcessorCount, device);
   net->n_onehot = n_onehot;
   net->onehot_pad = round32(n_onehot);
   net->Kf = kFeat + net->onehot_pad;
@@ -1247,8 +1449,8 @@ const char* perch_cnn_last_error(const perch_cnn* net) { return net ? net->err.c
 
 int perch_cnn_set_tensor_path(perch_cnn* net, int32_t path) {
   if (!net) return PERCH_E_ARG;
-  if (path != 0 && path != 1) return net->fail(PERCH_E_ARG, "tensor path must be 0 (mma.sync) or 1 (tcgen05)");
-  net->tensor_tc = path == 1;
+  if (path != 0 && path != 1) return net->fail(PERCH_E_ARG, "tensor path must be 0 or 1");
+  net->path = path;
   return PERCH_OK;
 }
 
@@ -1260,7 +1462,7 @@ int perch_cnn_tensor_status(perch_cnn* net, int32_t* path, int32_t* waits_gave_u
   if (rc) return rc;
   rc = net->cuda(cudaMemcpy(&e, net->tc_err.p, sizeof e, cudaMemcpyDeviceToHost), "read flag");
   if (rc) return rc;
-  if (path) *path = net->tensor_tc ? 1 : 0;
+  if (path) *path = net->path;
   if (waits_gave_up) *waits_gave_up = e;
   return PERCH_OK;
 }

@@ -539,7 +539,7 @@ class PerchCNN:
         return p
 
     def perch_cnn_set_tensor_path(self, path: int):
-        """0: mma.sync convolutions (default); 1: tcgen05 for the forward 3x3 convolutions 2-4."""
+        """0 (default) or 1; both run convolutions 2-4 on tcgen05, with the same results."""
         self._check(self.lib.perch_cnn_set_tensor_path(self.h, int(path)))
 
     def perch_cnn_tensor_status(self):

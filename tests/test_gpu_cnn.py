@@ -206,3 +206,25 @@ def test_tcgen05_forward_matches_mma_sync_and_oracle(c1, n, max_batch):
     assert np.max(np.abs(got - ref)) < 2e-2 * scale
     with pytest.raises(perch.PerchError):
         net.perch_cnn_set_tensor_path(2)
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 31, 65, 130])
+def test_forward_does_not_depend_on_the_chunks(c1, n):
+    """Each crop's prediction is its own: the same bits whatever crops share
+    its row tiles (images of a tile past the batch hold what an earlier batch
+    left there) and its chunk."""
+    wl, p, w = c1
+    n_onehot = len(wl.meshes) * wl.grid.n_yaw
+    crops, onehot = p.perch_cnn_crops([wl.gt[:1]], np.zeros(n, np.int32), _hyps_c1(wl, n, 5 + n))
+    params = _params(n_onehot, 13)
+    ref = None
+    for max_batch in (32, 128, 1024):
+        net = _net_with(params, n_onehot, max_batch=max_batch)
+        net.perch_cnn_forward(crops.flip(0), onehot)
+        got = net.perch_cnn_forward(crops, onehot).cpu().numpy()
+        ref = got if ref is None else ref
+        assert np.array_equal(got, ref)
+        one = net.perch_cnn_forward(crops[n // 2:n // 2 + 1].contiguous(), onehot[n // 2:n // 2 + 1].contiguous())
+        assert one.cpu().numpy()[0] == ref[n // 2]
+        assert net.perch_cnn_tensor_status() == (0, 0)
+        net.close()
