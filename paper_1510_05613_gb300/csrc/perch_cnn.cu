@@ -119,14 +119,6 @@ __device__ __forceinline__ const bf16* conv_src(const GemmArgs& p, const bf16* x
   return x + ((((long long)n * p.cH + r) * p.cH + cc) << p.lg_c) + c;
 }
 
-// Taps of one parity of a stride-2, pad-1, 3x3 convolution's input: an even
-// coordinate 2a is read by kernel offset 1 of output a; an odd one 2a + 1 by
-// offset 0 of output a + 1 and offset 2 of output a.
-__device__ __forceinline__ void dg_tap(int par, int t, int& kofs, int& d) {
-  kofs = par == 0 ? 1 : (t == 0 ? 0 : 2);
-  d = (par == 1 && t == 0) ? 1 : 0;
-}
-
 template <int BN, bool AK, bool BKC, bool CONV>
 __global__ void __launch_bounds__(256) k_gemm(GemmArgs p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -291,35 +283,42 @@ cudaError_t gemm(const GemmArgs& p, int splits, cudaStream_t s) {
 // - forward: the input pixels of one tap have one parity in y and in x, so
 //   each layer has four maps of its input, one per parity, with strides of
 //   two pixels (row 2i - 1 + kh is row i - [kh = 0] of parity [kh != 1]);
-// - data gradient: the input pixels of one parity class (py, px) take 1, 2, 2
-//   or 4 taps of dz at (y + dy, x + dx), dy, dx in {0, 1}; the four classes are
-//   tiles of the same launch, the longest first. Its B operand is the
-//   weights with input channels as rows (k_dgrad_weights).
-// K runs over (tap, channel) in order in steps of 16, as the mma.sync kernels
-// run it, and the results are the same bit for bit.
+// - data gradient: the input pixels of parity class (py, px) take 1, 2, 2 or 4
+//   taps of dz at (y + dy, x + dx), dy, dx in {0, 1}. A tile is 128 pixels of
+//   dz's grid with all four classes: each of the four boxes of dz is loaded
+//   once and multiplied with the taps of all classes that take it, side by side
+//   in one MMA (k_dgrad_weights lays them out so).
+// With 32 channels two horizontal neighbours are one 128-byte row of the box, taps
+// kw = 1 and 2 together. K runs over (tap, channel) in order in steps of 16 for
+// each output, as the mma.sync kernels run it, and the results are the same bit for bit.
 //
-// One CTA per SM: thread 0 of warp 0 fills a ring of S stages (A 128 x KC and
-// B N x KC, swizzled K-major rows of 2 KC bytes), thread 0 of warp 1 issues the
-// MMAs into one of two tensor-memory accumulators, warps 4-7 read the other
-// one back (bias + ReLU, or the ReLU mask of the layer input) and store
-// bfloat16 rows. Every wait is bounded; a wait that gives up raises s_abort,
-// which ends the other roles' waits, the copies and MMAs in flight are waited
-// for, the tensor memory is freed and *err is set.
+// One CTA per SM: warp 0 fills a ring of stages (A 128 x KC, swizzled K-major
+// rows), warp 1 issues the MMAs into one of two tensor-memory accumulators,
+// warps 4-7 and 8-11 take turns in reading the other one back (bias + ReLU, or
+// the ReLU mask of the layer input) and storing bfloat16 rows. The weights stay in
+// shared memory, loaded with the first tile (layer 4's 295 KB do not fit and
+// are staged with A). Warps 0 and 1 run their loops as whole warps and issue
+// from one elected lane: from a branch on a lane number an MMA took 62 clocks to
+// issue, not 23, and a k-block 800, not 510. Every wait is bounded; a wait that
+// gives up raises s_abort, which ends the other roles' waits, the copies and MMAs in
+// flight are waited for, the tensor memory is freed and *err is set.
 //
-// Bound by the operand boxes through L2 and the store of the output, not by the
-// tensor pipe: N is 32 to 128, so a 16 KB A box feeds 16 to 64 cycles of MMA.
-// 256 crops, before (cp.async gathers of the same GEMMs, mma.sync) and now:
-// conv2 64 -> 48 us, conv3 and conv4 52 -> 18 each (mean), the twelve class
-// launches of the data gradients 341 -> 78 + 39 + 22.
-constexpr int kTcRows = 128, kTcThreads = 256;
+// Bound by that issue chain per k-block (the MMAs of one take 256 clocks of the
+// tensor pipe) and, in the data gradient of layer 2, by reading the mask and
+// storing (134 MB). 256 crops, cp.async gathers of the same GEMMs on mma.sync -> first
+// tcgen05 version (one thread a role, weights staged, a class per tile, 4
+// epilogue warps) -> now: conv2 64 -> 48 -> 20 us, conv3 52 -> 22 -> 16, conv4
+// 52 -> 14 -> 11, data gradients 341 -> 139 -> 35 + 19 + 19.
+constexpr int kTcRows = 128, kTcThreads = 384;
 
 struct ConvMaps {
-  CUtensorMap a[4];  // forward: the input's parities 2 py + px; data gradient: a[0] = dz
-  CUtensorMap b;     // weights
+  CUtensorMap a[4];  // forward: the input's parities 2 py + px (KC = 96: 2 py + {tap 0, taps 1 and 2});
+                     // data gradient: a[0] = dz
+  CUtensorMap b[2];  // weights (KC = 96: the columns of taps 1 and 2, of tap 0)
 };
 
 struct ConvArgs {
-  int M, tiles;          // rows of one tile row space, 128-row tiles of it (per class in the data gradient)
+  int M, tiles;          // output rows (data gradient: pixels of one parity class), 128-row tiles of them
   int lg_wo, lg_ho;      // the row space: images of Ho x Wo pixels
   int lg_c;              // log2 channels per tap of A
   int k_blocks;          // forward: k-blocks of a tile
@@ -327,51 +326,63 @@ struct ConvArgs {
   bf16* out;
   long long ldc, ldg;    // forward: row m at (m / grp) ldg + (m % grp) ldc
   int grp;
-  const bf16* mask;      // data gradient: the layer input (ReLU mask), NHWC with N channels, side H
-  int H;
+  const bf16* mask;      // data gradient: the layer input (ReLU mask), NHWC with C channels, side H
+  int H, C, parts;       // its N-channel parts
 };
 
-__device__ __forceinline__ void tc_mbar_init(uint64_t* bar, int count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
+// barriers are given by their shared-memory address
+__device__ __forceinline__ void tc_mbar_init(uint32_t bar, int count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
-__device__ __forceinline__ uint64_t tc_now() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ bool tc_try(uint64_t* bar, uint32_t parity) {
+__device__ __forceinline__ bool tc_try(uint32_t bar, uint32_t parity) {
   uint32_t done;
   asm volatile(
       "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
       : "=r"(done)
-      : "r"(smem_addr(bar)), "r"(parity)
+      : "r"(bar), "r"(parity)
       : "memory");
   return done != 0;
 }
-// wait for the phase of the given parity: bounded by polls and by 2 s, and
-// ended by `stop` (nullptr: not)
-__device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity, volatile int* stop) {
-  if (tc_try(bar, parity)) return true;
-  const uint64_t t0 = tc_now();
+// wait for the phase of the given parity: bounded by polls and by 4e9 clocks
+// (about 2 s), and ended by `stop` (nullptr: not)
+__device__ __noinline__ bool tc_poll(uint32_t bar, uint32_t parity, volatile int* stop) {
+  const long long t0 = clock64();
   for (int i = 0; i < (1 << 22); ++i) {
     if (tc_try(bar, parity)) return true;
-    if ((i & 63) == 63 && ((stop && *stop) || tc_now() - t0 > 2000000000ull)) break;
+    if ((i & 63) == 63 && ((stop && *stop) || clock64() - t0 > 4000000000ll)) break;
   }
   if (stop) *stop = 1;
   return false;
 }
-__device__ __forceinline__ void tc_load4(void* dst, const CUtensorMap* map, int c, int x, int y, int n, uint64_t* bar) {
+// by whole warps: all lanes or none see it end
+__device__ __forceinline__ bool tc_wait(uint32_t bar, uint32_t parity, volatile int* stop) {
+  if (__all_sync(0xffffffffu, tc_try(bar, parity))) return true;
+  return __all_sync(0xffffffffu, tc_poll(bar, parity, stop));
+}
+__device__ __forceinline__ bool tc_elect() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
+__device__ __forceinline__ void tc_load4(uint32_t dst, const CUtensorMap* map, int c, int x, int y, int n, uint32_t bar) {
   asm volatile(
       "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
-      ::"r"(smem_addr(dst)), "l"(map), "r"(c), "r"(x), "r"(y), "r"(n), "r"(smem_addr(bar))
+      ::"r"(dst), "l"(map), "r"(c), "r"(x), "r"(y), "r"(n), "r"(bar)
       : "memory");
 }
-__device__ __forceinline__ void tc_load2(void* dst, const CUtensorMap* map, int k, int row, uint64_t* bar) {
+__device__ __forceinline__ void tc_load2(uint32_t dst, const CUtensorMap* map, int k, int row, uint32_t bar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-          smem_addr(dst)),
-      "l"(map), "r"(k), "r"(row), "r"(smem_addr(bar))
+          dst),
+      "l"(map), "r"(k), "r"(row), "r"(bar)
       : "memory");
+}
+__device__ __forceinline__ void tc_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+// arrives at the barrier when the MMAs issued so far have finished
+__device__ __forceinline__ void tc_commit(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 // shared-memory matrix descriptor of a K-major operand with rows of 2 KC bytes
 // in the 128-byte (KC = 64) or 64-byte (KC = 32) swizzle: start address, stride
@@ -381,148 +392,205 @@ __device__ __forceinline__ uint64_t tc_desc(uint32_t saddr) {
   return (uint64_t)((saddr >> 4) & 0x3FFFu) | (1ull << 16) | ((uint64_t)(8 * 2 * KC >> 4) << 32) | (1ull << 46) |
          ((uint64_t)(KC == 64 ? 2 : 4) << 61);
 }
+__device__ __forceinline__ void tc_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+      "l"(a), "l"(b), "r"(idesc), "r"(acc)
+      : "memory");
+}
+__device__ __forceinline__ void tc_expect(uint32_t bar, int bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
 // instruction descriptor of kind::f16: FP32 accumulator, BF16 A and B, both
 // K-major, M = 128, N
-template <int N>
-__device__ __forceinline__ uint32_t tc_idesc() {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kTcRows >> 4) << 24);
+__device__ __forceinline__ uint32_t tc_idesc(int n) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kTcRows >> 4) << 24);
 }
 
-template <int KC, int N, bool DGRAD>
+template <int KC, int N, bool DGRAD, bool RES, int STAGES>
 __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tma(const __grid_constant__ ConvMaps maps, ConvArgs p,
-                                                            int stages, int* err) {
-  static_assert((KC == 32 || KC == 64) && (N == 32 || N == 64 || N == 128), "operand shapes");
-  constexpr int A_BYTES = kTcRows * KC * 2, B_BYTES = N * KC * 2, STAGE = A_BYTES + B_BYTES, kMaxStages = 16;
+                                                            int* err) {
+  static_assert((KC == 64 || (KC == 96 && !DGRAD && RES)) && (N == 32 || N == 64 || N == 128), "operand shapes");
+  constexpr int A_BYTES = kTcRows * KC * 2, B_BYTES = N * KC * 2, STAGE = A_BYTES + (RES ? 0 : B_BYTES);
+  constexpr int NC = DGRAD ? 4 : 1;  // accumulators of a tile
+  constexpr int A0 = kTcRows * 64 * 2, B0 = N * 64 * 2;  // KC = 96: tap 0 lies after taps 1 and 2
   extern __shared__ __align__(1024) unsigned char smem[];
-  __shared__ __align__(8) uint64_t full[kMaxStages], empty[kMaxStages], acc_full[2], acc_empty[2], drain;
+  __shared__ __align__(8) uint64_t s_bar[2 * STAGES + 5];
   __shared__ uint32_t s_tmem;
   __shared__ int s_abort;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;  // warp: uniform
   const uint32_t sbase = (smem_addr(smem) + 1023u) & ~1023u;  // the swizzle's period
-  unsigned char* const sgen = smem + (sbase - smem_addr(smem));
+  const uint32_t full = smem_addr(s_bar), empty = full + 8 * STAGES, acc_full = empty + 8 * STAGES;
+  const uint32_t acc_empty = acc_full + 16, drain = acc_full + 32;
   if (tid == 0) {
-    for (int s = 0; s < stages; ++s) {
-      tc_mbar_init(&full[s], 1);
-      tc_mbar_init(&empty[s], 1);
-    }
+    for (int s = 0; s < 2 * STAGES; ++s) tc_mbar_init(full + 8 * s, 1);
     for (int k = 0; k < 2; ++k) {
-      tc_mbar_init(&acc_full[k], 1);
-      tc_mbar_init(&acc_empty[k], 4);
+      tc_mbar_init(acc_full + 8 * k, 1);
+      tc_mbar_init(acc_empty + 8 * k, 4);
     }
-    tc_mbar_init(&drain, 1);
+    tc_mbar_init(drain, 1);
     s_abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 1) {  // two accumulators of N columns
+  if (warp == 1) {  // two sets of accumulators
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&s_tmem)),
-                 "r"(2 * N)
+                 "r"(2 * NC * N)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = s_tmem;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, s_tmem, 0);
   volatile int* stop = &s_abort;
-  const int all = DGRAD ? 4 * p.tiles : p.tiles;
-  // a tile's class (data gradient: 3, 2, 1, 0 in order of the taps they take) and its k-blocks
-  auto cls = [&](int t) { return DGRAD ? 3 - t / p.tiles : 0; };
-  auto blocks = [&](int c) {
-    return DGRAD ? (((c >> 1) + 1) * ((c & 1) + 1) << p.lg_c) / KC : p.k_blocks;
+  const int part = DGRAD ? blockIdx.x % p.parts : 0;  // of the layer input's channels
+  const int t0 = DGRAD ? blockIdx.x / p.parts : blockIdx.x, dt = DGRAD ? gridDim.x / p.parts : gridDim.x;
+  const int sub = DGRAD ? p.lg_c - 6 : 0, nb = DGRAD ? 4 << sub : p.k_blocks;  // k-blocks of a tile
+  // resident weights of k-block kb; the data gradient's box b has 1, 2, 2, 4 classes
+  const uint32_t wbase = sbase + STAGES * STAGE;
+  auto n_cls = [](int b) { return b == 0 ? 1 : b == 3 ? 4 : 2; };
+  auto w_at = [&](int kb) -> uint32_t {
+    if (!DGRAD) return wbase + kb * B_BYTES;
+    const int b = kb >> sub, j = kb & ((1 << sub) - 1);
+    return wbase + (((2 * b - (b > 0)) << sub) + n_cls(b) * j) * B_BYTES;
   };
 
-  if (warp == 0) {
-    if (lane == 0) {  // producer
-      int q = 0;      // k-blocks issued
-      bool ok = true;
-      for (int t = blockIdx.x; ok && t < all; t += gridDim.x) {
-        const int c = cls(t), nb = blocks(c), ntw = (c & 1) + 1;
-        const int m0 = (DGRAD ? t % p.tiles : t) * kTcRows;
-        const int y0 = (m0 >> p.lg_wo) & ((1 << p.lg_ho) - 1), n0 = m0 >> (p.lg_wo + p.lg_ho);
-        for (int kb = 0; kb < nb; ++kb, ++q) {
-          const int s = q % stages;
-          if (q >= stages && !tc_wait(&empty[s], (uint32_t)(q / stages - 1) & 1u, stop)) {
-            ok = false;
-            break;
+  if (warp == 0) {  // producer: the warp runs the loop, its elected lane issues the copies
+    const bool lead = tc_elect();
+    int s = 0, used = 0;  // the next stage, stages filled so far (up to STAGES)
+    uint32_t ph = 0;      // phase of the round over the ring
+    bool ok = true;
+    for (int t = t0; ok && t < p.tiles; t += dt) {
+      const int m0 = t * kTcRows;
+      const int y0 = (m0 >> p.lg_wo) & ((1 << p.lg_ho) - 1), n0 = m0 >> (p.lg_wo + p.lg_ho);
+      for (int kb = 0; kb < nb; ++kb) {
+        if (used == STAGES && !(ok = tc_wait(empty + 8 * s, ph ^ 1u, stop))) break;
+        if (lead) {
+          const uint32_t a = sbase + s * STAGE, bar = full + 8 * s;
+          const int box = kb >> sub, cnt = DGRAD ? n_cls(box) : 1;
+          if (RES && t == t0) {  // with the first tile its block of the weights, which stays
+            tc_expect(bar, STAGE + cnt * B_BYTES);
+            const uint32_t b = w_at(kb);
+            if (DGRAD) {
+              const int r9 = part * 9 + 2 * box - (box > 0);
+              for (int k = 0; k < cnt; ++k)
+                tc_load2(b + k * B_BYTES, &maps.b[0], (kb & ((1 << sub) - 1)) * KC, (r9 + k) * N, bar);
+            } else {
+              tc_load2(b, &maps.b[0], kb * KC + (KC == 96 ? 32 : 0), 0, bar);
+              if (KC == 96) tc_load2(b + B0, &maps.b[1], kb * KC, 0, bar);
+            }
+          } else {
+            tc_expect(bar, STAGE);
           }
-          unsigned char* a = sgen + s * STAGE;
-          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&full[s])),
-                       "r"(STAGE)
-                       : "memory");
           const int k0 = kb * KC, tap = k0 >> p.lg_c, ch = k0 & ((1 << p.lg_c) - 1);
           if (DGRAD) {
-            const int dy = (c >> 1) && tap / ntw == 0, dx = (c & 1) && tap % ntw == 0;
-            tc_load4(a, &maps.a[0], ch, dx, y0 + dy, n0, &full[s]);
-            tc_load2(a + A_BYTES, &maps.b, k0, c * N, &full[s]);
+            tc_load4(a, &maps.a[0], ch, !(tap & 1), y0 + !(tap >> 1), n0, bar);
+          } else if (KC == 96) {  // row kb of the window
+            tc_load4(a, &maps.a[2 * (kb != 1) + 1], 0, 0, y0 - (kb == 0), n0, bar);
+            tc_load4(a + A0, &maps.a[2 * (kb != 1)], 32, -1, y0 - (kb == 0), n0, bar);
           } else {
             const int kh = tap / 3, kw = tap % 3;
-            tc_load4(a, &maps.a[2 * (kh != 1) + (kw != 1)], ch, kw == 0 ? -1 : 0, y0 - (kh == 0), n0, &full[s]);
-            tc_load2(a + A_BYTES, &maps.b, k0, 0, &full[s]);
+            tc_load4(a, &maps.a[2 * (kh != 1) + (kw != 1)], ch, kw == 0 ? -1 : 0, y0 - (kh == 0), n0, bar);
           }
+          if (!RES) tc_load2(a + A_BYTES, &maps.b[0], k0, 0, bar);
+        }
+        __syncwarp();
+        if (used < STAGES) ++used;
+        if (++s == STAGES) {
+          s = 0;
+          ph ^= 1u;
         }
       }
-      // after a failure wait for the copies in flight (each stage's last one)
-      if (!ok || *stop)
-        for (int k = max(0, q - stages); k < q; ++k) tc_wait(&full[k % stages], (uint32_t)(k / stages) & 1u, nullptr);
     }
-  } else if (warp == 1) {
-    if (lane == 0) {  // MMA issuer
-      int q = 0, i = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; ok && t < all; t += gridDim.x, ++i) {
-        const int nb = blocks(cls(t)), buf = i & 1;
-        if (i >= 2 && !tc_wait(&acc_empty[buf], (uint32_t)((i >> 1) - 1) & 1u, stop)) break;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        for (int kb = 0; kb < nb; ++kb, ++q) {
-          const int s = q % stages;
-          if (!tc_wait(&full[s], (uint32_t)(q / stages) & 1u, stop)) {
-            ok = false;
-            break;
-          }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t a = sbase + (uint32_t)(s * STAGE), b = a + A_BYTES;
-#pragma unroll
-          for (int j = 0; j < KC / 16; ++j) {
-            const uint64_t ad = tc_desc<KC>(a + 32 * j), bd = tc_desc<KC>(b + 32 * j);
-            const uint32_t acc = (kb | j) != 0;
-            asm volatile(
-                "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem + (uint32_t)(buf * N)),
-                "l"(ad), "l"(bd), "r"(tc_idesc<N>()), "r"(acc)
-                : "memory");
-          }
-          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                           smem_addr(&empty[s]))
-                       : "memory");
-        }
-        if (ok)
-          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                           smem_addr(&acc_full[buf]))
-                       : "memory");
-      }
-      // every MMA issued has finished before the tensor memory is freed
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                       smem_addr(&drain))
-                   : "memory");
-      tc_wait(&drain, 0, nullptr);
-    }
-  } else if (warp >= 4) {  // epilogue: rows 32 (warp - 4) .. + 31
-    const int qd = warp - 4;
-    int i = 0;
-    for (int t = blockIdx.x; t < all; t += gridDim.x, ++i) {
-      const int c = cls(t), buf = i & 1;
-      if (!__all_sync(0xffffffffu, tc_wait(&acc_full[buf], (uint32_t)(i >> 1) & 1u, stop))) break;
+    // after a failure wait for the copies in flight (each stage's last one)
+    if (!ok || *stop)
+      for (int k = 0; k < used; ++k) tc_wait(full + 8 * k, k < s ? ph : ph ^ 1u, nullptr);
+  } else if (warp == 1) {  // MMA issuer, likewise
+    const bool lead = tc_elect();
+    int s = 0, i = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    for (int t = t0; ok && t < p.tiles; t += dt, ++i) {
+      const int buf = i & 1;
+      const uint32_t d = tmem + (uint32_t)(buf * NC * N);
+      if (i >= 2 && !tc_wait(acc_empty + 8 * buf, (uint32_t)((i >> 1) - 1) & 1u, stop)) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const int row = (DGRAD ? t % p.tiles : t) * kTcRows + 32 * qd + lane;
-      long long off;
+      for (int kb = 0; kb < nb; ++kb) {
+        if (!(ok = tc_wait(full + 8 * s, ph, stop))) break;
+        const uint32_t a = sbase + (uint32_t)(s * STAGE), b = RES ? w_at(kb) : a + A_BYTES, acc = kb != 0;
+        if (lead) {
+          if (DGRAD) {
+            // the box's classes lie side by side in the accumulator (2, 3, 1, 0) and in the
+            // weights: one MMA for all, but for the class that starts with this box
+            const int box = kb >> sub, p0 = box & 1 ? 0 : 1 - (box == 3), cnt = n_cls(box);
+            const int fresh = (kb & ((1 << sub) - 1)) == 0 ? (box == 0 ? 1 : box == 1 ? 0 : box) : -1;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const uint64_t ad = tc_desc<64>(a + 32 * j);
+              int lo = p0, hi = p0 + cnt;
+              if (j == 0 && fresh >= 0) {
+                tc_mma(d + fresh * N, ad, tc_desc<64>(b + (fresh - p0) * B_BYTES), tc_idesc(N), 0);
+                if (fresh == lo) ++lo;
+                else --hi;
+              }
+              if (lo < hi)
+                tc_mma(d + lo * N, ad, tc_desc<64>(b + (lo - p0) * B_BYTES + 32 * j), tc_idesc((hi - lo) * N), 1);
+            }
+          } else {
+            if (KC == 96)
+#pragma unroll
+              for (int j = 0; j < 2; ++j)
+                tc_mma(d, tc_desc<32>(a + A0 + 32 * j), tc_desc<32>(b + B0 + 32 * j), tc_idesc(N), j ? 1u : acc);
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              tc_mma(d, tc_desc<64>(a + 32 * j), tc_desc<64>(b + 32 * j), tc_idesc(N), j || KC == 96 ? 1u : acc);
+          }
+          tc_commit(empty + 8 * s);
+          if (kb == nb - 1) tc_commit(acc_full + 8 * buf);
+        }
+        __syncwarp();
+        if (++s == STAGES) {
+          s = 0;
+          ph ^= 1u;
+        }
+      }
+    }
+    // every MMA issued has finished before the tensor memory is freed
+    if (lead) tc_commit(drain);
+    __syncwarp();
+    tc_wait(drain, 0, nullptr);
+  } else if (warp >= 4) {  // epilogue: warps 4-7 the even tiles, 8-11 the odd ones; rows 32 (warp % 4) .. + 31
+    const int qd = warp & 3, buf = (warp - 4) >> 2;
+    // after the exchange below a lane stores 16 bytes of rows r4 .. r4 + 3
+    const int r4 = 32 * qd + (lane & ~3), q8 = 8 * (lane & 3);
+    const long long rs = DGRAD ? 2LL * p.C : p.ldc;
+    int i = buf;
+    for (int t = t0 + buf * dt; t < p.tiles; t += 2 * dt, i += 2) {
+      const int row = t * kTcRows + r4;
+      const bool in = row < p.M;
+      long long base;
       if (DGRAD) {  // class pixel -> NHWC input pixel
         const int x = row & ((1 << p.lg_wo) - 1), y = (row >> p.lg_wo) & ((1 << p.lg_ho) - 1);
         const int n = row >> (p.lg_wo + p.lg_ho);
-        off = (((long long)n * p.H + 2 * y + (c >> 1)) * p.H + 2 * x + (c & 1)) * N;
+        base = (((long long)n * p.H + 2 * y) * p.H + 2 * x) * p.C + part * N + q8;
       } else {
-        off = (long long)(row / p.grp) * p.ldg + (long long)(row % p.grp) * p.ldc;
+        base = (long long)(row / p.grp) * p.ldg + (long long)(row % p.grp) * p.ldc + q8;
       }
-      for (int c0 = 0; c0 < N; c0 += 32) {
+      // columns c0 .. c0 + 31 of the accumulators: classes 2, 3, 1, 0 (2 py + px)
+      auto offset = [&](int c0) {
+        if (!DGRAD) return base + c0;
+        const int k = c0 / N, py = k < 2, px = k == 1 || k == 2;
+        return base + (py * p.H + px) * (long long)p.C + c0 % N;
+      };
+      uint4 mk[4];  // the mask of the next 32 columns, the first ones read before the accumulator is ready
+      if (DGRAD)
+#pragma unroll
+        for (int g = 0; g < 4; ++g)
+          mk[g] = in ? __ldg(reinterpret_cast<const uint4*>(p.mask + offset(0) + g * rs)) : make_uint4(0u, 0u, 0u, 0u);
+      if (!tc_wait(acc_full + 8 * buf, (uint32_t)(i >> 1) & 1u, stop)) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      for (int c0 = 0; c0 < NC * N; c0 += 32) {
         uint32_t v[32];
         asm volatile(
             "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
@@ -532,42 +600,64 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tma(const __grid_constan
               "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]),
               "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]),
               "=r"(v[30]), "=r"(v[31])
-            : "r"(tmem + ((uint32_t)(32 * qd) << 16) + (uint32_t)(buf * N + c0)));
+            : "r"(tmem + ((uint32_t)(32 * qd) << 16) + (uint32_t)(buf * NC * N + c0)));
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        if (row < p.M) {
-          uint4* dst = reinterpret_cast<uint4*>(p.out + off + c0);
-          const uint4* msk = reinterpret_cast<const uint4*>(p.mask + off + c0);
+        uint4 o[4];  // this lane's row: 4 x 8 channels
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          uint32_t h[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            float v0 = __uint_as_float(v[8 * g + 2 * e]), v1 = __uint_as_float(v[8 * g + 2 * e + 1]);
+            if (!DGRAD) {
+              const float2 b = __ldg(reinterpret_cast<const float2*>(p.bias + c0 + 8 * g + 2 * e));
+              v0 = fmaxf(v0 + b.x, 0.0f);
+              v1 = fmaxf(v1 + b.y, 0.0f);
+            }
+            const __nv_bfloat162 w = __floats2bfloat162_rn(v0, v1);
+            h[e] = *reinterpret_cast<const uint32_t*>(&w);
+          }
+          o[g] = make_uint4(h[0], h[1], h[2], h[3]);
+        }
+        // four lanes exchange their rows' 16-byte pieces, so that a store
+        // instruction writes eight rows of 64 bytes instead of 32 of 16
+        auto swap = [&](int x, int y, int bit) {
+          const bool up = lane & bit;
+          uint4 s4 = up ? o[x] : o[y];
+          s4.x = __shfl_xor_sync(0xffffffffu, s4.x, bit);
+          s4.y = __shfl_xor_sync(0xffffffffu, s4.y, bit);
+          s4.z = __shfl_xor_sync(0xffffffffu, s4.z, bit);
+          s4.w = __shfl_xor_sync(0xffffffffu, s4.w, bit);
+          if (up) o[x] = s4;
+          else o[y] = s4;
+        };
+        swap(0, 1, 1);
+        swap(2, 3, 1);
+        swap(0, 2, 2);
+        swap(1, 3, 2);
+        if (in) {
+          bf16* dst = p.out + offset(c0);
 #pragma unroll
           for (int g = 0; g < 4; ++g) {
-            uint32_t o[4], x[4] = {0u, 0u, 0u, 0u};
-            if (DGRAD) {
-              const uint4 q4 = __ldg(&msk[g]);
-              x[0] = q4.x;
-              x[1] = q4.y;
-              x[2] = q4.z;
-              x[3] = q4.w;
-            }
+            if (DGRAD) {  // zero where the layer input is not above zero
+              const uint32_t m[4] = {mk[g].x, mk[g].y, mk[g].z, mk[g].w};
+              uint32_t w[4] = {o[g].x, o[g].y, o[g].z, o[g].w};
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              float v0 = __uint_as_float(v[8 * g + 2 * e]), v1 = __uint_as_float(v[8 * g + 2 * e + 1]);
-              if (DGRAD) {
-                const __nv_bfloat162 m2 = *reinterpret_cast<const __nv_bfloat162*>(&x[e]);
-                if (!(__low2float(m2) > 0.0f)) v0 = 0.0f;
-                if (!(__high2float(m2) > 0.0f)) v1 = 0.0f;
-              } else {
-                v0 = fmaxf(v0 + __ldg(&p.bias[c0 + 8 * g + 2 * e]), 0.0f);
-                v1 = fmaxf(v1 + __ldg(&p.bias[c0 + 8 * g + 2 * e + 1]), 0.0f);
+              for (int e = 0; e < 4; ++e) {
+                const __nv_bfloat162 m2 = *reinterpret_cast<const __nv_bfloat162*>(&m[e]);
+                if (!(__low2float(m2) > 0.0f)) w[e] &= 0xffff0000u;
+                if (!(__high2float(m2) > 0.0f)) w[e] &= 0x0000ffffu;
               }
-              const __nv_bfloat162 h = __floats2bfloat162_rn(v0, v1);
-              o[e] = *reinterpret_cast<const uint32_t*>(&h);
+              o[g] = make_uint4(w[0], w[1], w[2], w[3]);
+              if (c0 + 32 < NC * N) mk[g] = __ldg(reinterpret_cast<const uint4*>(p.mask + offset(c0 + 32) + g * rs));
             }
-            dst[g] = make_uint4(o[0], o[1], o[2], o[3]);
+            *reinterpret_cast<uint4*>(dst + g * rs) = o[g];
           }
         }
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
-      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&acc_empty[buf])) : "memory");
+      if (lane == 0) tc_arrive(acc_empty + 8 * buf);
     }
   }
   __syncwarp();
@@ -576,26 +666,22 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tma(const __grid_constan
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (tid == 0 && s_abort) atomicOr(err, 1);
   if (warp == 1)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * N) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * NC * N) : "memory");
 }
 
-// Weights of the data gradients, input channels as rows: for each class
-// (py, px) row class Cin + c, column tap Cout + o = W[o][kh][kw][c], taps in
-// the order of dg_tap, rows of 4 Cout columns (classes with fewer taps leave the
-// rest unused)
-__global__ void k_dgrad_weights(const bf16* __restrict__ w, int Kp, int cin, int cout, bf16* __restrict__ out) {
-  const int n = 4 * cin * 4 * cout;
+// Weights of the data gradients, in the order of the boxes (dy, dx) = (1, 1),
+// (1, 0), (0, 1), (0, 0) of dz and of the parity classes 2 py + px that take
+// them: 3; 2, 3; 3, 1; 2, 3, 1, 0. Row (9 part + box's class) N + c is input
+// channel part N + c, column o is W[o][kh][kw][channel]; an even coordinate
+// takes the middle tap, an odd one taps 0 (offset 1) and 2.
+__global__ void k_dgrad_weights(const bf16* __restrict__ w, int Kp, int cin, int cout, int N, bf16* __restrict__ out) {
+  const int n = 9 * cin * cout;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
-    const int k = e % (4 * cout), row = e / (4 * cout), cls = row / cin, c = row % cin, tap = k / cout, o = k % cout;
-    const int ph = cls >> 1, pw = cls & 1, ntw = pw + 1;
-    bf16 v = __float2bfloat16_rn(0.0f);
-    if (tap < (ph + 1) * ntw) {
-      int kh, kw, d;
-      dg_tap(ph, tap / ntw, kh, d);
-      dg_tap(pw, tap % ntw, kw, d);
-      v = w[(long long)o * Kp + (kh * 3 + kw) * cin + c];
-    }
-    out[e] = v;
+    const int o = e % cout, row = e / cout, c = row / (9 * N) * N + row % N, r9 = row / N % 9;
+    const int box = (r9 > 0) + (r9 > 2) + (r9 > 4), k = r9 - (2 * box - (box > 0));
+    const int cls = box == 0 ? 3 : box == 1 ? 2 + k : box == 2 ? 3 - 2 * k : k < 2 ? 2 + k : 3 - k;
+    const int kh = cls >> 1 ? (box < 2 ? 0 : 2) : 1, kw = cls & 1 ? (box & 1 ? 2 : 0) : 1;
+    out[e] = w[(long long)o * Kp + (kh * 3 + kw) * cin + c];
   }
 }
 
@@ -629,15 +715,17 @@ cudaError_t encode_map(CUtensorMap* map, const void* base, int rank, const long 
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-template <int KC, int N, bool DGRAD>
+// K: the columns of the resident weights (0: staged with A)
+template <int KC, int N, bool DGRAD, int K>
 cudaError_t conv_tma_t(const ConvMaps& maps, const ConvArgs& p, int* err, int sm_count, cudaStream_t s) {
-  constexpr int stage = (kTcRows + N) * KC * 2, stages = 200 * 1024 / stage > 12 ? 12 : 200 * 1024 / stage;
-  constexpr int smem = stages * stage + 1024;
-  auto kern = k_conv_tma<KC, N, DGRAD>;
+  constexpr int stage = (kTcRows + (K ? 0 : N)) * KC * 2, wres = N * K * 2;
+  constexpr int stages = std::min(12, (224 * 1024 - wres) / stage), smem = stages * stage + wres + 1024;
+  static_assert(stages >= 3, "ring");
+  auto kern = k_conv_tma<KC, N, DGRAD, K != 0, stages>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  const int all = (DGRAD ? 4 : 1) * p.tiles;
-  kern<<<(unsigned)std::min(all, sm_count), kTcThreads, smem, s>>>(maps, p, stages, err);
+  const int parts = DGRAD ? p.parts : 1;
+  kern<<<(unsigned)(std::min(p.tiles, sm_count / parts) * parts), kTcThreads, smem, s>>>(maps, p, err);
   return cudaGetLastError();
 }
 
@@ -1145,27 +1233,32 @@ static void conv_tile(int l, int n, ConvArgs* p, int* box) {
 // n crops are computed from what is there and not stored.
 int perch_cnn::conv_fwd(int l, const bf16* x, int n) {
   perch_cnn* net = this;
-  const int H = kHin[l], Cin = kCin[l], N = kCout[l], Kp = kp_of(l), KC = Cin >= 64 ? 64 : 32;
+  const int H = kHin[l], Cin = kCin[l], N = kCout[l], Kp = kp_of(l);
+  const bool pair = Cin == 32;  // two horizontal neighbours make a 64-channel row
   ConvArgs p{};
-  int box[4] = {KC};
+  int box[4] = {64};
   conv_tile(l, n, &p, box);
   const long long imgs = (long long)(act[l - 1].cap / (2 * (size_t)H * H * Cin));
   const bf16* w = w16.as<bf16>() + off_w[l];
   if (fwd_for[l][0] != x || fwd_for[l][1] != w || fwd_n[l] != imgs) {
-    for (int par = 0; par < 4; ++par) {
-      const long long dims[4] = {Cin, H / 2, H / 2, imgs};
-      const long long st[3] = {4LL * Cin, 4LL * H * Cin, 2LL * H * H * Cin};
-      CKN(encode_map(&fwd[l].a[par], x + ((par >> 1) * H + (par & 1)) * (long long)Cin, 4, dims, st, box), "tensor map");
+    const long long dims[4] = {pair ? 64 : Cin, H / 2, H / 2, imgs};
+    const long long st[3] = {4LL * Cin, 4LL * H * Cin, 2LL * H * H * Cin};
+    const long long wdims[2] = {Kp, N}, wst[1] = {2LL * Kp};
+    for (int k = 0; k < 4; ++k) {
+      box[0] = pair && !(k & 1) ? 32 : 64;
+      CKN(encode_map(&fwd[l].a[k], x + ((k >> 1) * H + (pair ? 0 : k & 1)) * (long long)Cin, 4, dims, st, box),
+          "tensor map");
     }
-    const long long dims[2] = {Kp, N}, st[1] = {2LL * Kp};
-    const int wbox[2] = {KC, N};
-    CKN(encode_map(&fwd[l].b, w, 2, dims, st, wbox), "tensor map");
+    for (int k = 0; k < 2; ++k) {
+      const int wbox[2] = {k ? 32 : 64, N};
+      CKN(encode_map(&fwd[l].b[k], w, 2, wdims, wst, wbox), "tensor map");
+    }
     fwd_for[l][0] = x;
     fwd_for[l][1] = w;
     fwd_n[l] = imgs;
   }
   p.lg_c = ilog2(Cin);
-  p.k_blocks = Kp / KC;
+  p.k_blocks = Kp / (pair ? 96 : 64);
   p.bias = master.as<float>() + off_b[l];
   p.ldc = N;
   p.grp = 1 << 30;
@@ -1176,9 +1269,9 @@ int perch_cnn::conv_fwd(int l, const bf16* x, int n) {
     p.ldg = Kf;
   }
   int* e = tc_err.as<int>();
-  CKN(l == 1   ? (conv_tma_t<32, 64, false>(fwd[l], p, e, sm_count, stream))
-      : l == 2 ? (conv_tma_t<64, 128, false>(fwd[l], p, e, sm_count, stream))
-               : (conv_tma_t<64, 128, false>(fwd[l], p, e, sm_count, stream)),
+  CKN(l == 1   ? (conv_tma_t<96, 64, false, 288>(fwd[l], p, e, sm_count, stream))
+      : l == 2 ? (conv_tma_t<64, 128, false, 576>(fwd[l], p, e, sm_count, stream))
+               : (conv_tma_t<64, 128, false, 0>(fwd[l], p, e, sm_count, stream)),
       "convolution");
   return PERCH_OK;
 }
@@ -1187,22 +1280,25 @@ int perch_cnn::conv_fwd(int l, const bf16* x, int n) {
 // input, times the ReLU mask of that input
 int perch_cnn::conv_dgrad(int l, const bf16* d, int n, bf16* out) {
   perch_cnn* net = this;
-  const int H = kHin[l], Ho = H / 2, N = kCin[l], Co = kCout[l];
+  const int H = kHin[l], Ho = H / 2, C = kCin[l], Co = kCout[l];
   ConvArgs p{};
   int box[4] = {64};
   conv_tile(l, n, &p, box);
-  CKN(wt[l].ensure(2 * 16 * (size_t)N * Co), "alloc");
-  k_dgrad_weights<<<grid_for(16LL * N * Co), 256, 0, stream>>>(w16.as<bf16>() + off_w[l], kp_of(l), N, Co,
-                                                               wt[l].as<bf16>());
+  p.parts = C > 64 ? 2 : 1;  // weights of 64 input channels fit beside the ring
+  const int N = C / p.parts;
+  CKN(wt[l].ensure(2 * 9 * (size_t)C * Co), "alloc");
+  k_dgrad_weights<<<grid_for(9LL * C * Co), 256, 0, stream>>>(w16.as<bf16>() + off_w[l], kp_of(l), C, Co, N,
+                                                              wt[l].as<bf16>());
   CKN(cudaGetLastError(), "data-gradient weights");
   if (dgrad_for[l][0] != d || dgrad_for[l][1] != wt[l].p || dgrad_n[l] != n) {
     const long long dims[4] = {Co, Ho, Ho, n};
     const long long st[3] = {2LL * Co, 2LL * Ho * Co, 2LL * Ho * Ho * Co};
     CKN(encode_map(&dgrad[l].a[0], d, 4, dims, st, box), "tensor map");
     for (int k = 1; k < 4; ++k) dgrad[l].a[k] = dgrad[l].a[0];
-    const long long wdims[2] = {4LL * Co, 4LL * N}, wst[1] = {8LL * Co};
+    const long long wdims[2] = {Co, 9LL * C}, wst[1] = {2LL * Co};
     const int wbox[2] = {64, N};
-    CKN(encode_map(&dgrad[l].b, wt[l].p, 2, wdims, wst, wbox), "tensor map");
+    dgrad[l].b[1] = dgrad[l].b[0];
+    CKN(encode_map(&dgrad[l].b[0], wt[l].p, 2, wdims, wst, wbox), "tensor map");
     dgrad_for[l][0] = d;
     dgrad_for[l][1] = wt[l].p;
     dgrad_n[l] = n;
@@ -1211,10 +1307,10 @@ int perch_cnn::conv_dgrad(int l, const bf16* d, int n, bf16* out) {
   p.out = out;
   p.mask = act[l - 1].as<bf16>();
   p.H = H;
+  p.C = C;
   int* e = tc_err.as<int>();
-  CKN(l == 1   ? (conv_tma_t<64, 32, true>(dgrad[l], p, e, sm_count, stream))
-      : l == 2 ? (conv_tma_t<64, 64, true>(dgrad[l], p, e, sm_count, stream))
-               : (conv_tma_t<64, 128, true>(dgrad[l], p, e, sm_count, stream)),
+  CKN(l == 1 ? (conv_tma_t<64, 32, true, 9 * 64>(dgrad[l], p, e, sm_count, stream))
+             : (conv_tma_t<64, 64, true, 9 * 128>(dgrad[l], p, e, sm_count, stream)),
       "data gradient");
   return PERCH_OK;
 }
