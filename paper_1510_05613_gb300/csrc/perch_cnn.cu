@@ -10,18 +10,16 @@
 //   -> flatten (h, w, c) ++ one-hot -> FC 96 (ReLU) -> FC 1; loss 0.5 (pred - y)^2
 //
 // Data layout: activations NHWC bfloat16. Every convolution is one GEMM over
-// rows = output pixels (N x Ho x Wo) and columns = (tap, channel): the 2-channel
-// input layer directly from a strip of the crop (k_conv1, mma.sync), the others
-// and their data gradients on tcgen05 with operands loaded by TMA
-// (k_conv_tma). Weight gradients and the FC layers use k_gemm: mma.sync
-// m16n8k16 (BF16 in, FP32 accumulate) fed by a 3-stage cp.async pipeline and
-// ldmatrix (.trans for MN-contiguous operands); the weight gradients gather
-// 16-byte chunks of the NHWC input straight into shared memory (implicit
-// im2col, zero padding through the copy's source size; the input layer's from
-// an explicit im2col), split along the pixel reduction and summed in a fixed
-// order (deterministic). Gradients between layers are rounded to bfloat16,
-// like the activations; weights keep an FP32 master copy updated by Adam and
-// re-rounded to bfloat16 after each step.
+// rows = output pixels (N x Ho x Wo) and columns = (tap, channel). The 2-channel
+// input layer works on mma.sync from strips of the crop (k_conv1, k_wgrad1); the
+// others, their data gradients (k_conv_tma) and their weight gradients
+// (k_wgrad_tma) run on tcgen05 with operands loaded by TMA. Weight gradients are
+// split along the pixel reduction and summed in a fixed order (deterministic).
+// The FC layers use k_gemm: mma.sync m16n8k16 (BF16 in, FP32 accumulate) fed by
+// a 3-stage cp.async pipeline and ldmatrix (.trans for MN-contiguous operands).
+// Gradients between layers are rounded to bfloat16, like the activations;
+// weights keep an FP32 master copy updated by Adam and re-rounded to bfloat16
+// after each step.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -65,10 +63,6 @@ struct GemmArgs {
   int M, N, K, Ksplit;  // split z covers columns [z Ksplit, min(K, (z + 1) Ksplit))
   float* Cf;  // output (partial z at Cf + z split_stride)
   long long ldc, split_stride;
-  // implicit im2col (CONV): B is the NHWC input of a 3x3 pad-1 convolution with
-  // power-of-two channels and output side; pixel index (n, i, j) and column
-  // index (tap, c), tap = 3 kh + kw
-  int cH, cs, lg_c, lg_wo;
 };
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -107,19 +101,7 @@ __device__ __forceinline__ void mma_bf16(float* c, const uint32_t* a, uint32_t b
 // weight and data gradients need no transposed copies. 256 threads; CTA tile
 // 128 x BN; warp tile (128 / (8 / (BN / 32))) x 32. K and Ksplit multiples of
 // 32; an MN-contiguous operand needs its M (or N) to be a multiple of 8.
-// Source of one 16-byte chunk of an implicit im2col operand: output pixel
-// `m`, columns k .. k + 7 (one tap, 8 channels); nullptr where the tap falls
-// in the zero padding.
-__device__ __forceinline__ const bf16* conv_src(const GemmArgs& p, const bf16* x, int m, int k) {
-  const int tap = k >> p.lg_c, c = k & ((1 << p.lg_c) - 1);
-  const int wo = 1 << p.lg_wo;
-  const int j = m & (wo - 1), i = (m >> p.lg_wo) & (wo - 1), n = m >> (2 * p.lg_wo);
-  const int r = p.cs * i - 1 + tap / 3, cc = p.cs * j - 1 + tap % 3;
-  if (tap >= 9 || r < 0 || r >= p.cH || cc < 0 || cc >= p.cH) return nullptr;
-  return x + ((((long long)n * p.cH + r) * p.cH + cc) << p.lg_c) + c;
-}
-
-template <int BN, bool AK, bool BKC, bool CONV>
+template <int BN, bool AK, bool BKC>
 __global__ void __launch_bounds__(256) k_gemm(GemmArgs p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int A_LD = AK ? LDS : BM + 8, A_STAGE = AK ? BM * LDS : BK * (BM + 8);
@@ -170,15 +152,8 @@ __global__ void __launch_bounds__(256) k_gemm(GemmArgs p) {
     } else {
       for (int c = tid; c < BK * (BN / 8); c += 256) {
         const int r = c / (BN / 8), q = c % (BN / 8), gn = n0 + q * 8;
-        bool ok = gn < p.N;
-        const bf16* src = p.B;
-        if (CONV) {
-          const bf16* g = ok ? conv_src(p, p.B, k0 + r, gn) : nullptr;
-          ok = g != nullptr;
-          if (ok) src = g;
-        } else if (ok) {
-          src = p.B + (long long)(k0 + r) * p.ldb + gn;
-        }
+        const bool ok = gn < p.N;
+        const bf16* src = ok ? p.B + (long long)(k0 + r) * p.ldb + gn : p.B;
         cp_async16(smem_addr(bs + r * B_LD + q * 8), src, ok);
       }
     }
@@ -250,27 +225,26 @@ __global__ void __launch_bounds__(256) k_gemm(GemmArgs p) {
       }
 }
 
-template <int BN, bool AK, bool BKC, bool CONV>
+template <int BN, bool AK, bool BKC>
 cudaError_t gemm_bn(const GemmArgs& p, int splits, cudaStream_t s) {
   constexpr int A_STAGE = AK ? BM * LDS : BK * (BM + 8), B_STAGE = BKC ? BN * LDS : BK * (BN + 8);
   const int smem = STAGES * (A_STAGE + B_STAGE) * (int)sizeof(bf16);
   cudaError_t e =
-      cudaFuncSetAttribute(k_gemm<BN, AK, BKC, CONV>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      cudaFuncSetAttribute(k_gemm<BN, AK, BKC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   dim3 grid((p.N + BN - 1) / BN, (p.M + BM - 1) / BM, splits);
-  k_gemm<BN, AK, BKC, CONV><<<grid, 256, smem, s>>>(p);
+  k_gemm<BN, AK, BKC><<<grid, 256, smem, s>>>(p);
   return cudaGetLastError();
 }
 
 // C = A B^T (layouts as k_gemm); `splits` CTAs along K, each writing its
 // partial at Cf + z split_stride.
-template <bool AK = true, bool BKC = true, bool CONV = false>
+template <bool AK = true, bool BKC = true>
 cudaError_t gemm(const GemmArgs& p, int splits, cudaStream_t s) {
   if ((!AK && p.M % 8) || (!BKC && p.N % 8) || p.K % 32 || p.Ksplit % 32) return cudaErrorInvalidValue;
-  if (CONV && p.lg_c < 3) return cudaErrorInvalidValue;  // chunks of 8 channels within one tap
-  if (p.N <= 32) return gemm_bn<32, AK, BKC, CONV>(p, splits, s);
-  if (p.N <= 64) return gemm_bn<64, AK, BKC, CONV>(p, splits, s);
-  return gemm_bn<128, AK, BKC, CONV>(p, splits, s);
+  if (p.N <= 32) return gemm_bn<32, AK, BKC>(p, splits, s);
+  if (p.N <= 64) return gemm_bn<64, AK, BKC>(p, splits, s);
+  return gemm_bn<128, AK, BKC>(p, splits, s);
 }
 
 // --------------------------------------- tcgen05 convolutions fed by TMA
@@ -669,6 +643,171 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tma(const __grid_constan
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * NC * N) : "memory");
 }
 
+// Weight gradients of layers 2-4: D[co][tap, ci] = sum over output pixels of
+// dz[pixel][co] x[pixel at tap][ci], both operands pixel-major (MN-major for
+// the tensor core). A CTA takes one row kh of the window (N = 3 Cin columns in
+// tensor memory, one MMA per 16 pixels, two with N = 384) and one split of the pixels;
+// its boxes are 32 output pixels of dz and, from the parity maps, of x at each tap: TMA
+// loads them with the padding, PB boxes a stage. Roles and waits as in
+// k_conv_tma; at the end warps 0-3 write the partial sums, which
+// k_split_sum_wide adds in order. Splits and the order of pixels are those of the mma.sync
+// GEMM that it replaces (implicit im2col by cp.async gathers, which bound
+// it), and so are the results, bit for bit. 256 crops: layers 2, 3, 4
+// 56 us each (mean) -> 24, 23, 19.
+struct WgradArgs {
+  int blocks, split;  // 32-pixel blocks in all and of one split
+  int lg_wo;          // output side
+  float* part;        // partial z at part + z split_stride: [co][Kp]
+  long long split_stride;
+  int Kp;
+};
+
+// shared-memory matrix descriptor of an MN-major operand: rows (K) of W
+// channels in the swizzle of their length, groups of eight rows back to back,
+// `step` bytes between blocks of W channels
+template <int W>
+__device__ __forceinline__ uint64_t tc_desc_mn(uint32_t saddr, int step) {
+  return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)(step >> 4) << 16) | ((uint64_t)(8 * 2 * W >> 4) << 32) |
+         (1ull << 46) | ((uint64_t)(W == 64 ? 2 : 4) << 61);
+}
+
+// W: channels of an x box, NB of them; MB boxes of 64 channels of dz
+template <int W, int NB, int MB, int PB, int STAGES>
+__global__ void __launch_bounds__(128) k_wgrad_tma(const __grid_constant__ ConvMaps maps, WgradArgs p, int* err) {
+  constexpr int ABOX = 32 * 64 * 2, XBOX = 32 * W * 2, N = NB * W, COLS = N <= 128 ? 128 : N <= 256 ? 256 : 512;
+  constexpr int X0 = MB * PB * ABOX, STAGE = X0 + NB * PB * XBOX, N1 = N <= 256 ? N : N / 2;
+  extern __shared__ __align__(1024) unsigned char smem[];
+  __shared__ __align__(8) uint64_t s_bar[2 * STAGES + 1];
+  __shared__ uint32_t s_tmem;
+  __shared__ int s_abort;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  const uint32_t sbase = (smem_addr(smem) + 1023u) & ~1023u;
+  const uint32_t full = smem_addr(s_bar), empty = full + 8 * STAGES, acc_full = empty + 8 * STAGES;
+  if (tid == 0) {
+    for (int s = 0; s < 2 * STAGES + 1; ++s) tc_mbar_init(full + 8 * s, 1);
+    s_abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&s_tmem)),
+                 "r"(COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = __shfl_sync(0xffffffffu, s_tmem, 0);
+  volatile int* stop = &s_abort;
+  const int kh = blockIdx.x, b0 = blockIdx.y * p.split, nblk = min(p.blocks - b0, p.split);
+  const int rounds = (nblk + PB - 1) / PB;
+
+  if (warp == 0) {  // producer
+    const bool lead = tc_elect();
+    int s = 0, used = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    for (int r = 0; r < rounds; ++r) {
+      if (used == STAGES && !(ok = tc_wait(empty + 8 * s, ph ^ 1u, stop))) break;
+      if (lead) {
+        const int cnt = min(PB, nblk - r * PB);
+        const uint32_t a = sbase + s * STAGE, bar = full + 8 * s;
+        tc_expect(bar, cnt * (STAGE / PB));
+        for (int h = 0; h < cnt; ++h) {
+          const int m = (b0 + r * PB + h) * 32, y = (m >> p.lg_wo) & ((1 << p.lg_wo) - 1), n = m >> (2 * p.lg_wo);
+#pragma unroll
+          for (int k = 0; k < MB; ++k) tc_load4(a + (k * PB + h) * ABOX, &maps.b[0], 64 * k, 0, y, n, bar);
+#pragma unroll
+          for (int k = 0; k < NB; ++k) {
+            const int kw = k / (NB / 3), ch = k % (NB / 3) * W;
+            tc_load4(a + X0 + (k * PB + h) * XBOX, &maps.a[2 * (kh != 1) + (kw != 1)], ch, kw == 0 ? -1 : 0,
+                     y - (kh == 0), n, bar);
+          }
+        }
+      }
+      __syncwarp();
+      if (used < STAGES) ++used;
+      if (++s == STAGES) {
+        s = 0;
+        ph ^= 1u;
+      }
+    }
+    if (!ok || *stop)  // after a failure wait for the copies in flight
+      for (int k = 0; k < used; ++k) tc_wait(full + 8 * k, k < s ? ph : ph ^ 1u, nullptr);
+  } else if (warp == 1) {  // MMA issuer
+    const bool lead = tc_elect();
+    // M = 64 MB, both operands MN-major
+    const uint32_t idesc =
+        (1u << 4) | (1u << 7) | (1u << 10) | (3u << 15) | ((uint32_t)(N1 >> 3) << 17) | ((uint32_t)(4 * MB) << 24);
+    int s = 0;
+    uint32_t ph = 0;
+    for (int r = 0; r < rounds; ++r) {
+      if (!tc_wait(full + 8 * s, ph, stop)) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      if (lead) {
+        const uint32_t a = sbase + s * STAGE, x = a + X0;
+        const int steps = 2 * min(PB, nblk - r * PB);
+#pragma unroll
+        for (int j = 0; j < 2 * PB; ++j)
+          if (j < steps)
+#pragma unroll
+            for (int h = 0; h < N / N1; ++h)
+              tc_mma(tmem + h * N1, tc_desc_mn<64>(a + j * 2048, PB * ABOX),
+                     tc_desc_mn<W>(x + j * 32 * W + h * (NB / 2) * PB * XBOX, PB * XBOX), idesc, r > 0 || j > 0);
+        tc_commit(empty + 8 * s);
+      }
+      __syncwarp();
+      if (++s == STAGES) {
+        s = 0;
+        ph ^= 1u;
+      }
+    }
+    if (lead) tc_commit(acc_full);  // also after a failure: every MMA issued ends before the memory is freed
+    __syncwarp();
+    tc_wait(acc_full, 0, nullptr);
+  }
+  __syncwarp();
+  if (tc_wait(acc_full, 0, stop)) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    // with M = 64 a warp's first 16 lanes hold its rows
+    const int row = MB == 2 ? tid : 16 * warp + lane;
+    float* out = p.part + blockIdx.y * p.split_stride + (long long)row * p.Kp + kh * N;
+    for (int c0 = 0; c0 < N; c0 += 32) {
+      uint32_t v[32];
+      asm volatile(
+          "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
+          "%14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+          : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+            "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
+            "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
+            "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+          : "r"(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)c0));
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      if (MB == 2 || lane < 16)
+#pragma unroll
+        for (int g = 0; g < 8; ++g)
+          *reinterpret_cast<uint4*>(out + c0 + 4 * g) = make_uint4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
+    }
+  }
+  __syncwarp();
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if (tid == 0 && s_abort) atomicOr(err, 1);
+  if (warp == 1)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(COLS) : "memory");
+}
+
+template <int W, int NB, int MB, int PB, int STAGES>
+cudaError_t wgrad_tma_t(const ConvMaps& maps, const WgradArgs& p, int splits, int* err, cudaStream_t s) {
+  constexpr int smem = STAGES * PB * 64 * (64 * MB + NB * W) + 1024;
+  auto kern = k_wgrad_tma<W, NB, MB, PB, STAGES>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  kern<<<dim3(3, (unsigned)splits), 128, smem, s>>>(maps, p, err);
+  return cudaGetLastError();
+}
+
 // Weights of the data gradients, in the order of the boxes (dy, dx) = (1, 1),
 // (1, 0), (0, 1), (0, 0) of dz and of the parity classes 2 py + px that take
 // them: 3; 2, 3; 3, 1; 2, 3, 1, 0. Row (9 part + box's class) N + c is input
@@ -733,13 +872,6 @@ int ilog2(int v) {
   int l = 0;
   while ((1 << l) < v) ++l;
   return l;
-}
-
-void set_conv(GemmArgs& p, int l) {
-  p.cH = kHin[l];
-  p.cs = kStride[l];
-  p.lg_c = ilog2(kCin[l]);
-  p.lg_wo = ilog2(kHin[l] / kStride[l]);
 }
 
 // splits along K so that the grid has about two CTAs per SM (each split a
@@ -813,28 +945,76 @@ __global__ void __launch_bounds__(256) k_conv1(const uint32_t* __restrict__ x, c
   }
 }
 
-// ---------------------------------------------------------------- layout kernels
-// im2col of the 2-channel input layer (stride 1, Kp = 32): one thread per
-// output pixel gathers its 9 taps (4 bytes each) and writes one 64-byte row
-__global__ void k_im2col_c2(const uint32_t* __restrict__ x, int N, int H, int W, uint4* __restrict__ col) {
-  const long long total = (long long)N * H * W;
-  for (long long m = blockIdx.x * (long long)blockDim.x + threadIdx.x; m < total;
-       m += (long long)gridDim.x * blockDim.x) {
-    const int j = (int)(m % W), i = (int)((m / W) % H);
-    const long long n = m / ((long long)W * H);
-    uint32_t v[16];
-#pragma unroll
-    for (int t = 0; t < 16; ++t) v[t] = 0u;
-#pragma unroll
-    for (int tap = 0; tap < 9; ++tap) {
-      const int r = i - 1 + tap / 3, c = j - 1 + tap % 3;
-      if (r >= 0 && r < H && c >= 0 && c < W) v[tap] = x[(n * H + r) * W + c];
+// Weight gradient of the input layer: D[co][tap, channel] = sum over pixels of
+// dz[pixel][co] x[pixel at tap][channel], one split of the pixels a CTA. dz rows
+// pass once through a cp.async ring; a B fragment of mma.sync is two
+// neighbouring pixels of the crop at a tap, put together from the CTA's strip of
+// crop rows in shared memory (rows outside the image: a row of zeros). Warps
+// 0-5 hold 16 x 8 outputs each (18 of 32 columns exist). Bound by
+// reading dz (67 MB per 256 crops); splits and order of pixels are
+// those of the GEMM over an im2col matrix that it replaces, and so are the
+// results, bit for bit. 256 crops: 31 us instead of 81 (im2col 20, GEMM 61).
+constexpr int kW1Px = 128, kW1Ld = 80, kW1Stages = 7, kW1Row = kCrop + 2;
+__global__ void __launch_bounds__(256) k_wgrad1(const uint32_t* __restrict__ x, const bf16* __restrict__ dz, int M,
+                                                int ksplit, float* __restrict__ part) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  uint32_t* strip = reinterpret_cast<uint32_t*>(smem_raw + kW1Stages * kW1Px * kW1Ld);  // row 0: zeros
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  const int kbeg = blockIdx.x * ksplit, kend = min(M, kbeg + ksplit);
+  const int R0 = kbeg / kCrop - 1, nrows = (kend - 1) / kCrop + 1 - R0 + 1, rounds = (kend - kbeg + kW1Px - 1) / kW1Px;
+  auto load = [&](int st) {
+    const int m0 = kbeg + st * kW1Px;
+    const uint32_t dst = smem_addr(smem_raw + (st % kW1Stages) * kW1Px * kW1Ld);
+    for (int c = tid; c < kW1Px * 4; c += 256) {
+      const int m = m0 + (c >> 2);
+      cp_async16(dst + (c >> 2) * kW1Ld + (c & 3) * 16, dz + (long long)min(m, kend - 1) * 32 + (c & 3) * 8, m < kend);
     }
+  };
 #pragma unroll
-    for (int q = 0; q < 4; ++q) col[m * 4 + q] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+  for (int st = 0; st < kW1Stages - 1; ++st) {
+    if (st < rounds) load(st);
+    cp_commit();
   }
+  for (int i = tid; i < (nrows + 1) * kW1Row; i += 256) {
+    const int r = R0 + i / kW1Row - 1, c = i % kW1Row - 1;
+    const bool in = i >= kW1Row && r >= 0 && r < M / kCrop && c >= 0 && c < kCrop;
+    strip[i] = in ? __ldg(&x[(long long)r * kCrop + c]) : 0u;
+  }
+  const int mt = warp < 6 ? warp / 3 : warp - 6, nt = warp < 6 ? warp % 3 : 3;
+  const int col = 8 * nt + g, tap = col >> 1, kh = tap / 3, kw = tap % 3;
+  const uint32_t sel = col & 1 ? 0x7632u : 0x5410u;
+  float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  for (int st = 0; st < rounds; ++st) {
+    cp_wait<kW1Stages - 2>();
+    __syncthreads();  // stage st landed for every thread; stage st - 1 is free
+    if (st + kW1Stages - 1 < rounds) load(st + kW1Stages - 1);
+    cp_commit();
+    if (warp >= 6) continue;
+    const int m0 = kbeg + st * kW1Px;
+    const uint32_t a0 = smem_addr(smem_raw + (st % kW1Stages) * kW1Px * kW1Ld) +
+                        (8 * (lane >> 4) + (lane & 7)) * kW1Ld + (16 * mt + 8 * ((lane >> 3) & 1)) * 2;
+#pragma unroll
+    for (int h = 0; h < kW1Px / 32; ++h) {
+      const int m = m0 + 32 * h, R = m / kCrop, i = R % kCrop - 1 + kh;
+      if (m >= kend) break;
+      const bool in = col < 18 && i >= 0 && i < kCrop;
+      const uint32_t* row = strip + (in ? (R - 1 + kh - R0 + 1) * kW1Row + m % kCrop + kw : 0) + 2 * t;
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        uint32_t af[4];
+        ldsm_x4_t(a0 + (32 * h + 16 * k) * kW1Ld, af[0], af[1], af[2], af[3]);
+        mma_bf16(acc, af, __byte_perm(row[16 * k], row[16 * k + 1], sel),
+                 __byte_perm(row[16 * k + 8], row[16 * k + 9], sel));
+      }
+    }
+  }
+  cp_wait<0>();
+  float* out = part + (long long)blockIdx.x * 32 * 32 + (16 * mt + g) * 32 + 8 * nt + 2 * t;
+  *reinterpret_cast<float2*>(out) = make_float2(acc[0], acc[1]);
+  *reinterpret_cast<float2*>(out + 8 * 32) = make_float2(acc[2], acc[3]);
 }
 
+// ---------------------------------------------------------------- small kernels
 // part[b][c] = sum of column c over rows [b R, (b + 1) R) of a bfloat16
 // [M][C] matrix (bias gradients); 256 threads, 256 / C row groups.
 __global__ void k_col_sum(const bf16* __restrict__ in, long long M, int C, int R, float* __restrict__ part) {
@@ -1089,7 +1269,7 @@ struct perch_cnn {
   long long off_w[kConvs], off_f1, n_w16, off_b[kConvs], off_fb1, off_f2, off_fb2, n_total;
   DevBuf master, grad, adam_m, adam_v, w16;
   // batch buffers
-  DevBuf col[kConvs], act[kConvs], feat, h1, err_buf, pred_buf, loss_buf;
+  DevBuf act[kConvs], feat, h1, err_buf, pred_buf, loss_buf;
   DevBuf dz1, dfeat, dz, dcol, part, bpart;
   bool params_set = false;
   // tc_err: the convolution kernels' wait-gave-up flag (device int); path: the
@@ -1097,12 +1277,14 @@ struct perch_cnn {
   int path = 0;
   int sm_count = 152;
   DevBuf tc_err;
-  // tensor maps of the convolutions' operands (forward, data gradient), and
+  // tensor maps of the convolutions' operands (forward, data and
+  // weight gradient), and
   // the buffers they were made for
-  ConvMaps fwd[kConvs], dgrad[kConvs];
+  ConvMaps fwd[kConvs], dgrad[kConvs], wgrad[kConvs];
   const void* fwd_for[kConvs][2] = {};
   const void* dgrad_for[kConvs][2] = {};
-  long long fwd_n[kConvs] = {}, dgrad_n[kConvs] = {};
+  const void* wgrad_for[kConvs][2] = {};
+  long long fwd_n[kConvs] = {}, dgrad_n[kConvs] = {}, wgrad_n[kConvs] = {};
   DevBuf wt[kConvs];  // weights of the data gradients (k_dgrad_weights)
 
   int fail(int code, const char* fmt, ...) {
@@ -1124,7 +1306,6 @@ struct perch_cnn {
     std::vector<DevBuf*> v = {&master, &grad, &adam_m, &adam_v, &w16, &feat, &h1, &err_buf, &pred_buf,
                               &loss_buf, &dz1, &dfeat, &dz, &dcol, &part, &bpart, &tc_err};
     for (int l = 0; l < kConvs; ++l) {
-      v.push_back(&col[l]);
       v.push_back(&act[l]);
       v.push_back(&wt[l]);
     }
@@ -1176,6 +1357,7 @@ struct perch_cnn {
   int refresh_weights();
   int conv_fwd(int l, const bf16* x, int n);
   int conv_dgrad(int l, const bf16* dz, int n, bf16* out);
+  int conv_wgrad(int l, const bf16* dz, int n, int splits, int ksplit);
   int forward(const bf16* crops, const int32_t* onehot, int n, float* pred, const float* target);
   int backward(const bf16* crops, int n);
 };
@@ -1315,6 +1497,38 @@ int perch_cnn::conv_dgrad(int l, const bf16* d, int n, bf16* out) {
   return PERCH_OK;
 }
 
+// Partial weight gradients of layer l = 1 .. 3 (k_split_sum_wide adds them)
+int perch_cnn::conv_wgrad(int l, const bf16* d, int n, int splits, int ksplit) {
+  perch_cnn* net = this;
+  const int H = kHin[l], Ho = H / 2, C = kCin[l], Co = kCout[l], W = std::min(C, 64);
+  const bf16* x = act[l - 1].as<bf16>();
+  if (wgrad_for[l][0] != d || wgrad_for[l][1] != x || wgrad_n[l] != n) {
+    const int xbox[4] = {W, Ho, 32 / Ho, 1}, dbox[4] = {64, Ho, 32 / Ho, 1};
+    const long long xdims[4] = {C, Ho, Ho, n}, xst[3] = {4LL * C, 4LL * H * C, 2LL * H * H * C};
+    for (int k = 0; k < 4; ++k)
+      CKN(encode_map(&wgrad[l].a[k], x + ((k >> 1) * H + (k & 1)) * (long long)C, 4, xdims, xst, xbox), "tensor map");
+    const long long ddims[4] = {Co, Ho, Ho, n}, dst[3] = {2LL * Co, 2LL * Ho * Co, 2LL * Ho * Ho * Co};
+    CKN(encode_map(&wgrad[l].b[0], d, 4, ddims, dst, dbox), "tensor map");
+    wgrad[l].b[1] = wgrad[l].b[0];
+    wgrad_for[l][0] = d;
+    wgrad_for[l][1] = x;
+    wgrad_n[l] = n;
+  }
+  WgradArgs p{};
+  p.blocks = n * Ho * Ho / 32;
+  p.split = ksplit / 32;
+  p.lg_wo = ilog2(Ho);
+  p.part = part.as<float>();
+  p.Kp = kp_of(l);
+  p.split_stride = (long long)Co * p.Kp;
+  int* e = tc_err.as<int>();
+  CKN(l == 1   ? (wgrad_tma_t<32, 3, 1, 2, 3>(wgrad[l], p, splits, e, stream))
+      : l == 2 ? (wgrad_tma_t<64, 3, 2, 1, 5>(wgrad[l], p, splits, e, stream))
+               : (wgrad_tma_t<64, 6, 2, 1, 6>(wgrad[l], p, splits, e, stream)),
+      "weight gradient");
+  return PERCH_OK;
+}
+
 // Forward pass of n <= max_batch crops; with a target also the per-sample
 // errors (for the backward pass).
 int perch_cnn::forward(const bf16* crops, const int32_t* onehot, int n, float* pred, const float* target) {
@@ -1362,7 +1576,7 @@ int perch_cnn::backward(const bf16* crops, int n) {
   long long max_mk = 0, max_part = 0, max_bpart = 0;
   for (int l = 0; l < kConvs; ++l) {
     const long long Ho = kHin[l] / kStride[l], M = N * Ho * Ho;
-    max_mk = std::max(max_mk, M * std::max(kp_of(l), kCout[l]));
+    max_mk = std::max(max_mk, M * kCout[l]);
     int ks;
     const int S = choose_splits(kCout[l], kp_of(l), (int)M, &ks);
     max_part = std::max(max_part, (long long)S * kCout[l] * kp_of(l));
@@ -1423,34 +1637,19 @@ int perch_cnn::backward(const bf16* crops, int n) {
                                                              cur);
   CKN(cudaGetLastError(), "relu gradient kernel");
   for (int l = kConvs - 1; l >= 0; --l) {
-    const int H = kHin[l], s = kStride[l], Ho = H / s, Kp = kp_of(l), Co = kCout[l];
+    const int Ho = kHin[l] / kStride[l], Kp = kp_of(l), Co = kCout[l];
     const long long M = N * Ho * Ho;
     if (int rc = bias_grad(cur, M, Co, G + off_b[l])) return rc;
-    // dW = dz^T col: both operands pixel-major, split along the pixel reduction,
-    // partials summed in order
-    {
-      GemmArgs p{};
-      p.A = cur;
-      p.lda = Co;
-      p.M = Co;
-      p.N = Kp;
-      p.K = (int)M;
-      const int S = choose_splits(Co, Kp, (int)M, &p.Ksplit);
-      p.Cf = part.as<float>();
-      p.ldc = Kp;
-      p.split_stride = (long long)Co * Kp;
+    {  // dW, split along the pixel reduction, partials summed in order
+      int ks;
+      const int S = choose_splits(Co, Kp, (int)M, &ks);
       if (l == 0) {
-        CKN(col[0].ensure(2 * M * Kp), "alloc im2col");
-        k_im2col_c2<<<grid_for(M), 256, 0, stream>>>(reinterpret_cast<const uint32_t*>(crops), n, H, H,
-                                                     col[0].as<uint4>());
-        CKN(cudaGetLastError(), "im2col kernel");
-        p.B = col[0].as<bf16>();
-        p.ldb = Kp;
-        CKN((gemm<false, false>(p, S, stream)), "conv weight-gradient gemm");
-      } else {  // implicit im2col of this layer's input
-        p.B = act[l - 1].as<bf16>();
-        set_conv(p, l);
-        CKN((gemm<false, false, true>(p, S, stream)), "conv weight-gradient gemm");
+        const int smem = kW1Stages * kW1Px * kW1Ld + (ks / kCrop + 5) * kW1Row * 4;
+        CKN(cudaFuncSetAttribute(k_wgrad1, cudaFuncAttributeMaxDynamicSharedMemorySize, smem), "weight gradient");
+        k_wgrad1<<<S, 256, smem, stream>>>(reinterpret_cast<const uint32_t*>(crops), cur, (int)M, ks, part.as<float>());
+        CKN(cudaGetLastError(), "weight gradient");
+      } else if (int rc = conv_wgrad(l, cur, n, S, ks)) {
+        return rc;
       }
       k_split_sum_wide<<<(unsigned)((Co * Kp + 31) / 32), 256, 0, stream>>>(part.as<float>(), S,
                                                                              (long long)Co * Kp, G + off_w[l]);

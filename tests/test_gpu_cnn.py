@@ -228,3 +228,29 @@ def test_forward_does_not_depend_on_the_chunks(c1, n):
         assert one.cpu().numpy()[0] == ref[n // 2]
         assert net.perch_cnn_tensor_status() == (0, 0)
         net.close()
+
+
+@pytest.mark.parametrize("n", [32, 96, 160])
+def test_gradients_add_up_over_the_batch(c1, n):
+    """Gradients of n crops against the mean of the gradients of their groups of
+    32 (other tiles, splits and split lengths). Both sides carry the rounding of gradients
+    between layers (2^-9 relative to the error over n, which rounds alike up to the exact
+    factor n / 32 only when that is a power of two) and of FP32 sums; per
+    tensor the difference stays within 2^-8 of the gradient's norm."""
+    wl, p, w = c1
+    n_onehot = len(wl.meshes) * wl.grid.n_yaw
+    crops, onehot = p.perch_cnn_crops([wl.gt[:1]], np.zeros(n, np.int32), _hyps_c1(wl, n, 21 + n))
+    params = _params(n_onehot, 22)
+    target = torch.tensor(np.random.default_rng(23).uniform(0.0, 4.0, n), dtype=torch.float32, device="cuda")
+    net = _net_with(params, n_onehot, max_batch=160)
+    g, loss, _ = net.perch_cnn_gradients(crops, onehot, target)
+    parts = [net.perch_cnn_gradients(crops[k:k + 32].contiguous(), onehot[k:k + 32].contiguous(),
+                                     target[k:k + 32].contiguous()) for k in range(0, n, 32)]
+    mean = np.mean([q[0].astype(np.float64) for q in parts], axis=0)
+    assert abs(loss - np.mean([q[1] for q in parts])) <= 1e-5 * loss
+    off = 0
+    for a in params:
+        d = g[off:off + a.size] - mean[off:off + a.size]
+        assert np.linalg.norm(d) <= 2.0 ** -8 * np.linalg.norm(mean[off:off + a.size]) + 1e-30, (off, a.shape)
+        off += a.size
+    assert net.perch_cnn_tensor_status() == (0, 0)
