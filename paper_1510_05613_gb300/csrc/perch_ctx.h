@@ -89,6 +89,7 @@ struct perch_ctx {
   bool tables_valid = false;
   int tile_w = 0, tile_h = 0;             // largest over all meshes
   std::vector<int> mesh_tile_w, mesh_tile_h;  // per mesh
+  std::vector<int> mesh_order;            // meshes by falling triangle count, the order of their launches
   std::vector<int> mesh_threads;          // CTA width per mesh (autotuned; 256 by default)
   int sm_count = 0;
 
@@ -167,6 +168,12 @@ struct perch_ctx {
   static constexpr int kEvents = 5;
   cudaEvent_t ev[kEvents] = {nullptr, nullptr, nullptr, nullptr, nullptr};
   bool timed = false;
+
+  // side streams on which the launches of a phase's meshes run beside the
+  // context's stream, and the events that fork and join them
+  static constexpr int kSide = 3;
+  cudaStream_t side[kSide] = {};
+  cudaEvent_t fork = nullptr, join[kSide] = {};
 
   std::vector<DevBuf*> all_buffers() {
     return {&meshes, &chunk_verts, &chunk_info, &chunk_tris, &vol_normals, &yaw_mats, &pose_off, &vtab, &xs, &ys, &cs, &depth, &rx, &ry, &blockcnt, &blockoff,
