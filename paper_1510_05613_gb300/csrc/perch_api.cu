@@ -190,7 +190,7 @@ int perch_ctx::ensure_tile_store() {
   if (P > (1LL << 28) || bound >= (1LL << 31)) return PERCH_OK;
   CK(tile_sizes.ensure(4 * (size_t)P), "alloc tile sizes");
   CK(tile_off.ensure(4 * ((size_t)P + 1)), "alloc tile offsets");
-  CK(pg_tmp.ensure(4 * ((size_t)P / 1024 + 2)), "alloc");
+  CK(pg_tmp.ensure(8 * ((size_t)P / 1024 + 2)), "alloc");
   CK(pose_flags.ensure((size_t)P), "alloc pose flags");
   CK(tile_box.ensure(16 * (size_t)P), "alloc stored boxes");
   CK(pose_valid.ensure(4 * (size_t)P), "alloc render cache tags");
@@ -885,15 +885,13 @@ int perch_ctx::enqueue_eval(const perch_obj* d_parents, int parent_stride, const
     const int per_mesh = nx * ny * n_yaw, P = per_mesh * n_mesh;
     CK(pg_cnt.ensure(4 * (size_t)P), "alloc");
     CK(pg_start.ensure(4 * ((size_t)P + 1)), "alloc");
-    CK(pg_flag.ensure(4 * (size_t)P), "alloc");
-    CK(pg_gix.ensure(4 * ((size_t)P + 1)), "alloc");
     CK(pg_gpose.ensure(4 * (size_t)P), "alloc");
-    CK(pg_tmp.ensure(4 * ((size_t)P / 1024 + 2)), "alloc");
-    CK(pg_ranges.ensure(16 * (size_t)n_mesh), "alloc");
+    CK(pg_tmp.ensure(8 * ((size_t)P / 1024 + 2)), "alloc");
+    CK(pg_ranges.ensure(16 * ((size_t)n_mesh + 1)), "alloc");
     CK(g_order.ensure(sizeof(int) * (size_t)std::max(n_hyp, 1LL)), "alloc");
     CK(g_next.ensure(sizeof(int) * 2 * (size_t)n_mesh), "alloc");
-    PoseGroups pg{pg_cnt.as<int>(),   pg_start.as<int>(), pg_flag.as<int>(),   pg_gix.as<int>(),
-                  pg_gpose.as<int>(), pg_tmp.as<int>(),   pg_ranges.as<int>(), g_order.as<int>()};
+    PoseGroups pg{pg_cnt.as<int>(), pg_start.as<int>(), pg_gpose.as<int>(), pg_tmp.as<unsigned long long>(),
+                  pg_ranges.as<int>(), g_order.as<int>()};
     const uint32_t tag = 2u * render_epoch + (b.parent_scene ? 0u : 1u);
     uint32_t* valid = cache ? pose_valid.as<uint32_t>() : nullptr;
     CK(launch_group_by_pose(g, b, pg, valid, tag, stream), "group by pose");

@@ -104,7 +104,7 @@ struct perch_ctx {
   bool share_renders = true;
   bool store_ok = false;
   DevBuf tile_store, tile_off, tile_sizes, pose_flags, tile_box;
-  DevBuf pg_cnt, pg_start, pg_flag, pg_gix, pg_gpose, pg_tmp, pg_ranges;  // hypotheses grouped by pose
+  DevBuf pg_cnt, pg_start, pg_gpose, pg_tmp, pg_ranges;  // hypotheses grouped by pose
   std::vector<int> mesh_cost_threads;  // CTA width of k_cost per mesh (autotuned; 128 by default)
   std::vector<int> mesh_cost_stages;   // stage buffers of k_cost per mesh (1 or 2; autotuned; 1 by default)
   std::vector<int> mesh_inline;        // k_render's inline limit per mesh (autotuned; 16 by default)
@@ -181,7 +181,7 @@ struct perch_ctx {
             &scratch_small, &pose_bbox, &pose_general, &parent_z, &uset, &uset_count, &b_parents, &b_plen, &b_hp, &b_hyp,
             &b_out, &g_hist, &g_off, &g_cursor, &g_order, &g_next, &net_crops, &net_onehot, &net_pred,
             &solo, &solo_rec, &solo_hyp, &solo_hp, &solo_parent, &ptile_counts, &ptile_sat, &skip, &n_short,
-            &tile_store, &tile_off, &tile_sizes, &pose_flags, &pg_cnt, &pg_start, &pg_flag, &pg_gix, &pg_gpose,
+            &tile_store, &tile_off, &tile_sizes, &pose_flags, &pg_cnt, &pg_start, &pg_gpose,
             &pg_tmp, &pg_ranges, &pose_valid, &tile_box, &icp_src, &icp_pts, &icp_start, &icp_next,
             &icp_out, &icp_model, &icp_img_pts, &icp_img_lo, &icp_img_hi};
   }

@@ -167,12 +167,10 @@ struct CostWork {
 // Hypotheses grouped by pose; P = n_mesh x nx x ny x n_yaw. All device arrays.
 struct PoseGroups {
   int* cnt;     // P: hypotheses per pose (zero again after the grouping)
-  int* start;   // P + 1: exclusive scan of cnt
-  int* flag;    // P: cnt > 0
-  int* gix;     // P + 1: exclusive scan of flag
+  int* start;   // P: exclusive scan of cnt
   int* gpose;   // P: the distinct poses, in pose order
-  int* tmp;     // P / 1024 + 2: scan scratch
-  int* ranges;  // 4 per mesh: first hypothesis in order, hypotheses, first entry of gpose, entries
+  unsigned long long* tmp;  // min(P / 1024 + 1, 2048): scan scratch
+  int* ranges;  // 4 per mesh and 4 more: first hypothesis in order, hypotheses, first entry of gpose, entries
   int* order;   // n_hyp: hypotheses sorted by pose
 };
 

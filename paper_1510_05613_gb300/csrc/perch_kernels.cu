@@ -279,74 +279,100 @@ cudaError_t launch_fill_u32(uint32_t* p, uint32_t v, long long n, cudaStream_t s
   return cudaGetLastError();
 }
 
-// exclusive scan: out[0..n] with out[n] = total. 1024 elements per block.
-__global__ void k_scan_blocks(const int* in, int* out, int n, int* block_sums) {
-  __shared__ int warp_tot[8];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int base = blockIdx.x * 1024 + tid * 4;
-  int v[4], s = 0;
+// Exclusive scans in two launches (one for a single block): the sums of the
+// blocks' ranges, then each block adds the sums before its own and scans its
+// range. At most 2048 blocks, of 1024 elements or a multiple. F gives the elements
+// and takes each with its prefix: f.load(i), f.store(i, prefix, element),
+// f.total(sum). A scan of 120k elements takes
+// 3 + 4 us; three launches (block scans, their sums, the sums added) took 3 + 3 + 4.
+constexpr int kScanBlocks = 2048;
+
+template <typename F>
+__device__ __forceinline__ typename F::T scan_thread(const F& f, long long base, int n, typename F::T (&v)[4]) {
+  typename F::T s = 0;
+#pragma unroll
   for (int k = 0; k < 4; ++k) {
-    v[k] = (base + k < n) ? in[base + k] : 0;
+    v[k] = base + k < n ? f.load((int)(base + k)) : 0;
     s += v[k];
   }
-  int incl = s;
+  return s;
+}
+// inclusive scan over the block's 256 threads; every thread gets the block's sum
+template <typename T>
+__device__ __forceinline__ T scan_256(T v, T& sum) {
+  __shared__ T warp_tot[8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int d = 1; d < 32; d <<= 1) {
-    int t = __shfl_up_sync(0xffffffffu, incl, d);
-    if (lane >= d) incl += t;
+    const T t = __shfl_up_sync(0xffffffffu, v, d);
+    if (lane >= d) v += t;
   }
-  if (lane == 31) warp_tot[warp] = incl;
   __syncthreads();
-  int woff = 0;
-  for (int w = 0; w < warp; ++w) woff += warp_tot[w];
-  int run = woff + incl - s;
-  for (int k = 0; k < 4; ++k) {
-    if (base + k < n) out[base + k] = run;
-    run += v[k];
+  if (lane == 31) warp_tot[warp] = v;
+  __syncthreads();
+  sum = 0;
+  T before = 0;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) {
+    if (w == warp) before = sum;
+    sum += warp_tot[w];
   }
-  if (tid == 255) block_sums[blockIdx.x] = woff + incl;
+  return v + before;
 }
 
-__global__ void k_scan_single(int* sums, int nb, int* total_out) {
-  __shared__ int carry_s;
-  __shared__ int warp_tot[32];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) carry_s = 0;
-  __syncthreads();
-  for (int off = 0; off < nb; off += 1024) {
-    int i = off + tid;
-    int v = (i < nb) ? sums[i] : 0;
-    int incl = v;
-    for (int d = 1; d < 32; d <<= 1) {
-      int t = __shfl_up_sync(0xffffffffu, incl, d);
-      if (lane >= d) incl += t;
+template <typename F>
+__global__ void __launch_bounds__(256) k_scan_sums(F f, int n, long long per, typename F::T* sums) {
+  typename F::T a = 0, v[4], sum;
+  for (long long b = blockIdx.x * per; b < (blockIdx.x + 1) * per; b += 1024)
+    a += scan_thread(f, b + 4 * threadIdx.x, n, v);
+  scan_256(a, sum);
+  if (threadIdx.x == 0) sums[blockIdx.x] = sum;
+}
+
+template <typename F>
+__global__ void __launch_bounds__(256) k_scan_out(F f, int n, long long per, const typename F::T* sums) {
+  typename F::T a = 0, v[4], carry, sum;
+  for (int k = threadIdx.x; k < (int)blockIdx.x; k += 256) a += sums[k];
+  scan_256(a, carry);
+  for (long long b = blockIdx.x * per; b < (blockIdx.x + 1) * per; b += 1024) {
+    const long long base = b + 4 * threadIdx.x;
+    const typename F::T s = scan_thread(f, base, n, v);
+    typename F::T run = carry + scan_256(s, sum) - s;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (base + k < n) f.store((int)(base + k), run, v[k]);
+      run += v[k];
     }
-    if (lane == 31) warp_tot[warp] = incl;
-    __syncthreads();
-    int woff = 0;
-    for (int w = 0; w < warp; ++w) woff += warp_tot[w];
-    int carry = carry_s;
-    if (i < nb) sums[i] = carry + woff + incl - v;
-    __syncthreads();
-    if (tid == 1023) carry_s = carry + woff + incl;
-    __syncthreads();
+    carry += sum;
   }
-  if (tid == 0) *total_out = carry_s;
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) f.total(carry);
 }
 
-__global__ void k_scan_add(int* out, int n, const int* block_offsets) {
-  const int base = blockIdx.x * 1024;
-  const int add = block_offsets[blockIdx.x];
-  for (int k = threadIdx.x; k < 1024; k += blockDim.x)
-    if (base + k < n) out[base + k] += add;
+template <typename F>
+cudaError_t launch_scan(const F& f, int n, typename F::T* tmp, cudaStream_t s) {
+  const int units = std::max(1, (int)(((long long)n + 1023) / 1024));
+  const long long per = 1024LL * ((units + kScanBlocks - 1) / kScanBlocks);
+  const unsigned nb = (unsigned)std::max(1LL, (n + per - 1) / per);
+  if (nb > 1) k_scan_sums<<<nb, 256, 0, s>>>(f, n, per, tmp);
+  k_scan_out<<<nb, 256, 0, s>>>(f, n, per, tmp);
+  return cudaGetLastError();
 }
+
+// out[0..n] with out[n] = total; `copy` (or nullptr) gets out[0..n - 1] as well
+struct ScanInts {
+  typedef int T;
+  const int* in;
+  int *out, *copy;
+  int n;
+  __device__ int load(int i) const { return in[i]; }
+  __device__ void store(int i, int prefix, int) const {
+    out[i] = prefix;
+    if (copy) copy[i] = prefix;
+  }
+  __device__ void total(int sum) const { out[n] = sum; }
+};
 
 cudaError_t launch_exclusive_scan(const int* in, int* out, int n, int* tmp, cudaStream_t s) {
-  int nb = (n + 1023) / 1024;
-  if (nb == 0) nb = 1;
-  k_scan_blocks<<<nb, 256, 0, s>>>(in, out, n, tmp);
-  k_scan_single<<<1, 1024, 0, s>>>(tmp, nb, out + n);
-  k_scan_add<<<nb, 256, 0, s>>>(out, n, tmp);
-  return cudaGetLastError();
+  return launch_scan(ScanInts{in, out, nullptr, n}, n, tmp, s);
 }
 
 // ------------------------------------------------------- observation prep
@@ -1926,19 +1952,28 @@ cudaError_t preload_eval_kernels() {
 
 // group hypotheses by mesh: hist -> offsets (exclusive scan) -> order;
 // hypotheses whose record the shortcut already wrote (skip[h] = 1) are left out
+// counts (and below places) a warp's hypotheses of one mesh with one atomic:
+// on a counter each they took 37 + 38 us for 120k hypotheses of three meshes, now 3.7 + 3.8
+__device__ __forceinline__ int group_key(const perch_obj* hyp, long long h, long long n, int n_mesh, const uint8_t* skip) {
+  return h >= n || (skip && skip[h]) ? -1 : min((int)hyp[h].mesh, n_mesh - 1);
+}
+
 __global__ void k_group_hist(const perch_obj* hyp, long long n, int n_mesh, int* hist, const uint8_t* skip) {
-  const long long h = blockIdx.x * 256LL + threadIdx.x;
-  if (h >= n || (skip && skip[h])) return;
-  const int m = min((int)hyp[h].mesh, n_mesh - 1);
-  atomicAdd(&hist[m], 1);
+  const int m = group_key(hyp, blockIdx.x * 256LL + threadIdx.x, n, n_mesh, skip), lane = threadIdx.x & 31;
+  const unsigned peers = __match_any_sync(0xffffffffu, m);
+  if (m >= 0 && lane == __ffs(peers) - 1) atomicAdd(&hist[m], __popc(peers));
 }
 
 __global__ void k_group_scatter(const perch_obj* hyp, long long n, int n_mesh, int* cursor, int* order,
                                 const uint8_t* skip) {
   const long long h = blockIdx.x * 256LL + threadIdx.x;
-  if (h >= n || (skip && skip[h])) return;
-  const int m = min((int)hyp[h].mesh, n_mesh - 1);
-  order[atomicAdd(&cursor[m], 1)] = (int)h;
+  const int m = group_key(hyp, h, n, n_mesh, skip), lane = threadIdx.x & 31;
+  const unsigned peers = __match_any_sync(0xffffffffu, m);
+  const int lead = __ffs(peers) - 1;
+  int at = 0;
+  if (m >= 0 && lane == lead) at = atomicAdd(&cursor[m], __popc(peers));
+  at = __shfl_sync(0xffffffffu, at, lead) + __popc(peers & ((1u << lane) - 1));
+  if (m >= 0) order[at] = (int)h;
 }
 
 cudaError_t launch_group_by_mesh(const perch_obj* hyp, long long n, int n_mesh, int* hist, int* offsets,
@@ -1948,16 +1983,15 @@ cudaError_t launch_group_by_mesh(const perch_obj* hyp, long long n, int n_mesh, 
   const unsigned blocks = (unsigned)((n + 255) / 256);
   k_group_hist<<<blocks, 256, 0, s>>>(hyp, n, n_mesh, hist, skip);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if ((e = launch_exclusive_scan(hist, offsets, n_mesh, scan_tmp, s)) != cudaSuccess) return e;
-  if ((e = cudaMemcpyAsync(cursor, offsets, sizeof(int) * n_mesh, cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
-    return e;
+  if ((e = launch_scan(ScanInts{hist, offsets, cursor, n_mesh}, n_mesh, scan_tmp, s)) != cudaSuccess) return e;
   k_group_scatter<<<blocks, 256, 0, s>>>(hyp, n, n_mesh, cursor, order, skip);
   return cudaGetLastError();
 }
 
-// ---- hypotheses grouped by pose, for shared renders: counts per pose ->
-// starts (exclusive scan) -> the distinct poses (scan of cnt > 0) -> each
-// mesh's ranges -> hypotheses placed in their pose's range
+// ---- hypotheses grouped by pose, for shared renders: counts per pose, one
+// scan of the counts and of the distinct poses together, hypotheses placed in
+// their pose's range. Five launches; with separate scans, flags, list and ranges
+// it was eleven (120k poses: 45 us in all, now 19).
 __global__ void k_pose_count(Geometry g, Batch b, int* cnt) {
   const long long h = blockIdx.x * 256LL + threadIdx.x;
   if (h >= b.n_hyp || (b.skip && b.skip[h])) return;
@@ -1970,32 +2004,43 @@ __global__ void k_pose_count(Geometry g, Batch b, int* cnt) {
   atomicAdd(&cnt[a.pose], 1);
 }
 
-// a pose is rendered when some hypothesis has it and (with the render
-// cache) the store does not hold its render under this batch's tag already
-__global__ void k_pose_nonzero(const int* cnt, int P, const uint32_t* valid, uint32_t tag, int* flag) {
-  const int p = blockIdx.x * 256 + threadIdx.x;
-  if (p < P) flag[p] = cnt[p] > 0 && !(valid && valid[p] == tag) ? 1 : 0;
-}
+// Per pose the hypotheses before it (low word) and the poses to render before it
+// (high word). A pose is rendered when some hypothesis has it and (with the
+// render cache) the store does not hold its render under this batch's tag already.
+// Mesh m owns poses [m per_mesh, (m + 1) per_mesh): its ranges of order and of
+// gpose begin at ranges[4 m] and ranges[4 m + 2] (n_mesh + 1 entries: the last
+// has the totals).
+struct ScanPoses {
+  typedef unsigned long long T;
+  const int* cnt;
+  const uint32_t* valid;
+  uint32_t tag;
+  int *start, *gpose, *ranges;
+  int per_mesh, n_mesh;
+  __device__ T load(int i) const {
+    const int c = cnt[i];
+    return (T)(uint32_t)c | (T)(c > 0 && !(valid && valid[i] == tag)) << 32;
+  }
+  __device__ void store(int i, T prefix, T v) const {
+    start[i] = (int)(uint32_t)prefix;
+    if (v >> 32) gpose[prefix >> 32] = i;
+    if (i % per_mesh == 0) range(i / per_mesh, prefix);
+  }
+  __device__ void range(int m, T prefix) const {
+    ranges[4 * m] = (int)(uint32_t)prefix;
+    ranges[4 * m + 2] = (int)(prefix >> 32);
+  }
+  __device__ void total(T sum) const { range(n_mesh, sum); }
+};
 
-__global__ void k_pose_list(const int* flag, const int* gix, int P, int* gpose) {
-  const int p = blockIdx.x * 256 + threadIdx.x;
-  if (p < P && flag[p]) gpose[gix[p]] = p;
-}
-
-// mesh m owns poses [m * per_mesh, (m + 1) * per_mesh): its hypotheses are
-// order[start[m * per_mesh] ..) and its distinct poses gpose[gix[m * per_mesh] ..)
-__global__ void k_mesh_ranges(const int* start, const int* gix, int n_mesh, int per_mesh, int* ranges) {
-  const int m = blockIdx.x * 256 + threadIdx.x;
-  if (m >= n_mesh) return;
-  const int a = m * per_mesh, e = a + per_mesh;
-  ranges[4 * m + 0] = start[a];
-  ranges[4 * m + 1] = start[e] - start[a];
-  ranges[4 * m + 2] = gix[a];
-  ranges[4 * m + 3] = gix[e] - gix[a];
-}
-
-__global__ void k_pose_place(Geometry g, Batch b, const int* start, int* cnt, int* order) {
+// also the meshes' counts, from the beginnings of their ranges
+__global__ void k_pose_place(Geometry g, Batch b, const int* start, int* cnt, int* order, int* ranges) {
   const long long h = blockIdx.x * 256LL + threadIdx.x;
+  if (blockIdx.x == 0)
+    for (int m = threadIdx.x; m < g.n_mesh; m += 256) {
+      ranges[4 * m + 1] = ranges[4 * m + 4] - ranges[4 * m];
+      ranges[4 * m + 3] = ranges[4 * m + 6] - ranges[4 * m + 2];
+    }
   if (h >= b.n_hyp || (b.skip && b.skip[h])) return;
   HypArgs a;
   if (!hyp_args(g, b, h, a)) return;
@@ -2005,17 +2050,14 @@ __global__ void k_pose_place(Geometry g, Batch b, const int* start, int* cnt, in
 cudaError_t launch_group_by_pose(const Geometry& g, const Batch& b, const PoseGroups& pg, const uint32_t* valid,
                                  uint32_t tag, cudaStream_t s) {
   const int per_mesh = g.nx * g.ny * g.n_yaw, P = g.n_mesh * per_mesh;
-  const unsigned pb = (unsigned)((P + 255) / 256), hb = (unsigned)((b.n_hyp + 255) / 256);
+  const unsigned hb = (unsigned)std::max(1LL, (b.n_hyp + 255) / 256);
   cudaError_t e = cudaMemsetAsync(pg.cnt, 0, sizeof(int) * (size_t)P, s);
   if (e != cudaSuccess) return e;
   if (b.n_hyp > 0) k_pose_count<<<hb, 256, 0, s>>>(g, b, pg.cnt);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if ((e = launch_exclusive_scan(pg.cnt, pg.start, P, pg.tmp, s)) != cudaSuccess) return e;
-  k_pose_nonzero<<<pb, 256, 0, s>>>(pg.cnt, P, valid, tag, pg.flag);
-  if ((e = launch_exclusive_scan(pg.flag, pg.gix, P, pg.tmp, s)) != cudaSuccess) return e;
-  k_pose_list<<<pb, 256, 0, s>>>(pg.flag, pg.gix, P, pg.gpose);
-  k_mesh_ranges<<<(unsigned)((g.n_mesh + 255) / 256), 256, 0, s>>>(pg.start, pg.gix, g.n_mesh, per_mesh, pg.ranges);
-  if (b.n_hyp > 0) k_pose_place<<<hb, 256, 0, s>>>(g, b, pg.start, pg.cnt, pg.order);
+  const ScanPoses f{pg.cnt, valid, tag, pg.start, pg.gpose, pg.ranges, per_mesh, g.n_mesh};
+  if ((e = launch_scan(f, P, pg.tmp, s)) != cudaSuccess) return e;
+  k_pose_place<<<hb, 256, 0, s>>>(g, b, pg.start, pg.cnt, pg.order, pg.ranges);
   return cudaGetLastError();
 }
 
@@ -2046,23 +2088,52 @@ cudaError_t launch_tile_offsets(const Geometry& g, int* sizes, int* tile_off, in
 // (mesh, pose) against an empty parent and an empty observation.
 
 // summed-area table S[(r + 1) (cols + 1) + c + 1] = sum of counts[0..r][0..c]
-// of `mats` matrices (one block each); S's first row and column are zero
-__global__ void k_sat(const int* counts, int rows, int cols, int* sat) {
+// of `mats` matrices (one block of 512 threads each); S's first row and column
+// are zero. Warps scan rows, threads then add down columns, 16 rows read at a
+// time: bound by those round trips to L2 (60 x 80 cells, 4 matrices: 12 -> 7.5 us).
+__global__ void __launch_bounds__(512) k_sat(const int* counts, int rows, int cols, int* sat) {
   const int* cnt = counts + (size_t)blockIdx.x * rows * cols;
-  int* S = sat + (size_t)blockIdx.x * (rows + 1) * (cols + 1);
+  const int ld = cols + 1, lane = threadIdx.x & 31;
+  int* S = sat + (size_t)blockIdx.x * (rows + 1) * ld;
   for (int c = threadIdx.x; c <= cols; c += blockDim.x) S[c] = 0;
-  for (int r = threadIdx.x; r < rows; r += blockDim.x) {
-    int* row = S + (size_t)(r + 1) * (cols + 1);
-    row[0] = 0;
-    int a = 0;
-    for (int c = 0; c < cols; ++c) {
-      a += cnt[(size_t)r * cols + c];
-      row[c + 1] = a;
+  for (int r = threadIdx.x >> 5; r < rows; r += blockDim.x >> 5) {
+    int* row = S + (size_t)(r + 1) * ld;
+    if (lane == 0) row[0] = 0;
+    int carry = 0;
+    for (int c0 = 0; c0 < cols; c0 += 128) {
+      int v[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int c = c0 + 32 * k + lane;
+        v[k] = c < cols ? cnt[(size_t)r * cols + c] : 0;
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        for (int d = 1; d < 32; d <<= 1) {
+          const int t = __shfl_up_sync(0xffffffffu, v[k], d);
+          if (lane >= d) v[k] += t;
+        }
+        v[k] += carry;
+        carry = __shfl_sync(0xffffffffu, v[k], 31);
+        const int c = c0 + 32 * k + lane;
+        if (c < cols) row[c + 1] = v[k];
+      }
     }
   }
   __syncthreads();
-  for (int c = threadIdx.x; c < cols; c += blockDim.x)
-    for (int r = 1; r < rows; ++r) S[(size_t)(r + 1) * (cols + 1) + c + 1] += S[(size_t)r * (cols + 1) + c + 1];
+  for (int c = 1 + threadIdx.x; c <= cols; c += blockDim.x) {
+    int a = 0;
+    for (int r0 = 1; r0 <= rows; r0 += 16) {
+      int v[16];
+#pragma unroll
+      for (int k = 0; k < 16; ++k) v[k] = r0 + k <= rows ? S[(size_t)(r0 + k) * ld + c] : 0;
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {
+        a += v[k];
+        if (r0 + k <= rows) S[(size_t)(r0 + k) * ld + c] = a;
+      }
+    }
+  }
 }
 
 __global__ void k_cell_counts(const int* start2, int n, int* counts) {
@@ -2073,28 +2144,36 @@ __global__ void k_cell_counts(const int* start2, int n, int* counts) {
 cudaError_t launch_grid2_sat(const int* start2, int n2x, int n2y, int* counts, int* sat, cudaStream_t s) {
   const int n = n2x * n2y;
   k_cell_counts<<<(n + 255) / 256, 256, 0, s>>>(start2, n, counts);
-  k_sat<<<1, 1024, 0, s>>>(counts, n2y, n2x, sat);
+  k_sat<<<1, 512, 0, s>>>(counts, n2y, n2x, sat);
   return cudaGetLastError();
 }
 
 // occupied pixels of each parent render per 8x8 tile
-__global__ void k_parent_tile_counts(Camera cam, Batch b, int* counts) {
-  const int p = blockIdx.y;
-  const int t = blockIdx.x * 256 + threadIdx.x;
-  if (t >= b.tiles_w * b.tiles_h) return;
-  const int tx = t % b.tiles_w, ty = t / b.tiles_w;
-  const float* z = b.parent_z + (size_t)p * cam.W * cam.H;
+// (a warp: the eight rows of four tiles, eight pixels a lane)
+__global__ void __launch_bounds__(256) k_parent_tile_counts(Camera cam, Batch b, int* counts) {
+  const int p = blockIdx.y, lane = threadIdx.x & 31, quads = (b.tiles_w + 3) >> 2;
+  const int w = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (w >= quads * b.tiles_h) return;
+  const int ty = w / quads, tx = 4 * (w % quads) + (lane & 3), v = 8 * ty + (lane >> 2), u0 = 8 * tx;
+  const float* z = b.parent_z + (size_t)p * cam.W * cam.H + (size_t)v * cam.W;
   int c = 0;
-  for (int v = ty * 8; v < min(ty * 8 + 8, cam.H); ++v)
-    for (int u = tx * 8; u < min(tx * 8 + 8, cam.W); ++u) c += __float_as_uint(z[(size_t)v * cam.W + u]) != kInfBits;
-  counts[(size_t)p * b.tiles_w * b.tiles_h + t] = c;
+  if (v < cam.H && (cam.W & 3) == 0 && u0 + 8 <= cam.W) {  // rows start on 16 bytes
+    const uint4* q = reinterpret_cast<const uint4*>(z + u0);
+    const uint4 a = __ldg(q), d = __ldg(q + 1);
+    c = (a.x != kInfBits) + (a.y != kInfBits) + (a.z != kInfBits) + (a.w != kInfBits) + (d.x != kInfBits) +
+        (d.y != kInfBits) + (d.z != kInfBits) + (d.w != kInfBits);
+  } else if (v < cam.H) {
+    for (int u = u0; u < min(u0 + 8, cam.W); ++u) c += __float_as_uint(z[u]) != kInfBits;
+  }
+  for (int d = 4; d < 32; d <<= 1) c += __shfl_xor_sync(0xffffffffu, c, d);
+  if (lane < 4 && tx < b.tiles_w) counts[((size_t)p * b.tiles_h + ty) * b.tiles_w + tx] = c;
 }
 
 cudaError_t launch_parent_tiles(const Camera& cam, const Batch& b, int* counts, int* sat, cudaStream_t s) {
   if (b.n_par > 65535) return cudaErrorInvalidValue;
-  dim3 grid((b.tiles_w * b.tiles_h + 255) / 256, b.n_par);
+  dim3 grid((((b.tiles_w + 3) >> 2) * b.tiles_h + 7) / 8, b.n_par);
   k_parent_tile_counts<<<grid, 256, 0, s>>>(cam, b, counts);
-  k_sat<<<b.n_par, 128, 0, s>>>(counts, b.tiles_h, b.tiles_w, sat);
+  k_sat<<<b.n_par, 512, 0, s>>>(counts, b.tiles_h, b.tiles_w, sat);
   return cudaGetLastError();
 }
 
