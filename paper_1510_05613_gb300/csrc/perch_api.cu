@@ -5,6 +5,8 @@
 // squared thresholds) is done in double and rounded once to binary32, as the
 // arithmetic contract in include/perch.h states; this file is compiled with
 // -ffp-contract=off so no fused multiply-add changes those roundings.
+#include <unistd.h>
+
 #include <algorithm>
 #include <climits>
 #include <cmath>
@@ -60,6 +62,10 @@ int perch_ctx::cuda(cudaError_t e, const char* what) {
   if (e == cudaErrorMemoryAllocation) return fail(PERCH_E_OOM, "%s: %s", what, cudaGetErrorString(e));
   return fail(PERCH_E_CUDA, "%s: %s", what, cudaGetErrorString(e));
 }
+
+// batches from this many records on check their flags on the device: below, the
+// host's pass takes less than the launch
+static constexpr long long kDeviceCheck = 16384;
 
 int perch_ctx::check_records(const perch_cost* out, long long n) {
   long long bad = 0, first = -1;
@@ -960,6 +966,50 @@ static int check_obj(perch_ctx* ctx, const perch_obj& o, const char* what, long 
   return PERCH_OK;
 }
 
+// Every hypothesis within the meshes, the grid and the parents: one pass
+// without branches, and only after a bad one the pass that names it.
+static int check_hyps(perch_ctx* ctx, const int32_t* hyp_parent, const perch_obj* hyp, long long n_hyp, int n_par) {
+  const uint32_t n_mesh = ctx->n_mesh, nx = ctx->nx, ny = ctx->ny, n_yaw = ctx->n_yaw;
+  uint32_t bad = 0;
+  for (long long h = 0; h < n_hyp; ++h) {
+    const perch_obj o = hyp[h];  // a negative index is a large unsigned one
+    bad |= (uint32_t)((uint32_t)hyp_parent[h] >= (uint32_t)n_par) | (uint32_t)(o.mesh >= n_mesh) |
+           (uint32_t)((uint32_t)o.ix >= nx) | (uint32_t)((uint32_t)o.iy >= ny) | (uint32_t)(o.iyaw >= n_yaw);
+  }
+  if (!bad) return PERCH_OK;
+  for (long long h = 0; h < n_hyp; ++h) {
+    if (hyp_parent[h] < 0 || hyp_parent[h] >= n_par)
+      return ctx->fail(PERCH_E_ARG, "hypothesis %lld: parent %d out of range", h, hyp_parent[h]);
+    int rc = check_obj(ctx, hyp[h], "hypothesis", h);
+    if (rc) return rc;
+  }
+  return PERCH_OK;
+}
+
+// Records of an evaluation that is under way to the host array, and their check.
+// A fresh array's pages are touched while the device works: mapping them inside
+// the copy took 1.0 ms for the 13 MB of 480k records. Large batches' flags are
+// looked at on the device, and the records only if one is set. With check_hyps:
+// 480k hypotheses 6.12 -> 5.15 ms, 120k 3.17 -> 2.98.
+int perch_ctx::fetch_records(perch_cost* out, long long n) {
+  perch_ctx* ctx = this;
+  const size_t bytes = sizeof(perch_cost) * (size_t)n;
+  const bool large = n >= kDeviceCheck;
+  uint32_t flags = 0;
+  if (large) {
+    CK(scratch_small.ensure(64), "alloc");
+    CK(launch_any_flags(b_out.as<perch_cost>(), n, scratch_small.as<uint32_t>(), stream), "flags kernel");
+    const size_t page = (size_t)sysconf(_SC_PAGESIZE);
+    volatile char* p = reinterpret_cast<volatile char*>(out);
+    for (size_t k = 0; k < bytes; k += page) p[k] = p[k];
+    p[bytes - 1] = p[bytes - 1];
+  }
+  CK(cudaMemcpyAsync(out, b_out.p, bytes, cudaMemcpyDeviceToHost, stream), "copy results");
+  if (large) CK(cudaMemcpyAsync(&flags, scratch_small.p, 4, cudaMemcpyDeviceToHost, stream), "copy flags");
+  CK(cudaStreamSynchronize(stream), "eval");
+  return large && !(flags & (kFlagTimeout | kFlagBadIndex)) ? PERCH_OK : check_records(out, n);
+}
+
 extern "C" {
 
 int perch_eval_successors(perch_ctx* ctx, const perch_obj* parents, int32_t parent_stride, const int32_t* parent_len,
@@ -983,12 +1033,7 @@ int perch_eval_successors(perch_ctx* ctx, const perch_obj* parents, int32_t pare
       if (rc) return rc;
     }
   }
-  for (long long h = 0; h < n_hyp; ++h) {
-    if (hyp_parent[h] < 0 || hyp_parent[h] >= n_par)
-      return ctx->fail(PERCH_E_ARG, "hypothesis %lld: parent %d out of range", h, hyp_parent[h]);
-    int rc = check_obj(ctx, hyp[h], "hypothesis", h);
-    if (rc) return rc;
-  }
+  if (int rc = check_hyps(ctx, hyp_parent, hyp, n_hyp, n_par)) return rc;
   CK(cudaSetDevice(ctx->device), "cudaSetDevice");
   const size_t pbytes = sizeof(perch_obj) * std::max<size_t>((size_t)n_par * parent_stride, 1);
   CK(ctx->b_parents.ensure(pbytes), "alloc");
@@ -1007,10 +1052,7 @@ int perch_eval_successors(perch_ctx* ctx, const perch_obj* parents, int32_t pare
                              ctx->b_hp.as<int32_t>(), ctx->b_hyp.as<perch_obj>(), n_hyp, K_total,
                              ctx->b_out.as<perch_cost>());
   if (rc) return rc;
-  CK(cudaMemcpyAsync(out, ctx->b_out.p, sizeof(perch_cost) * (size_t)n_hyp, cudaMemcpyDeviceToHost, ctx->stream),
-     "copy results");
-  CK(cudaStreamSynchronize(ctx->stream), "eval");
-  return ctx->check_records(out, n_hyp);
+  return ctx->fetch_records(out, n_hyp);
 }
 
 int perch_eval_successors_dev(perch_ctx* ctx, const perch_obj* parents, int32_t parent_stride,
@@ -1185,12 +1227,7 @@ int perch_eval_successors_multi(perch_ctx* ctx, const perch_obj* parents, int32_
       if (rc) return rc;
     }
   }
-  for (long long h = 0; h < n_hyp; ++h) {
-    if (hyp_parent[h] < 0 || hyp_parent[h] >= n_par)
-      return ctx->fail(PERCH_E_ARG, "hypothesis %lld: parent %d out of range", h, hyp_parent[h]);
-    int rc = check_obj(ctx, hyp[h], "hypothesis", h);
-    if (rc) return rc;
-  }
+  if (int rc = check_hyps(ctx, hyp_parent, hyp, n_hyp, n_par)) return rc;
   CK(cudaSetDevice(ctx->device), "cudaSetDevice");
   const size_t pbytes = sizeof(perch_obj) * std::max<size_t>((size_t)n_par * parent_stride, 1);
   CK(ctx->b_parents.ensure(pbytes), "alloc");
@@ -1212,10 +1249,7 @@ int perch_eval_successors_multi(perch_ctx* ctx, const perch_obj* parents, int32_
                              ctx->b_hyp.as<perch_obj>(), n_hyp, 1, ctx->b_out.as<perch_cost>(), d_plen + n_par,
                              d_plen + 2 * n_par);
   if (rc) return rc;
-  CK(cudaMemcpyAsync(out, ctx->b_out.p, sizeof(perch_cost) * (size_t)n_hyp, cudaMemcpyDeviceToHost, ctx->stream),
-     "copy results");
-  CK(cudaStreamSynchronize(ctx->stream), "eval");
-  return ctx->check_records(out, n_hyp);
+  return ctx->fetch_records(out, n_hyp);
 }
 
 }  // extern "C"

@@ -190,6 +190,7 @@ struct perch_ctx {
   // PERCH_E_DEVICE if some record of a finished host-side evaluation carries
   // kFlagTimeout or kFlagBadIndex (no cost was computed for it)
   int check_records(const perch_cost* out, long long n);
+  int fetch_records(perch_cost* out, long long n);
   int cuda(cudaError_t e, const char* what);
   perch::Geometry geometry() const;
   int ensure_tables();

@@ -234,6 +234,7 @@ cudaError_t launch_grid2_sat(const int* start2, int n2x, int n2y, int* counts, i
 cudaError_t launch_parent_tiles(const Camera& cam, const Batch& b, int* counts, int* sat, cudaStream_t s);
 cudaError_t launch_shortcut(const Camera& cam, const Geometry& g, const ObsIndex& obs, const Batch& b,
                             cudaStream_t s);
+cudaError_t launch_any_flags(const perch_cost* rec, long long n, uint32_t* flags, cudaStream_t s);
 cudaError_t launch_solo_pack(const perch_cost* rec, long long n, int2* solo, cudaStream_t s);
 cudaError_t launch_eval_group(const Camera& cam, const Geometry& g, const ObsIndex& obs, const Batch& b,
                               const int* order, const int* offset, const int* count, int* next, long long max_items,

@@ -2234,6 +2234,21 @@ __global__ void k_solo_pack(const perch_cost* rec, long long n, int2* solo) {
   if (h < n) solo[h] = make_int2(rec[h].n_new, (int)(rec[h].flags & 1u));
 }
 
+// *flags = the flags of all records together
+__global__ void k_any_flags(const perch_cost* rec, long long n, uint32_t* flags) {
+  uint32_t a = 0;
+  for (long long h = blockIdx.x * 256LL + threadIdx.x; h < n; h += gridDim.x * 256LL) a |= (uint32_t)rec[h].flags;
+  a = __reduce_or_sync(0xffffffffu, a);
+  if ((threadIdx.x & 31) == 0 && a) atomicOr(flags, a);
+}
+
+cudaError_t launch_any_flags(const perch_cost* rec, long long n, uint32_t* flags, cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(flags, 0, 4, s);
+  if (e != cudaSuccess) return e;
+  k_any_flags<<<(unsigned)std::min<long long>((n + 255) / 256, 152 * 8), 256, 0, s>>>(rec, n, flags);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_solo_pack(const perch_cost* rec, long long n, int2* solo, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   k_solo_pack<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(rec, n, solo);
