@@ -254,3 +254,27 @@ def test_gradients_add_up_over_the_batch(c1, n):
         assert np.linalg.norm(d) <= 2.0 ** -8 * np.linalg.norm(mean[off:off + a.size]) + 1e-30, (off, a.shape)
         off += a.size
     assert net.perch_cnn_tensor_status() == (0, 0)
+
+
+@pytest.mark.parametrize("n", [32, 224])
+def test_two_streams_leave_no_race(c1, n):
+    """Gradients of repeated calls, one behind the other without a wait of the host
+    in between, and of a second network on its own stream: bit for bit the same."""
+    wl, p, w = c1
+    n_onehot = len(wl.meshes) * wl.grid.n_yaw
+    crops, onehot = p.perch_cnn_crops([wl.gt[:1]], np.zeros(n, np.int32), _hyps_c1(wl, n, 31 + n))
+    target = torch.tensor(np.random.default_rng(32).uniform(0.0, 4.0, n), dtype=torch.float32, device="cuda")
+    torch.cuda.synchronize()
+    params = _params(n_onehot, 33)
+    nets = [_net_with(params, n_onehot, max_batch=224) for _ in range(2)]
+    ref = nets[0].perch_cnn_gradients(crops, onehot, target)[0]
+    for _ in range(3):
+        assert np.array_equal(nets[1].perch_cnn_gradients(crops, onehot, target)[0], ref)
+    for _ in range(6):  # steps of both networks in flight at once
+        for net in nets:
+            net.perch_cnn_train_step(crops, onehot, target, 1e-3)
+    a, b = (net.perch_cnn_get_params() for net in nets)
+    assert np.array_equal(a, b) and np.all(np.isfinite(a))
+    for net in nets:
+        assert net.perch_cnn_tensor_status() == (0, 0)
+        net.close()
