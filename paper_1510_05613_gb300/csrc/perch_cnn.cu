@@ -1448,13 +1448,14 @@ struct perch_cnn {
     for (int o = 0; o < kHidden; ++o) f(q++, off_f2 + o);
     f(q++, off_fb2);
   }
-  int ensure_batch(int n);
+  int ensure_batch(int n, int chunk);
   int refresh_weights();
-  int conv_fwd(int l, const bf16* x, int n);
+  int conv_fwd(int l, const bf16* x, int n, long long at);
   int dgrad_weights(int l, cudaStream_t s);
   int conv_dgrad(int l, const bf16* dz, int n, bf16* out);
   int conv_wgrad(int l, const bf16* dz, int n, int splits, int ksplit, cudaStream_t s);
-  int forward(const bf16* crops, const int32_t* onehot, int n, float* pred, const float* target);
+  int convolve(const bf16* crops, const int32_t* onehot, int n, int at);
+  int forward(const bf16* crops, const int32_t* onehot, int n, float* pred, const float* target, int chunk);
   int backward(const bf16* crops, int n);
   int backward_pass(const bf16* crops, int n);
   void release();
@@ -1472,12 +1473,13 @@ struct perch_cnn {
     if (rc_ != PERCH_OK) return rc_;          \
   } while (0)
 
-int perch_cnn::ensure_batch(int n) {
+// buffers of n crops, the first two layers' of a chunk of them
+int perch_cnn::ensure_batch(int n, int chunk) {
   perch_cnn* net = this;
-  const long long N = std::max(n, 32);
-  for (int l = 0; l < kConvs; ++l) {
+  const long long N = std::max(n, 32), C = std::max(chunk, 32);
+  for (int l = 0; l < kConvs - 1; ++l) {
     const long long Ho = kHin[l] / kStride[l];
-    if (l < kConvs - 1) CKN(act[l].ensure(2 * N * Ho * Ho * kCout[l]), "alloc activations");
+    CKN(act[l].ensure(2 * (l == kConvs - 2 ? N : C) * Ho * Ho * kCout[l]), "alloc activations");
   }
   CKN(feat.ensure(2 * N * Kf), "alloc");
   CKN(h1.ensure(2 * N * kHidden), "alloc");
@@ -1508,10 +1510,11 @@ static void conv_tile(int l, int n, ConvArgs* p, int* box) {
 }
 
 // Forward convolution of layer l = 1 .. 3 over n crops: x to act[l] or, the last
-// one, straight into the FC input rows (crop m / 64, position m % 64). The maps
+// one, straight into the FC input rows (crop m / 64, position m % 64), from crop
+// `at` of it on. The maps
 // cover the whole buffer of x, so they stay until it is reallocated; rows past
 // n crops are computed from what is there and not stored.
-int perch_cnn::conv_fwd(int l, const bf16* x, int n) {
+int perch_cnn::conv_fwd(int l, const bf16* x, int n, long long at) {
   perch_cnn* net = this;
   const int H = kHin[l], Cin = kCin[l], N = kCout[l], Kp = kp_of(l);
   const bool pair = Cin == 32;  // two horizontal neighbours make a 64-channel row
@@ -1542,9 +1545,9 @@ int perch_cnn::conv_fwd(int l, const bf16* x, int n) {
   p.bias = master.as<float>() + off_b[l];
   p.ldc = N;
   p.grp = 1 << 30;
-  p.out = act[l].as<bf16>();
+  p.out = act[l].as<bf16>() + at * (H / 2) * (H / 2) * N;
   if (l == kConvs - 1) {
-    p.out = feat.as<bf16>();
+    p.out = feat.as<bf16>() + at * Kf;
     p.grp = (H / 2) * (H / 2);
     p.ldg = Kf;
   }
@@ -1635,18 +1638,29 @@ int perch_cnn::conv_wgrad(int l, const bf16* d, int n, int splits, int ksplit, c
   return PERCH_OK;
 }
 
-// Forward pass of n <= max_batch crops; with a target also the per-sample
-// errors (for the backward pass).
-int perch_cnn::forward(const bf16* crops, const int32_t* onehot, int n, float* pred, const float* target) {
+// The first three convolutions (and the one-hot columns) of n crops, to
+// crops at .. at + n - 1 of act[2] and of the FC input
+int perch_cnn::convolve(const bf16* crops, const int32_t* onehot, int n, int at) {
   perch_cnn* net = this;
-  int rc = ensure_batch(n);
-  if (rc) return rc;
   k_conv1<<<8 * n, 256, 0, stream>>>(reinterpret_cast<const uint32_t*>(crops), w16.as<bf16>() + off_w[0],
                                      master.as<float>() + off_b[0], act[0].as<bf16>(), onehot, onehot_pad, Kf,
-                                     feat.as<bf16>());
+                                     feat.as<bf16>() + (long long)at * Kf);
   CKN(cudaGetLastError(), "input layer");
-  for (int l = 1; l < kConvs; ++l)
-    if ((rc = conv_fwd(l, act[l - 1].as<bf16>(), n))) return rc;
+  if (int rc = conv_fwd(1, act[0].as<bf16>(), n, 0)) return rc;
+  return conv_fwd(2, act[1].as<bf16>(), n, at);
+}
+
+// Forward pass of n crops; with a target also the per-sample errors (for the
+// backward pass). Layers 1 to 3 run `chunk` crops at a time, so that a chunk's
+// activations (262 and 131 KB a crop) stay in L2 from one to the next; layer 4 and the
+// FC layers, whose few tiles leave SMs idle on one chunk, run on all n.
+int perch_cnn::forward(const bf16* crops, const int32_t* onehot, int n, float* pred, const float* target, int chunk) {
+  perch_cnn* net = this;
+  int rc = ensure_batch(n, chunk);
+  if (rc) return rc;
+  for (int at = 0; at < n; at += chunk)
+    if ((rc = convolve(crops + (long long)at * 2 * kCrop * kCrop, onehot + at, std::min(chunk, n - at), at))) return rc;
+  if ((rc = conv_fwd(3, act[2].as<bf16>(), n, 0))) return rc;
   // FC1: few output tiles over a long K, so split K and finish bias + ReLU in a second pass
   GemmArgs p{};
   p.A = feat.as<bf16>();
@@ -1656,7 +1670,8 @@ int perch_cnn::forward(const bf16* crops, const int32_t* onehot, int n, float* p
   p.M = n;
   p.N = kHidden;
   p.K = Kf;
-  const int S = choose_splits(n, kHidden, Kf, &p.Ksplit);
+  // (the splits, and so the order of the sums, are those of a chunk alone)
+  const int S = choose_splits(std::min(n, chunk), kHidden, Kf, &p.Ksplit);
   CKN(part.ensure(4 * (size_t)S * n * kHidden), "alloc");
   p.Cf = part.as<float>();
   p.ldc = kHidden;
@@ -1938,15 +1953,21 @@ int perch_cnn_get_params(perch_cnn* net, float* params, int64_t n) {
   return PERCH_OK;
 }
 
+// crops whose layer 4 and FC layers a prediction runs at once: 2048 crops in chunks of 256,
+// 728 us with 256, 629 with 512, 590 with 1024 (act[2] is then 67 MB)
+static constexpr int kGroup = 1024;
+
 int perch_cnn_forward(perch_cnn* net, const uint16_t* crops, const int32_t* onehot, int64_t n, float* pred) {
   if (!net) return PERCH_E_ARG;
   net->err.clear();
   if (n < 0 || (n > 0 && (!crops || !onehot || !pred))) return net->fail(PERCH_E_ARG, "bad arguments");
   CKN(cudaSetDevice(net->device), "cudaSetDevice");
-  for (int64_t b = 0; b < n; b += net->max_batch) {
-    const int nb = (int)std::min<int64_t>(net->max_batch, n - b);
-    int rc = net->forward(reinterpret_cast<const bf16*>(crops) + b * 2 * kCrop * kCrop, onehot + b, nb, pred + b,
-                          nullptr);
+  // whole chunks of max_batch in groups of up to kGroup crops, then the rest
+  const int64_t whole = n / net->max_batch * net->max_batch, group = std::max(kGroup / net->max_batch, 1) * net->max_batch;
+  for (int64_t b = 0, nb; b < n; b += nb) {
+    nb = b < whole ? std::min<int64_t>(group, whole - b) : n - b;
+    int rc = net->forward(reinterpret_cast<const bf16*>(crops) + b * 2 * kCrop * kCrop, onehot + b, (int)nb, pred + b,
+                          nullptr, net->max_batch);
     if (rc) return rc;
   }
   return PERCH_OK;
@@ -1960,9 +1981,9 @@ int perch_cnn_gradients(perch_cnn* net, const uint16_t* crops, const int32_t* on
     return net->fail(PERCH_E_ARG, "need device crops / one-hot / targets and 32 <= n <= %d, n %% 32 == 0",
                      net->max_batch);
   CKN(cudaSetDevice(net->device), "cudaSetDevice");
-  int rc = net->ensure_batch(n);
+  int rc = net->ensure_batch(n, n);  // pred_buf is passed below
   if (rc) return rc;
-  rc = net->forward(reinterpret_cast<const bf16*>(crops), onehot, n, net->pred_buf.as<float>(), target);
+  rc = net->forward(reinterpret_cast<const bf16*>(crops), onehot, n, net->pred_buf.as<float>(), target, n);
   if (rc) return rc;
   rc = net->backward(reinterpret_cast<const bf16*>(crops), n);
   if (rc) return rc;
@@ -1986,7 +2007,7 @@ int perch_cnn_train_step(perch_cnn* net, const uint16_t* crops, const int32_t* o
     return net->fail(PERCH_E_ARG, "need device crops / one-hot / targets, 32 <= n <= %d, n %% 32 == 0, lr > 0",
                      net->max_batch);
   CKN(cudaSetDevice(net->device), "cudaSetDevice");
-  int rc = net->forward(reinterpret_cast<const bf16*>(crops), onehot, n, net->pred_buf.as<float>(), target);
+  int rc = net->forward(reinterpret_cast<const bf16*>(crops), onehot, n, net->pred_buf.as<float>(), target, n);
   if (rc) return rc;
   rc = net->backward(reinterpret_cast<const bf16*>(crops), n);
   if (rc) return rc;
