@@ -1277,6 +1277,28 @@ __global__ void k_to_bf16(const float* __restrict__ in, long long n, bf16* __res
     out[e] = __float2bfloat16_rn(in[e]);
 }
 
+// The value of a depth d against the centre's depth zr, before it is rounded to
+// bfloat16: clamp(RN32(RN64(RN64(zr - d) scale))). The double operations run at a small
+// fraction of the binary32 rate and bound the kernel, so the value is first taken
+// in binary32, zr as zh + zl and the difference as a sum and its exact error:
+// within 2^-22 of itself (two roundings; the scale is exact) plus 2^-32 (zl's own
+// rounding, 2^-50 |zr|, |zr| < 2^14) of the double value. Rounding and clamp are
+// monotone: where both ends of twice that interval round to one bfloat16, so does the
+// value; else (one in 2^12) it is computed in double. 14336 crops of eight scenes:
+// 915 -> 209 us.
+__device__ __forceinline__ float crop_value(double zr, float zh, float zl, float d) {
+  const float s = __fsub_rn(zh, d), bb = __fsub_rn(s, zh);
+  const float err = __fsub_rn(__fsub_rn(zh, __fsub_rn(s, bb)), __fadd_rn(d, bb));
+  const float t = __fmul_rn(__fadd_rn(s, __fadd_rn(err, zl)), (float)kScale);
+  const float eps = __fadd_rn(__fmul_rn(fabsf(t), 0x1p-21f), 0x1p-31f);
+  const float lo = fminf(fmaxf(__fsub_rn(t, eps), -kClamp), kClamp), hi = fminf(fmaxf(__fadd_rn(t, eps), -kClamp), kClamp);
+  if (__bfloat16_as_ushort(__float2bfloat16_rn(lo)) == __bfloat16_as_ushort(__float2bfloat16_rn(hi)) &&
+      fabsf(zh) < 16384.0f)
+    return lo;
+  const float x = __double2float_rn(__dmul_rn(__dsub_rn(zr, (double)d), kScale));
+  return fminf(fmaxf(x, -kClamp), kClamp);
+}
+
 // ---------------------------------------------------------------- crops
 // One block per hypothesis. The centre is the projection of (x, y, middle of
 // V(O)'s height range), in double with every operation rounded separately:
@@ -1292,6 +1314,7 @@ __global__ void k_crops(Camera cam, const float* __restrict__ xs, const float* _
                         bf16* __restrict__ crops, int32_t* __restrict__ onehot) {
   __shared__ int s_cu, s_cv, s_ok;
   __shared__ double s_zr;
+  __shared__ float s_zh, s_zl;
   const long long h = blockIdx.x;
   if (h >= n_hyp) return;
   const perch_obj o = hyp[h];
@@ -1318,6 +1341,8 @@ __global__ void k_crops(Camera cam, const float* __restrict__ xs, const float* _
     s_cu = ok ? (int)floor(__dadd_rn(u, 0.5)) : 0;
     s_cv = ok ? (int)floor(__dadd_rn(v, 0.5)) : 0;
     s_zr = c[2];
+    s_zh = __double2float_rn(c[2]);
+    s_zl = __double2float_rn(__dsub_rn(c[2], (double)s_zh));
     onehot[h] = (int32_t)o.mesh * n_yaw + o.iyaw;
   }
   __syncthreads();
@@ -1326,16 +1351,14 @@ __global__ void k_crops(Camera cam, const float* __restrict__ xs, const float* _
   const float* img = scene_img[sc];
   const float* pz = parent_z + (long long)par * W * H;
   const double zr = s_zr;
+  const float zh = s_zh, zl = s_zl;
   for (int px = threadIdx.x; px < kCrop * kCrop; px += blockDim.x) {
     const int r = s_cv - kCrop / 2 + px / kCrop, c = s_cu - kCrop / 2 + px % kCrop;
     float val[2] = {kMissing, kMissing};
     if (s_ok && r >= 0 && r < H && c >= 0 && c < W) {
       const float d[2] = {img[(long long)r * W + c], pz[(long long)r * W + c]};
       for (int ch = 0; ch < 2; ++ch)
-        if (isfinite(d[ch]) && d[ch] > 0.0f) {
-          const float t = __double2float_rn(__dmul_rn(__dsub_rn(zr, (double)d[ch]), kScale));
-          val[ch] = fminf(fmaxf(t, -kClamp), kClamp);
-        }
+        if (isfinite(d[ch]) && d[ch] > 0.0f) val[ch] = crop_value(zr, zh, zl, d[ch]);
     }
     *reinterpret_cast<__nv_bfloat162*>(crops + (h * kCrop * kCrop + px) * 2) = __floats2bfloat162_rn(val[0], val[1]);
   }
