@@ -422,7 +422,8 @@ int perch_set_threads(perch_ctx* ctx, int32_t mesh, int32_t threads);
  * per-hypothesis evaluation) launch, the render's inline limit (a front-facing
  * triangle with at most about that many candidate pixel centres is rasterised
  * by its own thread, a larger one by several through the CTA's queue) and the CTA
- * width of the cost launch. With shared renders on, perch_autotune times
+ * width of the cost launch (before perch_autotune 128, which batches of up to
+ * 131072 hypotheses run as 256). With shared renders on, perch_autotune times
  * every render width with every inline limit (8, 16, 32), then the cost
  * widths 128 and 256. */
 int perch_launch_config(perch_ctx* ctx, int32_t* render_threads, int32_t* inline_pixels, int32_t* cost_threads);

@@ -172,7 +172,10 @@ int perch_ctx::ensure_tables() {
   std::stable_sort(mesh_order.begin(), mesh_order.end(),
                    [&](int a, int b2) { return h_meshes[a].n_tris > h_meshes[b2].n_tris; });
   if ((int)mesh_threads.size() != n_mesh) mesh_threads.assign(n_mesh, 256);
-  if ((int)mesh_cost_threads.size() != n_mesh) mesh_cost_threads.assign(n_mesh, 128);
+  if ((int)mesh_cost_threads.size() != n_mesh) {
+    mesh_cost_threads.assign(n_mesh, 128);
+    cost_by_size = true;
+  }
   if ((int)mesh_cost_stages.size() != n_mesh) mesh_cost_stages.assign(n_mesh, 1);
   if ((int)mesh_inline.size() != n_mesh) mesh_inline.assign(n_mesh, kInlinePixels);
   if ((int)mesh_queue.size() != n_mesh) mesh_queue.assign(n_mesh, kBigQueue);
@@ -796,6 +799,13 @@ int perch_ctx::ensure_solo() {
 // 3.21; 30k, two heavy meshes: 6.97 and 6.81; 4.7k: 1.55 and 1.30).
 static constexpr long long kForkHyps = 1 << 17;
 
+// Up to this many hypotheses the cost CTAs of meshes that were not autotuned have
+// 256 threads: the time of a batch is that of its hypotheses among observed points, a few
+// for each CTA (4.7k hypotheses near the objects: 1.25 ms with 128, 1.23 with
+// 256; eight scenes, 14k, with crops: 2.34 and 2.13). Larger batches are bound by
+// throughput (240k: 12.39 and 12.47).
+static constexpr long long kWideCostHyps = 1 << 17;
+
 int perch_ctx::enqueue_eval(const perch_obj* d_parents, int parent_stride, const int32_t* d_plen, int n_par,
                             const int32_t* d_hp, const perch_obj* d_hyp, long long n_hyp, int K_total,
                             perch_cost* d_out, const int32_t* d_parent_scene, const int32_t* d_parent_K) {
@@ -882,6 +892,7 @@ int perch_ctx::enqueue_eval(const perch_obj* d_parents, int parent_stride, const
     }
     return e;
   };
+  const bool wide_cost = cost_by_size && n_hyp <= kWideCostHyps;
   // a batch of one parent repeats no pose: rendering per hypothesis skips the
   // tile store's round trip
   const bool cache = render_cache && !capturing;  // a captured graph would keep one epoch's tag
@@ -921,7 +932,8 @@ int perch_ctx::enqueue_eval(const perch_obj* d_parents, int parent_stride, const
       bm.tile_h = mesh_tile_h[m];
       const CostWork c{pg.order, rg + 4 * m, rg + 4 * m + 1, g_next.as<int>() + n_mesh + m, tile_store.as<uint32_t>(),
                        tile_off.as<int>(), pose_flags.as<uint8_t>(), tile_box.as<int4>()};
-      return launch_cost_group(cam, g, obs, bm, c, n_hyp, mesh_cost_threads[m], mesh_cost_stages[m], sm_count, st);
+      return launch_cost_group(cam, g, obs, bm, c, n_hyp, wide_cost ? 256 : mesh_cost_threads[m], mesh_cost_stages[m],
+                               sm_count, st);
     }), "cost kernel");
     last_path = 2;
     if (!capturing) {

@@ -106,6 +106,7 @@ struct perch_ctx {
   DevBuf tile_store, tile_off, tile_sizes, pose_flags, tile_box;
   DevBuf pg_cnt, pg_start, pg_gpose, pg_tmp, pg_ranges;  // hypotheses grouped by pose
   std::vector<int> mesh_cost_threads;  // CTA width of k_cost per mesh (autotuned; 128 by default)
+  bool cost_by_size = true;  // not autotuned: the width follows the batch (kWideCostHyps)
   std::vector<int> mesh_cost_stages;   // stage buffers of k_cost per mesh (1 or 2; autotuned; 1 by default)
   std::vector<int> mesh_inline;        // k_render's inline limit per mesh (autotuned; 16 by default)
   std::vector<int> mesh_queue;         // depth of the render's bin of larger triangles per mesh (autotuned)

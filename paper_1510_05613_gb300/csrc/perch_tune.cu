@@ -80,12 +80,15 @@ extern "C" int perch_autotune(perch_ctx* ctx, int32_t n_sample, int32_t* threads
   } shortcut_off{ctx, ctx->shortcut, ctx->render_cache};
   ctx->shortcut = false;
   ctx->render_cache = false;
+  const bool by_size = ctx->cost_by_size;
+  ctx->cost_by_size = false;  // the widths tried below are the ones launched
   const bool shared = ctx->share_renders && ctx->store_ok;
   const std::vector<int> saved_cost = ctx->mesh_cost_threads, saved_inline = ctx->mesh_inline,
                          saved_bins = ctx->mesh_queue, saved_stages = ctx->mesh_cost_stages;
   auto restore = [&]() {
     ctx->mesh_threads = saved;
     ctx->mesh_cost_threads = saved_cost;
+    ctx->cost_by_size = by_size;
     ctx->mesh_inline = saved_inline;
     ctx->mesh_queue = saved_bins;
     ctx->mesh_cost_stages = saved_stages;
