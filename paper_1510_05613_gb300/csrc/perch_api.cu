@@ -820,7 +820,16 @@ int perch_ctx::enqueue_eval(const perch_obj* d_parents, int parent_stride, const
   CK(parent_z.ensure(4 * npx * std::max(n_par, 1)), "alloc parent z-buffers");
   const int ustride = std::max(d_parent_scene ? max_obs : obs.n, 1);
   CK(uset.ensure(4 * (size_t)ustride * std::max(n_par, 1)), "alloc U sets");
-  CK(uset_count.ensure(4 * (size_t)std::max(n_par, 1)), "alloc");
+  // a batch of one parent repeats no pose: rendering per hypothesis skips the
+  // tile store's round trip
+  const bool cache = render_cache && !capturing;  // a captured graph would keep one epoch's tag
+  const bool shared = share_renders && store_ok && (n_par >= 2 || cache);
+  const int per_mesh = shared ? nx * ny * n_yaw : 0, P = per_mesh * n_mesh;  // the store's poses: at most 2^28
+  const size_t n_count = 2 + 3 * (size_t)n_mesh + std::max(n_par, 1);
+  CK(counters.ensure(4 * n_count), "alloc");
+  int* const hist = counters.as<int>() + 2;  // see perch_ctx
+  int* const next = hist + n_mesh;
+  if (shared) CK(pg_cnt.ensure(4 * (size_t)P), "alloc");
   Batch b;
   std::memset(&b, 0, sizeof b);
   b.parents = d_parents;
@@ -829,7 +838,7 @@ int perch_ctx::enqueue_eval(const perch_obj* d_parents, int parent_stride, const
   b.n_par = n_par;
   b.parent_z = parent_z.as<float>();
   b.uset = uset.as<uint32_t>();
-  b.uset_count = uset_count.as<int>();
+  b.uset_count = next + 2 * n_mesh;
   b.uset_stride = ustride;
   b.scenes = d_scenes.as<ObsIndex>();
   b.n_scenes = (int)scenes.size();
@@ -849,8 +858,9 @@ int perch_ctx::enqueue_eval(const perch_obj* d_parents, int parent_stride, const
     if (rc != PERCH_OK) return rc;
   }
   if (!capturing) CK(cudaEventRecord(ev[0], stream), "event");
-  CK(launch_fill_u32(parent_z.as<uint32_t>(), kInfBits, (long long)npx * n_par, stream), "clear parents");
-  CK(cudaMemsetAsync(uset_count.p, 0, 4 * (size_t)std::max(n_par, 1), stream), "memset");
+  CK(launch_prepare(parent_z.as<uint32_t>(), (long long)npx * n_par, counters.as<int>(), (long long)n_count,
+                    pg_cnt.as<int>(), P, stream),
+     "prepare");
   CK(launch_render_parents(cam, g, b, max_chunks, nullptr, stream), "render parents");
   CK(launch_uset(cam, g, obs, b, stream), "U sets");
   if (use_short) {  // records fixed by the solo render, written now and left out of the evaluation
@@ -860,12 +870,10 @@ int perch_ctx::enqueue_eval(const perch_obj* d_parents, int parent_stride, const
     CK(ptile_counts.ensure(4 * per * std::max(n_par, 1)), "alloc");
     CK(ptile_sat.ensure(4 * per_sat * std::max(n_par, 1)), "alloc");
     CK(skip.ensure((size_t)n_hyp), "alloc");
-    CK(n_short.ensure(8), "alloc");
-    CK(cudaMemsetAsync(n_short.p, 0, 8, stream), "memset");
     b.solo = solo.as<int2>();
     b.parent_sat = ptile_sat.as<int>();
     b.skip = skip.as<uint8_t>();
-    b.n_short = n_short.as<unsigned long long>();
+    b.n_short = counters.as<unsigned long long>();
     CK(launch_parent_tiles(cam, b, ptile_counts.as<int>(), ptile_sat.as<int>(), stream), "parent tiles");
     CK(launch_shortcut(cam, g, obs, b, stream), "shortcut");
   }
@@ -893,26 +901,19 @@ int perch_ctx::enqueue_eval(const perch_obj* d_parents, int parent_stride, const
     return e;
   };
   const bool wide_cost = cost_by_size && n_hyp <= kWideCostHyps;
-  // a batch of one parent repeats no pose: rendering per hypothesis skips the
-  // tile store's round trip
-  const bool cache = render_cache && !capturing;  // a captured graph would keep one epoch's tag
-  if (share_renders && store_ok && (n_par >= 2 || cache)) {
+  if (shared) {
     // shared renders: group by pose; per mesh one persistent launch renders
     // its distinct poses into the tile store, then one costs its hypotheses
-    const int per_mesh = nx * ny * n_yaw, P = per_mesh * n_mesh;
-    CK(pg_cnt.ensure(4 * (size_t)P), "alloc");
     CK(pg_start.ensure(4 * ((size_t)P + 1)), "alloc");
     CK(pg_gpose.ensure(4 * (size_t)P), "alloc");
     CK(pg_tmp.ensure(8 * ((size_t)P / 1024 + 2)), "alloc");
     CK(pg_ranges.ensure(16 * ((size_t)n_mesh + 1)), "alloc");
     CK(g_order.ensure(sizeof(int) * (size_t)std::max(n_hyp, 1LL)), "alloc");
-    CK(g_next.ensure(sizeof(int) * 2 * (size_t)n_mesh), "alloc");
     PoseGroups pg{pg_cnt.as<int>(), pg_start.as<int>(), pg_gpose.as<int>(), pg_tmp.as<unsigned long long>(),
                   pg_ranges.as<int>(), g_order.as<int>()};
     const uint32_t tag = 2u * render_epoch + (b.parent_scene ? 0u : 1u);
     uint32_t* valid = cache ? pose_valid.as<uint32_t>() : nullptr;
     CK(launch_group_by_pose(g, b, pg, valid, tag, stream), "group by pose");
-    CK(cudaMemsetAsync(g_next.p, 0, sizeof(int) * 2 * (size_t)n_mesh, stream), "memset");
     if (!capturing) CK(cudaEventRecord(ev[2], stream), "event");
     int* rg = pg.ranges;
     CK(each_mesh([&](int m, cudaStream_t st) {
@@ -920,7 +921,7 @@ int perch_ctx::enqueue_eval(const perch_obj* d_parents, int parent_stride, const
       bm.tile_w = mesh_tile_w[m];
       bm.tile_h = mesh_tile_h[m];
       bm.queue_cap = mesh_queue[m];
-      const RenderWork w{pg.gpose, rg + 4 * m + 2, rg + 4 * m + 3, g_next.as<int>() + m, tile_store.as<uint32_t>(),
+      const RenderWork w{pg.gpose, rg + 4 * m + 2, rg + 4 * m + 3, next + m, tile_store.as<uint32_t>(),
                          tile_off.as<int>(), pose_flags.as<uint8_t>(), valid, tag, tile_box.as<int4>()};
       return launch_render_group(cam, g, obs, bm, w, std::min<long long>(n_hyp, per_mesh), mesh_threads[m],
                                  mesh_inline[m], sm_count, st);
@@ -930,7 +931,7 @@ int perch_ctx::enqueue_eval(const perch_obj* d_parents, int parent_stride, const
       Batch bm = b;
       bm.tile_w = mesh_tile_w[m];
       bm.tile_h = mesh_tile_h[m];
-      const CostWork c{pg.order, rg + 4 * m, rg + 4 * m + 1, g_next.as<int>() + n_mesh + m, tile_store.as<uint32_t>(),
+      const CostWork c{pg.order, rg + 4 * m, rg + 4 * m + 1, next + n_mesh + m, tile_store.as<uint32_t>(),
                        tile_off.as<int>(), pose_flags.as<uint8_t>(), tile_box.as<int4>()};
       return launch_cost_group(cam, g, obs, bm, c, n_hyp, wide_cost ? 256 : mesh_cost_threads[m], mesh_cost_stages[m],
                                sm_count, st);
@@ -943,24 +944,20 @@ int perch_ctx::enqueue_eval(const perch_obj* d_parents, int parent_stride, const
     return PERCH_OK;
   }
   // group by mesh; one persistent launch per mesh with its own tile and CTA width
-  CK(g_hist.ensure(sizeof(int) * (size_t)n_mesh), "alloc");
   CK(g_off.ensure(sizeof(int) * ((size_t)n_mesh + 1)), "alloc");
   CK(g_cursor.ensure(sizeof(int) * (2 * (size_t)n_mesh + 1)), "alloc");
-  CK(g_next.ensure(sizeof(int) * (size_t)n_mesh), "alloc");
   CK(g_order.ensure(sizeof(int) * (size_t)std::max(n_hyp, 1LL)), "alloc");
   CK(scan_tmp.ensure(sizeof(int) * ((size_t)n_mesh / 1024 + 2)), "alloc");
-  CK(launch_group_by_mesh(d_hyp, n_hyp, n_mesh, g_hist.as<int>(), g_off.as<int>(), g_cursor.as<int>(),
+  CK(launch_group_by_mesh(d_hyp, n_hyp, n_mesh, hist, g_off.as<int>(), g_cursor.as<int>(),
                           g_order.as<int>(), scan_tmp.as<int>(), stream, use_short ? skip.as<uint8_t>() : nullptr),
      "group by mesh");
-  CK(cudaMemsetAsync(g_next.p, 0, sizeof(int) * (size_t)n_mesh, stream), "memset");
   if (!capturing) CK(cudaEventRecord(ev[2], stream), "event");
   CK(each_mesh([&](int m, cudaStream_t st) {
     Batch bm = b;
     bm.tile_w = mesh_tile_w[m];
     bm.tile_h = mesh_tile_h[m];
     bm.queue_cap = mesh_queue[m];
-    return launch_eval_group(cam, g, obs, bm, g_order.as<int>(), g_off.as<int>() + m, g_hist.as<int>() + m,
-                             g_next.as<int>() + m, n_hyp, mesh_threads[m], sm_count, st);
+    return launch_eval_group(cam, g, obs, bm, g_order.as<int>(), g_off.as<int>() + m, hist + m, next + m, n_hyp, mesh_threads[m], sm_count, st);
   }), "eval kernel");
   last_path = 1;
   if (!capturing) {
@@ -1185,7 +1182,7 @@ int perch_shortcut_stats(perch_ctx* ctx, int64_t* n_short, int64_t* n_total) {
   int64_t a = 0;
   if (ctx->short_counted) {
     unsigned long long v = 0;
-    CK(cudaMemcpyAsync(&v, ctx->n_short.p, 8, cudaMemcpyDeviceToHost, ctx->stream), "copy");
+    CK(cudaMemcpyAsync(&v, ctx->counters.p, 8, cudaMemcpyDeviceToHost, ctx->stream), "copy");
     CK(cudaStreamSynchronize(ctx->stream), "shortcut stats");
     a = (int64_t)v;
   }

@@ -94,8 +94,11 @@ struct perch_ctx {
   int sm_count = 0;
 
   // per-batch buffers
-  DevBuf parent_z, uset, uset_count;
-  DevBuf g_hist, g_off, g_cursor, g_order, g_next;  // hypotheses grouped by mesh
+  DevBuf parent_z, uset;
+  // hypotheses grouped by mesh; counters: what a batch counts in, zeroed in one
+  // launch: shortcut records (2 ints), then per mesh hypotheses and two work cursors, per
+  // parent points of U
+  DevBuf counters, g_off, g_cursor, g_order;
 
   // shared renders (perch_set_share_renders, on by default): the tile store
   // holds one render per pose, indexed by pose; it is sized once per
@@ -133,7 +136,7 @@ struct perch_ctx {
   // for the geometry version and camera it was built for
   bool shortcut = true;
   bool building_solo = false;
-  DevBuf solo, solo_rec, solo_hyp, solo_hp, solo_parent, ptile_counts, ptile_sat, skip, n_short;
+  DevBuf solo, solo_rec, solo_hyp, solo_hp, solo_parent, ptile_counts, ptile_sat, skip;
   long long geom_version = 0, solo_version = -1;
   perch::Camera solo_cam{};
   long long last_short = 0, last_total = 0;
@@ -179,9 +182,9 @@ struct perch_ctx {
   std::vector<DevBuf*> all_buffers() {
     return {&meshes, &chunk_verts, &chunk_info, &chunk_tris, &vol_normals, &yaw_mats, &pose_off, &vtab, &xs, &ys, &cs, &depth, &rx, &ry, &blockcnt, &blockoff,
             &scan_tmp, &cam_pts, &world_pts, &keys, &counts, &cursor, &d_scenes, &d_scene_img,
-            &scratch_small, &pose_bbox, &pose_general, &parent_z, &uset, &uset_count, &b_parents, &b_plen, &b_hp, &b_hyp,
-            &b_out, &g_hist, &g_off, &g_cursor, &g_order, &g_next, &net_crops, &net_onehot, &net_pred,
-            &solo, &solo_rec, &solo_hyp, &solo_hp, &solo_parent, &ptile_counts, &ptile_sat, &skip, &n_short,
+            &scratch_small, &pose_bbox, &pose_general, &parent_z, &uset, &counters, &b_parents, &b_plen, &b_hp, &b_hyp,
+            &b_out, &g_off, &g_cursor, &g_order, &net_crops, &net_onehot, &net_pred,
+            &solo, &solo_rec, &solo_hyp, &solo_hp, &solo_parent, &ptile_counts, &ptile_sat, &skip,
             &tile_store, &tile_off, &tile_sizes, &pose_flags, &pg_cnt, &pg_start, &pg_gpose,
             &pg_tmp, &pg_ranges, &pose_valid, &tile_box, &icp_src, &icp_pts, &icp_start, &icp_next,
             &icp_out, &icp_model, &icp_img_pts, &icp_img_lo, &icp_img_hi};

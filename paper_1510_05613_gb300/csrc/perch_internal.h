@@ -166,7 +166,7 @@ struct CostWork {
 
 // Hypotheses grouped by pose; P = n_mesh x nx x ny x n_yaw. All device arrays.
 struct PoseGroups {
-  int* cnt;     // P: hypotheses per pose (zero again after the grouping)
+  int* cnt;     // P: hypotheses per pose (zero before and after the grouping)
   int* start;   // P: exclusive scan of cnt
   int* gpose;   // P: the distinct poses, in pose order
   unsigned long long* tmp;  // min(P / 1024 + 1, 2048): scan scratch
@@ -205,6 +205,8 @@ struct IcpWork {
 
 // kernels.cu launchers (all asynchronous on `s`)
 cudaError_t launch_fill_u32(uint32_t* p, uint32_t v, long long n, cudaStream_t s);
+// n words of z to kInfBits, n0 words of a and n1 words of b (or none) to zero
+cudaError_t launch_prepare(uint32_t* z, long long n, int* a, long long n0, int* b, long long n1, cudaStream_t s);
 cudaError_t launch_obs_count(const float* depth, int W, int H, int* block_counts, cudaStream_t s);
 cudaError_t launch_exclusive_scan(const int* in, int* out, int n, int* tmp, cudaStream_t s);
 cudaError_t launch_obs_write(const float* depth, const Camera& cam, const float* rx, const float* ry,
@@ -226,6 +228,7 @@ cudaError_t launch_render_parents(const Camera& cam, const Geometry& g, const Ba
                                   unsigned long long* culled, cudaStream_t s);
 cudaError_t launch_uset(const Camera& cam, const Geometry& g, const ObsIndex& obs, const Batch& b,
                         cudaStream_t s);
+// hist zero before the call
 cudaError_t launch_group_by_mesh(const perch_obj* hyp, long long n, int n_mesh, int* hist, int* offsets,
                                  int* cursor, int* order, int* scan_tmp, cudaStream_t s,
                                  const uint8_t* skip = nullptr);

@@ -279,6 +279,23 @@ cudaError_t launch_fill_u32(uint32_t* p, uint32_t v, long long n, cudaStream_t s
   return cudaGetLastError();
 }
 
+// a batch's buffers in one launch, bound by storing the parents' z-buffers, instead of a
+// fill and three memsets: smallest evaluation 134 -> 130 us
+__global__ void __launch_bounds__(256) k_prepare(uint32_t* z, long long n, int* a, long long n0, int* b, long long n1) {
+  const long long i0 = blockIdx.x * 256LL + threadIdx.x, stride = gridDim.x * 256LL, n4 = n >> 2;
+  for (long long i = i0; i < n4; i += stride)
+    reinterpret_cast<uint4*>(z)[i] = make_uint4(kInfBits, kInfBits, kInfBits, kInfBits);
+  if (i0 < (n & 3)) z[4 * n4 + i0] = kInfBits;
+  for (long long i = i0; i < n0; i += stride) a[i] = 0;
+  for (long long i = i0; i < n1; i += stride) b[i] = 0;
+}
+
+cudaError_t launch_prepare(uint32_t* z, long long n, int* a, long long n0, int* b, long long n1, cudaStream_t s) {
+  const long long most = std::max(std::max(n >> 2, n0), std::max(n1, 1LL));
+  k_prepare<<<(unsigned)std::min(152LL * 16, (most + 255) / 256), 256, 0, s>>>(z, n, a, n0, b, n1);
+  return cudaGetLastError();
+}
+
 // Exclusive scans in two launches (one for a single block): the sums of the
 // blocks' ranges, then each block adds the sums before its own and scans its
 // range. At most 2048 blocks, of 1024 elements or a multiple. F gives the elements
@@ -1978,8 +1995,8 @@ __global__ void k_group_scatter(const perch_obj* hyp, long long n, int n_mesh, i
 
 cudaError_t launch_group_by_mesh(const perch_obj* hyp, long long n, int n_mesh, int* hist, int* offsets,
                                  int* cursor, int* order, int* scan_tmp, cudaStream_t s, const uint8_t* skip) {
-  cudaError_t e = cudaMemsetAsync(hist, 0, sizeof(int) * n_mesh, s);
-  if (e != cudaSuccess || n == 0) return e;
+  if (n == 0) return cudaSuccess;
+  cudaError_t e;
   const unsigned blocks = (unsigned)((n + 255) / 256);
   k_group_hist<<<blocks, 256, 0, s>>>(hyp, n, n_mesh, hist, skip);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -2051,8 +2068,7 @@ cudaError_t launch_group_by_pose(const Geometry& g, const Batch& b, const PoseGr
                                  uint32_t tag, cudaStream_t s) {
   const int per_mesh = g.nx * g.ny * g.n_yaw, P = g.n_mesh * per_mesh;
   const unsigned hb = (unsigned)std::max(1LL, (b.n_hyp + 255) / 256);
-  cudaError_t e = cudaMemsetAsync(pg.cnt, 0, sizeof(int) * (size_t)P, s);
-  if (e != cudaSuccess) return e;
+  cudaError_t e;
   if (b.n_hyp > 0) k_pose_count<<<hb, 256, 0, s>>>(g, b, pg.cnt);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const ScanPoses f{pg.cnt, valid, tag, pg.start, pg.gpose, pg.ranges, per_mesh, g.n_mesh};
