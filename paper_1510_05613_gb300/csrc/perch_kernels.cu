@@ -932,6 +932,7 @@ struct EvalShared {
   int* qn;         // [2]: queued larger triangles of even and odd chunks
   unsigned char* dyn;
   uint32_t pv;     // parity of the barrier's next phase
+  struct EvalHyp* hyp;  // k_eval: the hypothesis at work
 };
 
 // Outcome of one render or evaluation: done; a bounded wait gave up but
@@ -1113,11 +1114,11 @@ __device__ __noinline__ void raster_queued_general(RenderSmem s, uint32_t pk, ui
 // a pose instead of 78-110k. Meshes of 2k-50k triangles, one parent: 7.2 ms
 // instead of 9.0 for 30k hypotheses.
 //
-// `culled` is set in the threads that dropped a triangle; `cov` grows to hold
-// every covered pixel (x0, x1, y0, y1 within bb). On kEvalTimedOut /
+// `culled` is set in the threads that dropped a triangle; with COV `cov` grows to
+// hold every covered pixel (x0, x1, y0, y1 within bb). On kEvalTimedOut /
 // kEvalStop the tile is incomplete; the caller reports the failure and must
 // pass a CTA barrier before reusing the tile.
-template <int NT, int INL>
+template <int NT, int INL, bool COV>
 __device__ __forceinline__ int render_chunks(const Camera& cam, const Geometry& g, const Batch& b, const DevMesh& m,
                                              const perch_obj& o, long long pose, int4 bb, const RenderSmem& s,
                                              EvalShared& sh, unsigned& culled, float4& cov) {
@@ -1160,8 +1161,8 @@ __device__ __forceinline__ int render_chunks(const Camera& cam, const Geometry& 
     pending = more;
     if (more && tid == 0) load_slice(g, o.iyaw, ci.x, ci.y, s, sh.bar);
     if (general) {
-      const GeneralResult r = raster_general<NT, INL>(s, tris, n_tri, tw, th, qn, qcap, cov);
-      cov = r.cov;
+      const GeneralResult r = raster_general<NT, INL>(s, tris, n_tri, tw, th, qn, qcap, COV ? cov : kNoCover);
+      if (COV) cov = r.cov;
       culled |= r.culled;
     }
     for (int t = general ? n_tri : tid; t < n_tri; t += NT) {
@@ -1184,10 +1185,12 @@ __device__ __forceinline__ int render_chunks(const Camera& cam, const Geometry& 
       }
       const float xw = fsub(xmax, px0), yw = fsub(ymax, py0);  // columns past the first, rows past the first
       if (fminf(xw, yw) < 0.0f) continue;
-      cov.x = fminf(cov.x, px0);
-      cov.y = fmaxf(cov.y, xmax);
-      cov.z = fminf(cov.z, py0);
-      cov.w = fmaxf(cov.w, ymax);
+      if (COV) {
+        cov.x = fminf(cov.x, px0);
+        cov.y = fmaxf(cov.y, xmax);
+        cov.z = fminf(cov.z, py0);
+        cov.w = fmaxf(cov.w, ymax);
+      }
       if (fmul(fadd(xw, 0.5f), fadd(yw, 0.5f)) > (float)INL) {
         const int slot = atomicAdd(qn, 1);
         if (slot < qcap) {
@@ -1583,6 +1586,12 @@ struct HypArgs {
   long long pose;
 };
 
+struct EvalHyp {
+  HypArgs a;
+  int4 bb;
+  long long h;
+};
+
 __device__ __forceinline__ bool hyp_args(const Geometry& g, const Batch& b, long long h, HypArgs& a) {
   a.o = b.hyp[h];
   a.pid = b.hyp_parent[h];
@@ -1621,24 +1630,34 @@ __device__ int eval_one(long long h, const Camera& cam, const Geometry& g, const
     reinterpret_cast<int*>(s_obs)[tid] = reinterpret_cast<const int*>(&b.scenes[a.scene])[tid];
   const ObsIndex& obs = MULTI ? *s_obs : obs0;
   const RenderSmem s = render_smem(sh.dyn);
-  float* rxs = reinterpret_cast<float*>(s.tile + b.tile_w * b.tile_h);
-  float* rys = rxs + b.tile_w;
   const int tw = bb.z, th = bb.w;
   const DevMesh m = g.meshes[a.o.mesh];
   if (tid == 0) render_start(g, m, a.o.iyaw, s, sh.bar);
+  {
+    float* rxs = reinterpret_cast<float*>(s.tile + b.tile_w * b.tile_h);
+    float* rys = rxs + b.tile_w;
+    for (int i = tid; i < tw; i += NT) rxs[i] = g.rx[bb.x + i];
+    for (int i = tid; i < th; i += NT) rys[i] = g.ry[bb.y + i];
+  }
   for (int ly = warp; ly < th; ly += NW)
     for (int lx = lane; lx < tw; lx += 32) s.tile[ly * tw + lx] = 0u;  // 1/z = 0: empty
-  for (int i = tid; i < tw; i += NT) rxs[i] = g.rx[bb.x + i];
-  for (int i = tid; i < th; i += NT) rys[i] = g.ry[bb.y + i];
   if (tid < 7) s_cnt[tid] = 0;
 
   unsigned culled = 0;
   float4 cov = kNoCover;  // not needed here
-  const int st = render_chunks<NT, kInlinePixels>(cam, g, b, m, a.o, a.pose, bb, s, sh, culled, cov);
+  // The cost needs these again. In registers they were spilled in the render's loops, with the
+  // covered box that only k_render needs 108 bytes a thread, now 40: root expansion 2.97 -> 2.73 ms,
+  // 30k hypotheses of uneven meshes 6.73 -> 6.10.
+  if (tid == 0) {
+    sh.hyp->a = a;
+    sh.hyp->bb = bb;
+    sh.hyp->h = h;
+  }
+  const int st = render_chunks<NT, kInlinePixels, false>(cam, g, b, m, a.o, a.pose, bb, s, sh, culled, cov);
   if (st != kEvalDone) {
     if (tid == 0) {
       perch_cost r = {0, 0, 0, 0, 0, kFlagTimeout, 0};
-      b.out[h] = r;
+      b.out[sh.hyp->h] = r;
     }
     __syncthreads();  // s_cnt and the tile are reused by the next hypothesis
     return st;
@@ -1647,8 +1666,10 @@ __device__ int eval_one(long long h, const Camera& cam, const Geometry& g, const
   __syncthreads();
   // the render's projected vertices are done with: their buffer holds the list
   static_assert(sizeof(float2) * kChunkMaxVerts >= sizeof(int) * (kNearList + 1), "the list fits");
-  cost_phase<NT>(h, a.pid, a.plen, a.K_total, a.o, bb, m, cam, g, obs, b, s.tile, rxs, rys, s_cnt,
-                 reinterpret_cast<int*>(s.sXY));
+  const EvalHyp& e = *sh.hyp;
+  float* rxs = reinterpret_cast<float*>(s.tile + b.tile_w * b.tile_h);
+  cost_phase<NT>(e.h, e.a.pid, e.a.plen, e.a.K_total, e.a.o, e.bb, g.meshes[e.a.o.mesh], cam, g, obs, b, s.tile, rxs,
+                 rxs + b.tile_w, s_cnt, reinterpret_cast<int*>(s.sXY));
   return kEvalDone;
 }
 
@@ -1670,12 +1691,13 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_eval(Camera cam, Geometry g, 
   __shared__ int s_cnt[7];
   __shared__ int s_qn[2];
   __shared__ int s_item;
+  __shared__ EvalHyp s_hyp;
   if (threadIdx.x == 0) {
     mbar_init(&s_bar, 1);
     fence_barrier_init();
   }
   __syncthreads();
-  EvalShared sh{&s_bar, s_cnt, s_qn, smem, 0u};
+  EvalShared sh{&s_bar, s_cnt, s_qn, smem, 0u, &s_hyp};
   const int count = *grp.count, offset = grp.order ? *grp.offset : 0;
   for (;;) {
     if (threadIdx.x == 0) s_item = atomicAdd(grp.next, 1);
@@ -1703,6 +1725,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_render(Camera cam, Geometry g
   __shared__ int s_qn[2];
   __shared__ int s_pose;  // the pose to render, -1 = none left
   __shared__ int s_box[4];  // the covered pixels' box within the pose's box: x0, x1, y0, y1
+  __shared__ perch_obj s_obj;  // the pose's object and box, which the store reads again:
+  __shared__ int4 s_bb;        // in registers they would be spilled in the render's loops
   constexpr int NW = NT / 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid == 0) {
@@ -1710,7 +1734,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_render(Camera cam, Geometry g
     fence_barrier_init();
   }
   __syncthreads();
-  EvalShared sh{&s_bar, nullptr, s_qn, smem, 0u};
+  EvalShared sh{&s_bar, nullptr, s_qn, smem, 0u, nullptr};
   const RenderSmem s = render_smem(smem);
   const int count = *w.count, offset = *w.offset;
   // the store holds at most 2^28 poses; with the divisions below in 64 bits a step of
@@ -1744,17 +1768,22 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_render(Camera cam, Geometry g
       __syncthreads();
       continue;
     }
-    const int tw = bb.z;
     const DevMesh m = g.meshes[o.mesh];
-    if (tid == 0) render_start(g, m, o.iyaw, s, sh.bar);
+    if (tid == 0) {
+      render_start(g, m, o.iyaw, s, sh.bar);
+      s_obj = o;
+      s_bb = bb;
+    }
     if (tid < 4) s_box[tid] = (tid & 1) ? -1 : 0x7fffffff;  // ordered by render_chunks' first barrier
     unsigned culled = 0;
     float4 cov = kNoCover;  // x0, x1, y0, y1 of this thread's triangle boxes
-    const int st = render_chunks<NT, INL>(cam, g, b, m, o, p, bb, s, sh, culled, cov);
+    const int st = render_chunks<NT, INL, true>(cam, g, b, m, o, p, bb, s, sh, culled, cov);
+    const int4 box = s_bb;
+    const int tw = box.z;
     if (st != kEvalDone) {
-      for (int i = tid; i < tw * bb.w; i += NT) s.tile[i] = 0u;
+      for (int i = tid; i < tw * box.w; i += NT) s.tile[i] = 0u;
       if (tid == 0) {
-        w.pose_flags[p] = kPoseFailed;
+        w.pose_flags[s_pose] = kPoseFailed;
         s_pose = pose_of(atomicAdd(w.next, 1));
       }
       __syncthreads();
@@ -1781,10 +1810,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_render(Camera cam, Geometry g
     // each rendered point against I in the sign bit: it depends on the pose
     // and the scene, not on the parent. A pose with no observed point near
     // its footprint explains no point.
-    const bool probe = EXPL && obs_near(cam, g, obs, o);
-    uint32_t* dst = w.store + 4 * (size_t)w.tile_off[p];
+    const bool probe = EXPL && obs_near(cam, g, obs, s_obj);
+    uint32_t* dst = w.store + 4 * (size_t)w.tile_off[s_pose];
     for (int ly = warp; ly < ch; ly += NW) {
-      const float ry = EXPL ? g.ry[bb.y + cy0 + ly] : 0.0f;
+      const float ry = EXPL ? g.ry[box.y + cy0 + ly] : 0.0f;
       for (int lx = lane; lx < cw; lx += 32) {
         uint32_t* px = &s.tile[(cy0 + ly) * tw + cx0 + lx];
         const uint32_t izb = *px;
@@ -1793,16 +1822,16 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_render(Camera cam, Geometry g
           *px = 0u;
           const float z = __frcp_rn(__uint_as_float(izb));
           v = __float_as_uint(z);
-          if (probe && explained_by_obs(obs, fmul(g.rx[bb.x + cx0 + lx], z), fmul(ry, z), z, cam.delta2))
+          if (probe && explained_by_obs(obs, fmul(g.rx[box.x + cx0 + lx], z), fmul(ry, z), z, cam.delta2))
             v |= kExplainedBit;
         }
         dst[ly * cw + lx] = v;
       }
     }
     if (tid == 0) {
-      w.pose_flags[p] = any_culled ? kPoseCulled : 0;
-      w.tile_box[p] = make_int4(bb.x + cx0, bb.y + cy0, cw, ch);
-      if (w.valid) w.valid[p] = w.tag;  // read by later launches only
+      w.pose_flags[s_pose] = any_culled ? kPoseCulled : 0;
+      w.tile_box[s_pose] = make_int4(box.x + cx0, box.y + cy0, cw, ch);
+      if (w.valid) w.valid[s_pose] = w.tag;  // read by later launches only
       s_pose = pose_of(atomicAdd(w.next, 1));
     }
     __syncthreads();
@@ -2662,7 +2691,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 3 : 1) k_icp(Camera cam, Geome
     fence_barrier_init();
   }
   __syncthreads();
-  EvalShared sh{&s_bar, nullptr, s_qn, smem, 0u};
+  EvalShared sh{&s_bar, nullptr, s_qn, smem, 0u, nullptr};
   const RenderSmem s = render_smem(smem);
   uint32_t* tile = s.tile;
   for (;;) {
@@ -2689,7 +2718,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 3 : 1) k_icp(Camera cam, Geome
     }
     unsigned culled = 0;
     float4 cov = kNoCover;  // not needed here
-    const int st = render_chunks<NT, kInlinePixels>(cam, g, b, m, a.o, a.pose, bb, s, sh, culled, cov);
+    const int st = render_chunks<NT, kInlinePixels, false>(cam, g, b, m, a.o, a.pose, bb, s, sh, culled, cov);
     if (st != kEvalDone) {
       if (tid == 0) w.out[h] = perch_icp{0.0, 0.0, 0.0, 0.0, 0, 0, 0, (int32_t)kFlagTimeout};
       __syncthreads();  // the tile is cleared by the next hypothesis
