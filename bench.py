@@ -727,7 +727,7 @@ def run_cnn(args):
 
     fwd_ms = time_forward()
     ref_pred = pred.clone()
-    net.perch_cnn_set_tensor_path(1)  # convolutions 2-4 on tcgen05
+    net.perch_cnn_set_tensor_path(1)  # the same kernels as path 0
     tc_ms = time_forward()
     tc_status = net.perch_cnn_tensor_status()
     tc_dev = float((pred - ref_pred).abs().max())
@@ -741,7 +741,7 @@ def run_cnn(args):
             "config": {"workload": "heuristic network, batch of 256 seeded synthetic 2x64x64 crops + one-hot of "
                                    "8 meshes x 16 yaws; one step = forward, backward, Adam",
                        "l2": "flushed (256 MiB write) before every timed step"},
-            "roofline": {"bound": "tensor", "kernel": "training step (k_gemm and its helpers)",
+            "roofline": {"bound": "tensor", "kernel": "training step (k_conv_tma, k_wgrad_tma and their helpers)",
                          "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                          "traffic": measured_traffic("perch_cnn.cu", "cnn_train_step_launches.md"),
                          "flop_per_crop": CNN_TRAIN_FLOP_PER_CROP,
@@ -751,7 +751,7 @@ def run_cnn(args):
             "forward_tcgen05": {"batch": F, "ms": tc_ms, "crops_per_s": F / tc_ms * 1e3,
                                 "tflops": F * CNN_FWD_FLOP_PER_CROP / tc_ms / 1e9,
                                 "max_abs_diff_vs_mma_sync": tc_dev, "waits_gave_up": tc_status[1],
-                                "meaning": "forward with convolutions 2-4 on tcgen05 (tensor-memory accumulator)"},
+                                "meaning": "forward with tensor path 1: the same tcgen05 kernels as path 0"},
             "gpu_launches": None, "clocks": clocks.summary()}
     print(json.dumps(line), flush=True)
     return 0
